@@ -14,7 +14,8 @@
 
 namespace mra {
 
-constexpr int NT = 256;          // threads per CTA for every kernel
+constexpr int NT = 256;          // threads per CTA (the kernels of the emulation engine: EM_NT, mra_emu.cuh);
+                                 // helpers used by both take the count as NTH
 constexpr int KC = 32;           // k-chunk of the staged tile product
 constexpr int MAX_R_DEV = 64;    // largest r (knots per internal region)
 constexpr double SQRT3 = 1.7320508075688772935;
@@ -604,6 +605,7 @@ __device__ __forceinline__ void tri_decode(int t, int& i, int& k) {
   k = t - ii * (ii + 1) / 2;
 }
 
+template <int NTH = NT>
 __device__ inline void chol_smem(double* A, int n, int lda, int* bad) {
   // The pivot of column j (L_jj = d rsqrt(d), and rsqrt(d) to scale the
   // column; long sequences on this chip's narrow FP64 pipe) is formed by
@@ -624,10 +626,10 @@ __device__ inline void chol_smem(double* A, int n, int lda, int* bad) {
   __syncthreads();
   for (int j = 0; j < n; ++j) {
     const double inv = piv;
-    for (int i = j + 1 + threadIdx.x; i < n; i += NT) A[i * lda + j] *= inv;
+    for (int i = j + 1 + threadIdx.x; i < n; i += NTH) A[i * lda + j] *= inv;
     __syncthreads();                       // column j scaled; piv read by every thread
     const int m = n - j - 1;
-    for (int t = threadIdx.x; t < m * (m + 1) / 2; t += NT) {   // lower triangle of the trailing block
+    for (int t = threadIdx.x; t < m * (m + 1) / 2; t += NTH) {   // lower triangle of the trailing block
       int ii, kk;
       tri_decode(t, ii, kk);
       const int i = j + 1 + ii, k = j + 1 + kk;
@@ -644,7 +646,7 @@ __device__ inline void chol_smem(double* A, int n, int lda, int* bad) {
     }
     __syncthreads();
   }
-  for (int t = threadIdx.x; t < n * n; t += NT) {
+  for (int t = threadIdx.x; t < n * n; t += NTH) {
     int i = t / n, k = t - i * n;
     if (k > i) A[i * lda + k] = 0.0;
   }
@@ -670,7 +672,7 @@ __device__ __forceinline__ int seg_block(const int* seg, int nb, int i) {   // b
   return b;
 }
 
-template <bool STK = false>
+template <bool STK = false, int NTH = NT>
 __device__ inline void chol_seg(double* A, int lda, const int* seg, int nb, int* bad, double* pv) {
   __syncthreads();
   int nmax = 0;
@@ -692,7 +694,7 @@ __device__ inline void chol_seg(double* A, int lda, const int* seg, int nb, int*
       tot += m;
       tri += m * (m + 1) / 2;
     }
-    for (int t = threadIdx.x; t < tot; t += NT) {   // column j of every block scaled
+    for (int t = threadIdx.x; t < tot; t += NTH) {   // column j of every block scaled
       int b = 0, u = t;
       for (int m = max(0, seg[1] - seg[0] - j - 1); u >= m; m = max(0, seg[b + 1] - seg[b] - j - 1)) {
         u -= m;
@@ -702,7 +704,7 @@ __device__ inline void chol_seg(double* A, int lda, const int* seg, int nb, int*
       A[(s0 + j + 1 + u) * lda + s0 + j - cs] *= pv[b];
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < tri; t += NT) {   // trailing lower triangles; element 0: the next pivot
+    for (int t = threadIdx.x; t < tri; t += NTH) {   // trailing lower triangles; element 0: the next pivot
       int b = 0, u = t;
       for (int m = max(0, seg[1] - seg[0] - j - 1); u >= m * (m + 1) / 2; m = max(0, seg[b + 1] - seg[b] - j - 1)) {
         u -= m * (m + 1) / 2;
@@ -726,12 +728,12 @@ __device__ inline void chol_seg(double* A, int lda, const int* seg, int nb, int*
   }
   const int n = seg[nb];
   if (STK) {                                   // (stacked: row i holds its block's columns only, lda of them)
-    for (int t = threadIdx.x; t < n * lda; t += NT) {
+    for (int t = threadIdx.x; t < n * lda; t += NTH) {
       const int i = t / lda, k = t - i * lda;
       if (k > i - seg[seg_block(seg, nb, i)]) A[t] = 0.0;
     }
   } else {
-    for (int t = threadIdx.x; t < n * n; t += NT) {
+    for (int t = threadIdx.x; t < n * n; t += NTH) {
       const int i = t / n, k = t - i * n;
       if (k > i || k < seg[seg_block(seg, nb, i)]) A[i * lda + k] = 0.0;
     }
@@ -739,7 +741,7 @@ __device__ inline void chol_seg(double* A, int lda, const int* seg, int nb, int*
   __syncthreads();
 }
 
-template <bool STK = false>
+template <bool STK = false, int NTH = NT>
 __device__ inline void trinv_seg(double* A, int lda, const int* seg, int nb, double* tmp, double* pv) {
   __syncthreads();
   int nmax = 0;
@@ -760,7 +762,7 @@ __device__ inline void trinv_seg(double* A, int lda, const int* seg, int nb, dou
         upd += (nbk - k - 1) * (k + 1);
       }
     }
-    for (int t = threadIdx.x; t < tot; t += NT) {
+    for (int t = threadIdx.x; t < tot; t += NTH) {
       int b = 0, u = t;
       for (int c = k < seg[1] - seg[0] ? seg[1] - seg[0] : 0; u >= c;
            c = k < seg[b + 1] - seg[b] ? seg[b + 1] - seg[b] : 0) {
@@ -778,7 +780,7 @@ __device__ inline void trinv_seg(double* A, int lda, const int* seg, int nb, dou
     }
     // phase 2: X_ij -= L_ik X_kj for i > k, j <= k, within every block
     const int w = k + 1;
-    for (int t = threadIdx.x; t < upd; t += NT) {
+    for (int t = threadIdx.x; t < upd; t += NTH) {
       int b = 0, u = t;
       for (int c = k < seg[1] - seg[0] ? (seg[1] - seg[0] - k - 1) * w : 0; u >= c;
            c = k < seg[b + 1] - seg[b] ? (seg[b + 1] - seg[b] - k - 1) * w : 0) {
@@ -798,6 +800,7 @@ __device__ inline void trinv_seg(double* A, int lda, const int* seg, int nb, dou
 // subtracts L_ik times it from every row i > k.  Each step is a rank-1 update
 // over all threads, so the FP64 work is spread over every warp (the pipe of
 // every SM sub-partition).  tmp: n doubles of shared scratch.
+template <int NTH = NT>
 __device__ inline void trinv_smem(double* A, int n, int lda, double* tmp) {
   __shared__ double piv;
   __syncthreads();
@@ -807,13 +810,13 @@ __device__ inline void trinv_smem(double* A, int n, int lda, double* tmp) {
     // phase 1: row k of X (columns < k) scaled by 1 / L_kk, X_kk = 1 / L_kk;
     // column k of L below the diagonal saved before it is overwritten
     const double rk = piv;
-    for (int t = threadIdx.x; t <= k; t += NT) A[k * lda + t] = t < k ? A[k * lda + t] * rk : rk;
-    for (int i = k + 1 + threadIdx.x; i < n; i += NT) tmp[i] = A[i * lda + k];
+    for (int t = threadIdx.x; t <= k; t += NTH) A[k * lda + t] = t < k ? A[k * lda + t] * rk : rk;
+    for (int i = k + 1 + threadIdx.x; i < n; i += NTH) tmp[i] = A[i * lda + k];
     __syncthreads();
     if (threadIdx.x == 0 && k + 1 < n) piv = 1.0 / A[(k + 1) * lda + k + 1];   // next step's reciprocal
     // phase 2: X_ij -= L_ik X_kj for i > k, j <= k (X_ik starts from 0)
     const int w = k + 1, nr = n - k - 1;
-    for (int t = threadIdx.x; t < nr * w; t += NT) {
+    for (int t = threadIdx.x; t < nr * w; t += NTH) {
       const int ii = t / w, j = t - ii * w, i = k + 1 + ii;
       const double x0 = j == k ? 0.0 : A[i * lda + j];
       A[i * lda + j] = fma(-tmp[i], A[k * lda + j], x0);
@@ -885,13 +888,14 @@ __device__ __forceinline__ double cov0_d(const Cov& c, double x1, double y1, dou
 }
 
 // Sum over the CTA; every thread gets the result.  red: 32 doubles of shared.
+template <int NTH = NT>
 __device__ __forceinline__ double block_sum(double v, double* red) {
   v = warp_sum(v);
   __syncthreads();
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
   double s = 0.0;
-  for (int w = 0; w < NT / 32; ++w) s += red[w];
+  for (int w = 0; w < NTH / 32; ++w) s += red[w];
   __syncthreads();
   return s;
 }

@@ -3,70 +3,80 @@
 // GB300 retires 2 FP64 FMA per clock per SM, so FP64 contractions are emulated
 // with the error-free splitting of Ozaki et al. (2012, "Error-free
 // transformations of matrix multiplication by using fast routines of matrix
-// multiplication and its applications"), written here for bf16 tensor cores:
+// multiplication and its applications"), written here for f16 tensor cores:
 //
 //  * every row of A and of B is scaled, per group of 128 K-columns, by a power
-//    of two 2^e with |x| < 2^e over the group, and its 49 leading bits are cut
-//    into S = 7 slices of 7 bits: x = sum_p a_p 2^(e - 7p), a_p integer,
-//    |a_p| < 128, exact in bf16;
-//  * a_p b_q products are exact (< 2^14) and the FP32 sums of every pair with
-//    the same weight t = p + q over a group stay below 128 * 7 * 127^2 < 2^24,
-//    so the tensor-memory accumulation is exact too; the 28 pairs with
-//    t <= S + 1 go to 7 accumulators (one per t, 64 TMEM columns each);
-//  * every group is drained: the 7 accumulators of a column are combined in
-//    units of the leading weight (double-float, TwoSum for the three largest
-//    corrections), scaled by 2^(e_i + f_j - 14) (exact) and added to a
+//    of two 2^e with |x| < 2^e over the group, rounded to the nearest multiple
+//    of 2^(e - 48) and cut into S = 6 signed digits of 8 bits: x = sum_p d_p
+//    2^(e - 8p), d_p integer, |d_1| <= 256, |d_p| <= 128 for p > 1, exact in
+//    f16 (integers to 2048);
+//  * d_p d_q products are exact and the FP32 sums of every pair with the same
+//    weight t = p + q over a group stay at or below 128 (2 256 128 + 4 128^2)
+//    = 2^24, so the tensor-memory accumulation is exact too; the 21 pairs with
+//    t <= S + 1 go to 6 accumulators (one per t, up to 64 TMEM columns each);
+//  * every group is drained: the 6 accumulators of a column are combined in
+//    units of the leading weight (double-float, Fast2Sum for the two largest
+//    corrections), scaled by 2^(e_i + f_j - 16) (exact) and added to a
 //    double-float register accumulator, converted to FP64 once at the end.
 //
-// The only rounding is the truncation of each operand to 49 bits below its
-// group's largest element and the double-float sums (about 2^-48 relative), so
-// a product matches FP64 to about 1e-14 relative to sum |a b| while running on
-// the tensor cores; the FP64 pipe only does the final conversion.  Range: the
-// running sums are FP32 pairs, so |results| < 2^127, and a group whose scale
-// product 2^(e_i + f_j) is below 2^-88 is dropped (its contribution is below
-// 2^-80 in absolute value).
+// Signed digits carry 8 bits a slice where sign-and-magnitude slices of the
+// same magnitude (|a| < 128) carry 7: 6 slices and 21 products hold what took
+// 7 and 28, the operand error (at most 2^-49 of the group's largest element)
+// is rounded instead of truncated, and the dropped pairs (t = 8) have random
+// signs.  So a product matches FP64 to about 1e-14 relative to sum |a b| while
+// running on the tensor cores; the FP64 pipe only does the final conversion.
+// Range: the running sums are FP32 pairs, so |results| < 2^127, and a group
+// whose scale product 2^(e_i + f_j) is below 2^-110 is dropped.
 //
 // Pipeline: the K range is staged in chunks of 16 (one MMA K-step) into two
-// shared-memory buffers; while the MMAs of one chunk run, the CTA splits the
-// next chunk into the other buffer.  Row scales of up to four groups are found
-// in one pass before the chunks that use them.
+// shared-memory buffers.  Warps 1..15 split: the work of a chunk is cut into
+// slots of 16 rows x 16 columns, one warp each, and the warps take the slots
+// of all chunks in turn, each loading its next slot's elements before it splits
+// the current one.  Warp 0 issues the MMAs.  They meet in mbarriers per buffer
+// (staged, free) and per group (accumulators complete, accumulators read), so
+// no barrier of the whole CTA stands between two chunks.
 #pragma once
 #include "mra_tc.cuh"
 
 namespace mra {
 
-constexpr int EM_S = 7;                       // slices per operand
-constexpr int EM_BITS = EM_S * 7;             // 49 leading bits
-constexpr int EM_KC = 16;                     // staged K chunk (bf16 elements) = one MMA K-step
+constexpr int EM_NT = 512;                    // threads per CTA of the engine's kernels
+constexpr int EM_S = 6;                       // digits per operand
+constexpr int EM_KC = 16;                     // staged K chunk (f16 elements) = one MMA K-step
 constexpr int EM_KG = 128;                    // K group sharing one scale per row (drain period)
+constexpr int EM_GCH = EM_KG / EM_KC;         // chunks per group
 constexpr int EM_MAXG = 4;                    // groups whose scales one pass finds
-constexpr int EM_CC = EM_KC / 8;              // 16-byte core columns (8 bf16) per chunk
-constexpr int EM_A_HALFS = TC_M * EM_KC;      // bf16 per slice plane of A (4 KB)
+constexpr int EM_CC = EM_KC / 8;              // 16-byte core columns (8 f16) per chunk
+constexpr int EM_A_HALFS = TC_M * EM_KC;      // f16 per digit plane of A (4 KB)
 constexpr int EM_B_HALFS = TC_N * EM_KC;      // (2 KB)
 constexpr int EM_BUF_HALFS = EM_S * (EM_A_HALFS + EM_B_HALFS);
-constexpr int EM_STAGE_BYTES = 2 * 2 * EM_BUF_HALFS;                    // two buffers: 86016
+constexpr int EM_STAGE_BYTES = 2 * 2 * EM_BUF_HALFS;                    // two buffers: 73728
 constexpr int EM_REXP = EM_MAXG * TC_M;       // ints of row scales of A (shared)
 constexpr int EM_CEXP = EM_MAXG * TC_N;       // ints of row scales of B (shared)
 constexpr uint32_t EM_TMEM_COLS = 512;
+constexpr int EM_SLOT = 16;                   // rows of one warp's slot
+constexpr int EM_SLOTS = (TC_M + TC_N) / EM_SLOT;   // slots of a full chunk, and its arrivals
+constexpr int EM_EMIN = -900;                 // scales below 2^-900 are raised to it (the elements become zero)
+// mbarriers: buffer b staged / free, group accumulated / read, and the last
+// resort of a timed-out product
+enum : int { EM_FULL = 0, EM_FREE = 2, EM_DONE = 4, EM_READ = 5, EM_LAST = 6, EM_MBARS = 7 };
 // The engine takes all 512 TMEM columns of an SM; its kernels ask for more than
 // half of the SM's shared memory so that a second CTA is never resident (it
 // would only wait in tcgen05.alloc).
 constexpr size_t EM_SOLO_SMEM = 116 * 1024;
-static_assert(EM_KG * EM_S * 127 * 127 < (1 << 24), "group sums must stay exact in FP32");
+static_assert(EM_KG * (2 * 256 * 128 + (EM_S - 2) * 128 * 128) <= (1 << 24), "group sums must stay exact in FP32");
 static_assert(EM_S * TC_N <= (int)EM_TMEM_COLS, "accumulators exceed the tensor-memory allocation");
-// kind::f16 instruction descriptor: D = F32, A = B = BF16, both K-major, 128 x 64.
-constexpr uint32_t EM_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TC_N >> 3) << 17) |
-                              ((uint32_t)(TC_M >> 4) << 24);
+
+// kind::f16 instruction descriptor: D = F32, A = B = F16, both K-major, 128 x n.
+__device__ __forceinline__ uint32_t em_idesc(int n) {
+  return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(TC_M >> 4) << 24);
+}
 
 // Shared-memory matrix descriptor, no swizzle, K-major core matrices of 8 rows x
 // 16 bytes: 128 B between K-adjacent cores, EM_CC * 128 B between 8-row groups.
 __device__ __forceinline__ uint64_t em_desc(uint32_t saddr) {
   return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)((128u >> 4) & 0x3FFF) << 16) |
          ((uint64_t)(((EM_CC * 128u) >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46);
-}
-
-__device__ __forceinline__ int em_cm(int row, int k) {   // bf16 index in a staged plane
-  return (((row >> 3) * EM_CC + (k >> 3)) << 6) + ((row & 7) << 3) + (k & 7);
 }
 
 // Binary exponent e with |x| < 2^e (x != 0, normal); -2000 for zero.
@@ -76,16 +86,31 @@ __device__ __forceinline__ int em_exp(double x) {
   return be == 0 ? -2000 : be - 1022;
 }
 
+// Output ownership: thread (warp w, lane l) holds row 32 (w % 4) + l and the
+// 16 columns starting at 16 (w / 4) of the 128 x 64 tile.
+struct EmAcc {
+  static constexpr int NC = 16;
+  double v[NC];
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) v[c] = 0.0;
+  }
+  __device__ __forceinline__ int row() const { return (((threadIdx.x >> 5) & 3) << 5) | (threadIdx.x & 31); }
+  __device__ __forceinline__ int col0() const { return (threadIdx.x >> 7) * NC; }
+};
+static_assert((EM_NT / 128) * EmAcc::NC == TC_N, "the warps cover the tile's columns");
+
 struct EmCtx {
-  uint16_t* stage;   // EM_STAGE_BYTES of shared memory: two buffers of 7 A planes, then 7 B planes
+  uint16_t* stage;   // EM_STAGE_BYTES of shared memory: two buffers of 6 A planes, then 6 B planes (of nb rows, to 16)
   int* rexp;         // EM_REXP row scales of A, [group][row], when the scale pass forms them
   int* cexp;         // EM_CEXP row scales of B
   const int* ra;     // row scales of A in use: ra[g * rs + i] (rexp or a producer's table)
-  const int* cb;     // row scales of B in use: cb[g * cs + j]
+  const int* cb;     // row scales of B in use: cb[g * cs + j] (the drains: cexp[g * TC_N + j])
   int rs, cs;
-  uint64_t* mbar;    // two mbarriers, one per staging buffer
+  uint64_t* mbar;    // EM_MBARS mbarriers
   uint32_t tmem;
-  uint32_t phase;    // bit b: parity of the next completion of mbar[b] (tracked by warp 0)
+  uint32_t chunks;   // chunks staged and groups drained by the products so far (uniform): the barriers' phases
+  uint32_t groups;
   int* fail;
 };
 
@@ -96,8 +121,10 @@ __device__ inline void em_init(EmCtx& cx, uint32_t* tmem_slot) {
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (threadIdx.x == 0) {
-    for (int b = 0; b < 2; ++b)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(cx.mbar + b)), "r"(1));
+    for (int b = 0; b < EM_MBARS; ++b) {
+      const int count = b < EM_FREE ? EM_SLOTS : (b == EM_READ ? EM_NT / 32 : (b == EM_DONE ? 2 : 1));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(cx.mbar + b)), "r"(count));
+    }
     asm volatile("fence.mbarrier_init.release.cluster;");
     *cx.fail = 0;
   }
@@ -105,7 +132,7 @@ __device__ inline void em_init(EmCtx& cx, uint32_t* tmem_slot) {
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   cx.tmem = *tmem_slot;
-  cx.phase = 0;
+  cx.chunks = cx.groups = 0;
 }
 
 __device__ inline void em_release(EmCtx& cx) {
@@ -115,13 +142,34 @@ __device__ inline void em_release(EmCtx& cx) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(cx.tmem), "r"(EM_TMEM_COLS));
 }
 
-// Wait (bounded) for the MMAs committed to buffer b; flips b's phase once they
-// completed.  Called by warp 0 only, which alone tracks the phases.
-__device__ __forceinline__ bool em_poll(EmCtx& cx, int b) {
-  uint32_t ph = (cx.phase >> b) & 1u;
-  const bool done = tc_wait_phase(cx.mbar + b, ph);
-  if (done) cx.phase ^= 1u << b;
-  return done;
+// Wait (bounded) until the phase of the given parity of mbarrier k completed.
+// False after the limit, or once another warp gave up.
+constexpr int EM_WAIT_LIMIT = 1 << 22;
+__device__ __forceinline__ bool em_wait(const EmCtx& cx, int k, uint32_t parity) {
+  const uint32_t a = smem_addr(cx.mbar + k);
+  uint32_t done = 0;
+  for (int it = 0; it < EM_WAIT_LIMIT && !done; ++it) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(done)
+        : "r"(a), "r"(parity)
+        : "memory");
+    if (!done && (it & 63) == 63 && *(volatile int*)cx.fail) break;
+  }
+  if (__all_sync(0xffffffffu, done != 0)) return true;   // (whole warps wait)
+  *(volatile int*)cx.fail = 1;
+  return false;
+}
+
+__device__ __forceinline__ void em_arrive(const EmCtx& cx, int k, uint32_t count) {
+  asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(cx.mbar + k)), "r"(count)
+               : "memory");
+}
+
+__device__ __forceinline__ void em_commit(const EmCtx& cx, int k) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                   smem_addr(cx.mbar + k))
+               : "memory");
 }
 
 // Row scales of the groups of K columns [K0, K0 + KS), KS <= EM_MAXG * EM_KG:
@@ -152,7 +200,7 @@ __device__ inline void em_scales(EmCtx& cx, const double* A, long sai, long sak,
     __syncthreads();                         // scratch (and, on the first slab, earlier scales) no longer read
     if (s0 == 0) {
       const int ng = (KS + EM_KG - 1) / EM_KG;
-      for (int t = threadIdx.x; t < ng * (TC_M + TC_N); t += NT) {
+      for (int t = threadIdx.x; t < ng * (TC_M + TC_N); t += EM_NT) {
         if (t < ng * TC_M) cx.rexp[t] = -2000;
         else cx.cexp[t - ng * TC_M] = -2000;
       }
@@ -166,7 +214,7 @@ __device__ inline void em_scales(EmCtx& cx, const double* A, long sai, long sak,
       const int n = q == 0 ? na : nb, r0 = q == 0 ? 0 : na;
       const bool in_smem = __isShared(X);
       const int cnt = n * sn;
-      for (int t = threadIdx.x; t < cnt; t += NT) {
+      for (int t = threadIdx.x; t < cnt; t += EM_NT) {
         int i, k;
         if (sk == 1) { i = t / sn; k = t - i * sn; }
         else { k = t / n; i = t - k * n; }
@@ -178,7 +226,7 @@ __device__ inline void em_scales(EmCtx& cx, const double* A, long sai, long sak,
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_all;" ::: "memory");
     __syncthreads();
     const int g = s0 / EM_KG;
-    for (int i = threadIdx.x; i < rows; i += NT) {   // (the scanned rows are the kept ones)
+    for (int i = threadIdx.x; i < rows; i += EM_NT) {   // (the scanned rows are the kept ones)
       const uint32_t* wr = words + i * EM_SLAB_LD;
       int be = 0;
       for (int k = 0; k < sn; ++k) be = max(be, (int)((wr[k] >> 20) & 0x7FFu));
@@ -191,106 +239,172 @@ __device__ inline void em_scales(EmCtx& cx, const double* A, long sai, long sak,
   __syncthreads();
 }
 
-// The 49-bit magnitude window of x relative to scale e (|x| < 2^e):
-// X = floor(|x| 2^(49 - e)) as h (top 17 bits) and l (low 32 bits); 0 for zero.
-__device__ __forceinline__ void em_window(double x, int e, uint32_t& h, uint32_t& l) {
+// |x| in units of 2^(E - 1022 - 56) (E = 1022 + e, |x| < 2^e) plus the digit
+// bias: the magnitude's 56-bit window plus 128 at every digit, so that the low
+// six bytes are the digits 6 (rounding, dropped) .. 2 plus 128 and the top 16
+// bits the first digit plus 0x6400 (f16 1024).  Zero and subnormal x shift out
+// entirely (E >= 122); shr.b64 clamps shifts of 64 and more.
+__device__ __forceinline__ uint64_t em_window(double x, int E) {
   const uint32_t hw = (uint32_t)__double2hiint(x), lw = (uint32_t)__double2loint(x);
-  const int be = (int)((hw >> 20) & 0x7FFu);
-  const uint32_t mh = (hw & 0xFFFFFu) | 0x100000u;                   // mantissa = mh : lw (53 bits)
-  const int sh = min(e + 1026 - be, 63);                              // >= 4 when |x| < 2^e
-  const uint32_t l_lo = __funnelshift_r(lw, mh, (uint32_t)sh);        // used when sh < 32
-  const uint32_t l_hi = sh < 53 ? mh >> (sh - 32 < 0 ? 0 : sh - 32) : 0u;
-  l = be == 0 ? 0u : (sh < 32 ? l_lo : l_hi);
-  h = (be == 0 || sh >= 32) ? 0u : mh >> sh;
+  const uint32_t d = (uint32_t)(E - (int)((hw >> 20) & 0x7FFu));
+  const uint32_t mh = (__funnelshift_l(lw, hw, 3) & 0x7FFFFFu) | 0x800000u;   // (1.mantissa) 2^55
+  uint64_t m = ((uint64_t)mh << 32) | (lw << 3);
+  asm("shr.b64 %0, %1, %2;" : "=l"(m) : "l"(m), "r"(d));
+  return m + 0x6400808080808080ull;
 }
 
-// bf16x2 fused multiply-add: exact here (small integers).
+// f16x2 fused multiply-add: exact here (small integers).
 __device__ __forceinline__ uint32_t em_hfma2(uint32_t a, uint32_t b, uint32_t c) {
   uint32_t d;
-  asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
   return d;
 }
 
-// The 7 slice planes of a pair of elements (x0 low half, x1 high half) as
-// bf16x2 words: slice p of X is the 7-bit field at bits 49 - 7 (p + 1); the two
-// fields go to bits 0-6 and 16-22 of a word biased to bf16 (128 + a), and one
-// bf16x2 FMA gives sg (128 + a) - 128 sg = sg a exactly.
-__device__ __forceinline__ void em_split_pair(double x0, double x1, int e, uint32_t* w) {
-  uint32_t h0, l0, h1, l1;
-  em_window(x0, e, h0, l0);
-  em_window(x1, e, h1, l1);
-  const uint32_t sgn = (((uint32_t)__double2hiint(x0) >> 16) & 0x8000u) | ((uint32_t)__double2hiint(x1) & 0x80000000u);
-  const uint32_t sg = 0x3F803F80u | sgn;              // (+-1, +-1) in bf16
-  const uint32_t nb = 0xC300C300u ^ sgn;              // -128 sg
-  const uint32_t bias = 0x43004300u;
-  const uint32_t M0 = 0x7Fu, M1 = 0x7F0000u;
-  // field of element 0 in bits 0-6 (t0), of element 1 in bits 16-22 (t1)
-  uint32_t t0, t1;
-  t0 = h0 >> 10;                        t1 = h1 << 6;                        w[0] = em_hfma2(t0 | (t1 & M1) | bias, sg, nb);
-  t0 = h0 >> 3;                         t1 = h1 << 13;                       w[1] = em_hfma2((t0 & M0) | (t1 & M1) | bias, sg, nb);
-  t0 = __funnelshift_r(l0, h0, 28);     t1 = __funnelshift_r(l1, h1, 12);    w[2] = em_hfma2((t0 & M0) | (t1 & M1) | bias, sg, nb);
-  t0 = l0 >> 21;                        t1 = l1 >> 5;                        w[3] = em_hfma2((t0 & M0) | (t1 & M1) | bias, sg, nb);
-  t0 = l0 >> 14;                        t1 = l1 << 2;                        w[4] = em_hfma2((t0 & M0) | (t1 & M1) | bias, sg, nb);
-  t0 = l0 >> 7;                         t1 = l1 << 9;                        w[5] = em_hfma2((t0 & M0) | (t1 & M1) | bias, sg, nb);
-  t0 = l0;                              t1 = l1 << 16;                       w[6] = em_hfma2((t0 & M0) | (t1 & M1) | bias, sg, nb);
+// The 6 digit planes of a pair of elements (x0 low half, x1 high half) as f16x2
+// words: a byte b of the window joins 0x64 to the f16 1024 + b, and one f16x2
+// FMA with the signs gives sg (1024 + b) - sg 1152 = sg (b - 128) exactly (the
+// first digit: minus 1024).
+__device__ __forceinline__ void em_split_pair(double x0, double x1, int E, uint32_t* w) {
+  const uint64_t y0 = em_window(x0, E), y1 = em_window(x1, E);
+  const uint32_t h0 = (uint32_t)(y0 >> 32), l0 = (uint32_t)y0, h1 = (uint32_t)(y1 >> 32), l1 = (uint32_t)y1;
+  const uint32_t sgn = __byte_perm((uint32_t)__double2hiint(x0), (uint32_t)__double2hiint(x1), 0x7632) & 0x80008000u;
+  const uint32_t sg = 0x3C003C00u | sgn;              // (+-1, +-1) in f16
+  const uint32_t n1 = 0xE400E400u ^ sgn;              // -1024 sg
+  const uint32_t nb = 0xE480E480u ^ sgn;              // -1152 sg
+  const uint32_t k64 = 0x64646464u;
+  const uint32_t a = __byte_perm(h0, h1, 0x5410);     // bytes: digits 3, 2 of x0, then of x1
+  const uint32_t b = __byte_perm(l0, l1, 0x7632);     // digits 5, 4
+  const uint32_t c = __byte_perm(l0, l1, 0x0501);     // digit 6 (in bytes 0 and 2)
+  w[0] = em_hfma2(__byte_perm(h0, h1, 0x7632), sg, n1);
+  w[1] = em_hfma2(__byte_perm(a, k64, 0x4341), sg, nb);
+  w[2] = em_hfma2(__byte_perm(a, k64, 0x4240), sg, nb);
+  w[3] = em_hfma2(__byte_perm(b, k64, 0x4341), sg, nb);
+  w[4] = em_hfma2(__byte_perm(b, k64, 0x4240), sg, nb);
+  w[5] = em_hfma2((c & 0x00FF00FFu) | 0x64006400u, sg, nb);
 }
 
-// The 7 slice planes of 4 consecutive K of row i, as bf16 pairs, into planes.
-__device__ __forceinline__ void em_split_store(uint16_t* planes, int pstride, int e, const double* x, int i, int k4) {
-  uint32_t w0[EM_S], w1[EM_S];
-  em_split_pair(x[0], x[1], e, w0);
-  em_split_pair(x[2], x[3], e, w1);
-  const int off = em_cm(i, 4 * k4);
-#pragma unroll
-  for (int s = 0; s < EM_S; ++s) *reinterpret_cast<uint2*>(planes + s * pstride + off) = make_uint2(w0[s], w1[s]);
+// One operand of a product as its slots see it.
+//
+// A slot is 16 rows x 16 columns, a warp's 8 elements per lane.  Rows that are
+// contiguous along K and aligned are read four elements at a time, four lanes
+// to a row's 128 bytes (lane: row l / 4 and row l / 4 + 8, columns 4 (l % 4) ..):
+// 8 cache lines a load, where a lane to a row took 16 and kept the L1's tag
+// stage busier than anything else in the engine.  Other operands give every
+// lane 8 columns of one row (row l % 16, columns 8 (l / 16) ..), so that loads
+// of a K-major operand run along its rows.
+struct EmOperand {
+  const double* p;
+  long si, sk;      // element (i, k) at p[i * si + k * sk]
+  int n;            // rows kept
+  int vec;          // elements a load (4: 32-byte aligned global rows, 2: 16-byte aligned rows, 1: any layout)
+};
+
+__device__ __forceinline__ EmOperand em_operand(const double* p, long si, long sk, int n) {
+  const uintptr_t a = reinterpret_cast<uintptr_t>(p);
+  const int vec = sk != 1 ? 1 : ((a & 31) == 0 && (si & 3) == 0 && __isGlobal(p) ? 4 : ((a & 15) == 0 && (si & 1) == 0 ? 2 : 1));
+  return EmOperand{p, si, sk, n, vec};
 }
 
-constexpr int EM_MAX_ITEMS = (4 * (TC_M + TC_N) + NT - 32 - 1) / (NT - 32);   // per staging thread
-
-// Split K columns [k0, k0 + kn) (kn <= EM_KC) of rows i < na of A and j < nb of
-// B into buffer b.  Rows beyond na (nb) are left as they are: they only reach
-// output rows (columns) that the caller discards.  Item = half a 16-byte core
-// row (4 K) of one row; the 32 lanes of a warp cover 8 rows x 2 core columns
-// x 2 halves, i.e. 256 contiguous bytes per plane.  Warp 0 issues the MMAs of
-// the previous chunk meanwhile, so the items go to warps 1..7.
-__device__ inline void em_stage(EmCtx& cx, int b, int g, const double* A, long sai, long sak, int na,
-                                const double* B, long sbj, long sbk, int nb, int k0, int kn) {
-  if (threadIdx.x < 32) return;
-  uint16_t* base = cx.stage + b * EM_BUF_HALFS;
-  const int ia = 4 * ((na + 7) & ~7), items = ia + 4 * ((nb + 7) & ~7);
-  // every load of this thread's items first, so that one memory latency
-  // covers the chunk; then the splits
-  double x[EM_MAX_ITEMS][4];
+// This lane's 8 elements of the slot with first row i0 and first column k0 (zero
+// beyond the kept rows and beyond the K range, k1), and the scales of its rows
+// from tab (0 beyond).
+__device__ __forceinline__ void em_load(const EmOperand& o, const int* tab, int i0, int k0, int k1, double* x, int* e) {
+  const int lane = threadIdx.x & 31;
+  if (o.vec > 1) {
+    const int k = k0 + 4 * (lane & 3), kn = k1 - k;
 #pragma unroll
-  for (int u = 0; u < EM_MAX_ITEMS; ++u) {
-    const int it = threadIdx.x - 32 + u * (NT - 32);
-    const bool isA = it < ia;
-    const int jt = isA ? it : it - ia;
-    const int i = ((jt >> 1) & 7) | ((jt >> 5) << 3), k4 = ((jt >> 4) & 1) * 2 + (jt & 1);
-    const double* X = isA ? A : B;
-    const long si = isA ? sai : sbj, sk = isA ? sak : sbk;
-    const bool ok = it < items && i < (isA ? na : nb);
-    const double* p = X + (long)i * si + (long)(k0 + 4 * k4) * sk;
+    for (int j = 0; j < 2; ++j) {
+      const int i = i0 + (lane >> 2) + 8 * j;
+      const double* p = o.p + (long)i * o.si + k;
+      double* y = x + 4 * j;
+      const bool in = i < o.n;
+      e[j] = in ? tab[i] : 0;
+      if (in && kn >= 4) {
+        if (o.vec == 4) {
+          asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(y[0]), "=d"(y[1]), "=d"(y[2]), "=d"(y[3]) : "l"(p) : "memory");
+        } else {
+          const double2 u = *reinterpret_cast<const double2*>(p), v = *reinterpret_cast<const double2*>(p + 2);
+          y[0] = u.x;
+          y[1] = u.y;
+          y[2] = v.x;
+          y[3] = v.y;
+        }
+      } else {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) x[u][j] = (ok && 4 * k4 + j < kn) ? p[(long)j * sk] : 0.0;
+        for (int c = 0; c < 4; ++c) y[c] = in && c < kn ? p[c] : 0.0;
+      }
+    }
+  } else {
+    const int i = i0 + (lane & 15), k = k0 + 8 * (lane >> 4), kn = i < o.n ? k1 - k : 0;
+    const double* p = o.p + (long)i * o.si + (long)k * o.sk;
+    e[0] = e[1] = i < o.n ? tab[i] : 0;
+    if (kn >= 8) {
+#pragma unroll
+      for (int c = 0; c < 8; ++c) x[c] = p[(long)c * o.sk];
+    } else {
+#pragma unroll
+      for (int c = 0; c < 8; ++c) x[c] = c < kn ? p[(long)c * o.sk] : 0.0;
+    }
   }
+}
+
+// Split a slot's elements and store their digit planes (pstride f16 apart) from
+// `planes`, where the operand's row 0 lies.
+__device__ __forceinline__ void em_split_slot(const EmOperand& o, int i0, const double* x, const int* e,
+                                              uint16_t* planes, int pstride) {
+  const int lane = threadIdx.x & 31;
+  const int E0 = max(e[0], EM_EMIN) + 1022, E1 = max(e[1], EM_EMIN) + 1022;
+  uint32_t w[4][EM_S];
+  em_split_pair(x[0], x[1], E0, w[0]);
+  em_split_pair(x[2], x[3], E0, w[1]);
+  em_split_pair(x[4], x[5], E1, w[2]);
+  em_split_pair(x[6], x[7], E1, w[3]);
+  uint16_t* d = planes + (i0 >> 3) * EM_CC * 64;   // (i0 is a multiple of 16)
+  if (o.vec > 1) {
+    const int l = lane & 3;
+    d += (l >> 1) * 64 + (lane >> 2) * 8 + (l & 1) * 4;
 #pragma unroll
-  for (int u = 0; u < EM_MAX_ITEMS; ++u) {
-    const int it = threadIdx.x - 32 + u * (NT - 32);
-    if (it >= items) break;
-    const bool isA = it < ia;
-    const int jt = isA ? it : it - ia;
-    const int i = ((jt >> 1) & 7) | ((jt >> 5) << 3), k4 = ((jt >> 4) & 1) * 2 + (jt & 1);
-    if (isA) em_split_store(base, EM_A_HALFS, cx.ra[g * cx.rs + i], x[u], i, k4);
-    else em_split_store(base + EM_S * EM_A_HALFS, EM_B_HALFS, cx.cb[g * cx.cs + i], x[u], i, k4);
+    for (int s = 0; s < EM_S; ++s) {
+      *reinterpret_cast<uint2*>(d + s * pstride) = make_uint2(w[0][s], w[1][s]);
+      *reinterpret_cast<uint2*>(d + s * pstride + EM_CC * 64) = make_uint2(w[2][s], w[3][s]);
+    }
+  } else {
+    d += ((lane >> 3) & 1) * EM_CC * 64 + (lane >> 4) * 64 + (lane & 7) * 8;
+#pragma unroll
+    for (int s = 0; s < EM_S; ++s)
+      *reinterpret_cast<uint4*>(d + s * pstride) = make_uint4(w[0][s], w[1][s], w[2][s], w[3][s]);
   }
 }
 
-__device__ __forceinline__ void em_issue(uint32_t tmem, uint64_t da, uint64_t db, uint32_t accumulate) {
+__device__ __forceinline__ void em_issue(uint32_t tmem, uint64_t da, uint64_t db, uint32_t accumulate,
+                                         uint32_t idesc = em_idesc(TC_N)) {
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem),
-      "l"(da), "l"(db), "r"(EM_IDESC), "r"(accumulate));
+      "l"(da), "l"(db), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
+// Issue the digit-pair products of one staged chunk (one thread; stage: the
+// buffer's shared-memory address).  The B planes of nbp rows follow each other,
+// and so do the accumulators of nbp columns: digit p of A times the digits
+// 1 .. 7 - p of B is one product of nbp (7 - p) columns into the accumulators
+// p .. 6, cut at 256 columns.  So 8 MMAs of up to 256 columns do the work of 21
+// of 64, which took the issuing thread 86 cycles each on a busy SM and read A
+// from shared memory 21 times.
+__device__ __forceinline__ void em_issue_chunk(const EmCtx& cx, uint32_t stage, int nbp, bool gfirst) {
+  // plane descriptors differ only in the start-address field (addr >> 4, 14 bits; shared memory
+  // addresses stay below 2^18, so the offsets below never carry out of the field)
+  const uint64_t da0 = em_desc(stage), db0 = em_desc(stage + 2 * EM_S * EM_A_HALFS);
+#pragma unroll
+  for (int p = 1; p <= EM_S; ++p) {
+    const int cols = nbp * (EM_S + 1 - p);
+    const uint64_t da = da0 + (uint64_t)(((p - 1) * EM_A_HALFS * 2) >> 4);
+    const uint32_t dt = cx.tmem + (uint32_t)((p - 1) * nbp), ac = gfirst && p == 1 ? 0u : 1u;
+    em_issue(dt, da, db0, ac, em_idesc(min(cols, 256)));
+    if (p < 3 && cols > 256)                       // (a row of a plane is 32 bytes)
+      em_issue(dt + 256, da, db0 + 256 * 2, ac, em_idesc(cols - 256));
+  }
 }
 
 __device__ __forceinline__ void two_sum_add(float& hi, float& lo, float v) {
@@ -307,57 +421,46 @@ __device__ __forceinline__ void em_ld8(uint32_t taddr, uint32_t* r) {
                : "r"(taddr));
 }
 
-// Drain the group with row scale ei and column scales cexp[c0 + c] into the
-// running double-float sums (hi, lo) of this thread's 32 columns.
-__device__ inline void em_drain(EmCtx& cx, const int* cexp, int ei, int c0, int na, int nb, float* hi, float* lo) {
+// Add the group with row scale ei and column scales cexp[c0 + c] (shared memory,
+// 16-byte aligned; columns beyond nb are discarded) to the running double-float
+// sums (hi, lo) of this thread's 16 columns (first: the sums are set).
+__device__ inline void em_drain(const EmCtx& cx, const int* cexp, int ei, int c0, int na, int nb, int nbp, bool first,
+                                float* hi, float* lo) {
   const int wq = (threadIdx.x >> 5) & 3;
   if (wq * 32 >= na) return;                         // warp-uniform: every row of this warp is discarded
-  const uint32_t lane_off = (uint32_t)wq << 21;
+  const uint32_t base = cx.tmem + ((uint32_t)wq << 21);
 #pragma unroll
-  for (int cb = 0; cb < 32; cb += 8) {
+  for (int cb = 0; cb < EmAcc::NC; cb += 8) {
     if (c0 + cb >= nb) break;                        // warp-uniform
     uint32_t v[EM_S][8];
 #pragma unroll
-    for (int t = 0; t < EM_S; ++t) em_ld8(cx.tmem + lane_off + (uint32_t)(t * TC_N + c0 + cb), v[t]);
-    asm volatile("tcgen05.wait::ld.sync.aligned;");
+    for (int t = 0; t < EM_S; ++t) em_ld8(base + (uint32_t)(t * nbp + c0 + cb), v[t]);
+    int f[8];
+    *reinterpret_cast<int4*>(f) = *reinterpret_cast<const int4*>(cexp + c0 + cb);
+    *reinterpret_cast<int4*>(f + 4) = *reinterpret_cast<const int4*>(cexp + c0 + cb + 4);
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
-      // group value in units of 2^(e_i + f_j - 14): sum_t v_t 2^(-7 (t - 2))
-      float gh = __uint_as_float(v[0][c]), gl = 0.0f;
-      two_sum_add(gh, gl, __uint_as_float(v[1][c]) * 0x1p-7f);
-      two_sum_add(gh, gl, __uint_as_float(v[2][c]) * 0x1p-14f);
-      two_sum_add(gh, gl, __uint_as_float(v[3][c]) * 0x1p-21f);
-      gl = fmaf(__uint_as_float(v[4][c]), 0x1p-28f, gl);
-      gl = fmaf(__uint_as_float(v[5][c]), 0x1p-35f, gl);
-      gl = fmaf(__uint_as_float(v[6][c]), 0x1p-42f, gl);
-      const int e = ei + cexp[c0 + cb + c] - 14;
-      if (e >= -102 && e <= 127) {
-        const float s = __int_as_float((e + 127) << 23);
+      // group value in units of 2^(e_i + f_j - 16): sum_t v_t 2^(-8 (t - 2)).  The v_t are integers of at
+      // most 2^24, so that Fast2Sum (Dekker 1971) is exact in both steps whichever operand is larger: where
+      // the second one is, both lie on a grid that leaves their sum's rounding representable
+      const float v0 = __uint_as_float(v[0][c]), v1 = __uint_as_float(v[1][c]), v2 = __uint_as_float(v[2][c]);
+      const float s1 = fmaf(v1, 0x1p-8f, v0), r1 = fmaf(v1, 0x1p-8f, -(s1 - v0));
+      const float gh = fmaf(v2, 0x1p-16f, s1), r2 = fmaf(v2, 0x1p-16f, -(gh - s1));
+      const float tail = fmaf(fmaf(__uint_as_float(v[5][c]), 0x1p-8f, __uint_as_float(v[4][c])), 0x1p-8f,
+                              __uint_as_float(v[3][c]));
+      const float gl = fmaf(tail, 0x1p-24f, r1 + r2);
+      const int e = ei + f[c] + (127 - 16);
+      const float s = (uint32_t)(e - 1) < 254u ? __int_as_float(e << 23) : 0.0f;
+      if (first) {
+        hi[cb + c] = gh * s;
+        lo[cb + c] = gl * s;
+      } else {
         two_sum_add(hi[cb + c], lo[cb + c], gh * s);
         lo[cb + c] = fmaf(gl, s, lo[cb + c]);
       }
     }
   }
-}
-
-// Issue the 28 slice-pair MMAs of one staged chunk (lane 0 of warp 0).
-__device__ __forceinline__ void em_issue_chunk(const EmCtx& cx, int b, bool gfirst) {
-  // plane descriptors differ only in the start-address field (addr >> 4, 14 bits; shared memory
-  // addresses stay below 2^18, so the offsets below never carry out of the field)
-  const uint16_t* aP = cx.stage + b * EM_BUF_HALFS;
-  const uint64_t da0 = em_desc(smem_addr(aP)), db0 = em_desc(smem_addr(aP + EM_S * EM_A_HALFS));
-#pragma unroll
-  for (int t = 2; t <= EM_S + 1; ++t) {
-    const uint32_t dt = cx.tmem + (uint32_t)(t - 2) * TC_N;
-#pragma unroll
-    for (int p = 1; p < t; ++p) {                 // q = t - p in [1, 7] since t <= 8
-      const uint64_t da = da0 + (uint64_t)(((p - 1) * EM_A_HALFS * 2) >> 4);
-      const uint64_t db = db0 + (uint64_t)(((t - p - 1) * EM_B_HALFS * 2) >> 4);
-      em_issue(dt, da, db, (gfirst && p == 1) ? 0u : 1u);
-    }
-  }
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-      smem_addr(cx.mbar + b)));
 }
 
 // Exact float -> double by bit moves (subnormal floats, below 2^-126, become 0).
@@ -370,27 +473,44 @@ __device__ __forceinline__ double em_widen(float f) {
   return __hiloint2double((int)hi, (int)(u << 29));
 }
 
+// hi + lo rounded to FP64, on the FP32 and integer pipes: after a TwoSum |lo| is
+// at most half an ulp of hi, so lo is an integer number k of FP64 ulps of hi
+// (|k| <= 2^28, rounded to nearest even) and the sum's bits are hi's plus or minus
+// k.  (8192 DADD take 2.5 us on the narrow FP64 pipe.)  Powers of two, below
+// which the ulp halves, and |hi| < 2^-75 take the DADD.
+__device__ __forceinline__ double em_sum(float a, float b) {
+  const float hi = a + b, t = hi - a;
+  const float lo = (a - (hi - t)) + (b - t);
+  const uint32_t u = __float_as_uint(hi), m = u & 0x7FFFFFFFu;
+  if (m == 0u) return 0.0;
+  if ((m & 0x7FFFFFu) == 0u || m < (52u << 23) || m >= 0x7F800000u) return em_widen(hi) + em_widen(lo);
+  const float ulps = lo * __uint_as_float((306u << 23) - (m & 0x7F800000u));   // lo 2^(52 - exponent of hi)
+  const int k = __float2int_rn(__uint_as_float(__float_as_uint(ulps) ^ (u & 0x80000000u)));
+  const long long d = ((long long)m << 29) + (896LL << 52) + k;
+  return __longlong_as_double(d | (long long)((unsigned long long)(u & 0x80000000u) << 32));
+}
+
 // acc(i, j) = sum_k A(i, k) B(j, k) with FP64-grade accuracy, i < na <= 128,
 // j < nb <= 64 (acc is overwritten).  Returns false (uniformly) if a
-// tensor-core wait timed out.
-//
-// Software pipeline over the 16-column chunks of each scale pass: in step c,
-// warps 1..7 split chunk c into buffer c & 1 while warp 0 issues the MMAs of
-// chunk c - 1 (buffer (c - 1) & 1) and waits for them; the barrier that ends
-// the step therefore leaves buffer c & 1 staged and buffer (c - 1) & 1 free.
+// tensor-core wait timed out.  Opens and ends with a barrier of the CTA.
 //
 // pa / pb, when not null, hold the operands' row scales from their producers:
 // pa[g * pas + i] = the exponent e with |A(i, k)| < 2^e over K group g (any
 // upper bound a producer can form cheaply, e.g. a maximum over a superset of
 // the group's columns); the scale pass then skips that operand.
-__device__ inline bool em_mma(EmCtx& cx, TcAcc& acc, const double* A, long sai, long sak, int na, const double* B,
+__device__ inline bool em_mma(EmCtx& cx, EmAcc& acc, const double* A, long sai, long sak, int na, const double* B,
                               long sbj, long sbk, int nb, int K, const int* pa = nullptr, int pas = 0,
                               const int* pb = nullptr, int pbs = 0) {
   const int row = acc.row(), c0 = acc.col0();
-  float hi[32], lo[32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float hi[EmAcc::NC], lo[EmAcc::NC];
 #pragma unroll
-  for (int c = 0; c < 32; ++c) hi[c] = lo[c] = 0.f;
-  for (int K0 = 0; K0 < K; K0 += EM_MAXG * EM_KG) {
+  for (int c = 0; c < EmAcc::NC; ++c) hi[c] = lo[c] = 0.f;
+  const EmOperand oa = em_operand(A, sai, sak, na), ob = em_operand(B, sbj, sbk, nb);
+  const int sa = (na + EM_SLOT - 1) / EM_SLOT, ns = sa + (nb + EM_SLOT - 1) / EM_SLOT;   // slots of a chunk
+  const int nbp = ((nb + 15) >> 4) << 4;           // rows of a B plane, columns of an accumulator
+  bool ok = true;
+  for (int K0 = 0; K0 < K && ok; K0 += EM_MAXG * EM_KG) {
     const int KS = min(EM_MAXG * EM_KG, K - K0);
     const int g0 = K0 / EM_KG;
     cx.ra = pa ? pa + g0 * pas : cx.rexp;
@@ -398,44 +518,117 @@ __device__ inline bool em_mma(EmCtx& cx, TcAcc& acc, const double* A, long sai, 
     cx.cb = pb ? pb + g0 * pbs : cx.cexp;
     cx.cs = pb ? pbs : TC_N;
     em_scales(cx, A, sai, sak, pa ? 0 : na, B, sbj, sbk, pb ? 0 : nb, K0, KS);
-    const int nch = (KS + EM_KC - 1) / EM_KC;
-    for (int c = 0; c <= nch; ++c) {
-      bool done = true;
-      if (threadIdx.x < 32) {
-        if (c > 0) {
-          if (threadIdx.x == 0) em_issue_chunk(cx, (c - 1) & 1, ((c - 1) * EM_KC) % EM_KG == 0);
-          __syncwarp();
-          done = em_poll(cx, (c - 1) & 1);
-          asm volatile("tcgen05.fence::before_thread_sync;");
-        }
-      } else if (c < nch) {
-        em_stage(cx, c & 1, (c * EM_KC) / EM_KG, A, sai, sak, na, B, sbj, sbk, nb, K0 + c * EM_KC,
-                 min(EM_KC, KS - c * EM_KC));
-        asm volatile("fence.proxy.async.shared::cta;");
-      }
-      if (__syncthreads_or(!done)) {                     // uniform: every thread leaves
-        if (threadIdx.x == 0) *cx.fail = 1;
-        if (threadIdx.x < 32) em_poll(cx, (c - 1) & 1);  // one more bounded wait for the MMAs in flight
-        __syncthreads();
-        return false;
-      }
+    const int nch = (KS + EM_KC - 1) / EM_KC, ngr = (KS + EM_KG - 1) / EM_KG;
+    const uint32_t n0 = cx.chunks, m0 = cx.groups;
+    // the accumulators of group g: wait, add them to the sums, hand them back
+    auto drain = [&](int g) {
+      if (!em_wait(cx, EM_DONE, (m0 + g) & 1u)) return false;
       asm volatile("tcgen05.fence::after_thread_sync;");
-      const int last = (c - 1) * EM_KC;                   // first column of the chunk whose MMAs completed
-      if (c > 0 && ((last + EM_KC) % EM_KG == 0 || last + EM_KC >= KS)) {   // its group is complete
-        const int g = last / EM_KG;
-        em_drain(cx, cx.cb + g * cx.cs, row < na ? cx.ra[g * cx.rs + row] : -2000, c0, na, nb, hi, lo);
-        asm volatile("tcgen05.fence::before_thread_sync;");
-        __syncthreads();                                  // accumulators are read before the next group's MMAs
-        asm volatile("tcgen05.fence::after_thread_sync;");
+      em_drain(cx, cx.cexp + g * TC_N, row < na ? cx.ra[g * cx.rs + row] : -2000, c0, na, nb, nbp, K0 + g == 0,
+               hi, lo);
+      asm volatile("tcgen05.fence::before_thread_sync;");
+      __syncwarp();
+      if (lane == 0) em_arrive(cx, EM_READ, 1);
+      return true;
+    };
+    if (warp == 0) {
+      if (pb) {                                  // the drains read the column scales from shared memory
+        for (int t = lane; t < ngr * TC_N; t += 32)
+          if ((t & (TC_N - 1)) < nb) cx.cexp[t] = cx.cb[(t / TC_N) * cx.cs + (t & (TC_N - 1))];
+        __syncwarp();
       }
+      for (int c = 0; c < nch && ok; ++c) {
+        const uint32_t n = n0 + c;
+        const int b = (int)(n & 1u), g = c / EM_GCH;
+        const bool gfirst = c % EM_GCH == 0;
+        ok = em_wait(cx, EM_FULL + b, (n >> 1) & 1u);
+        if (ok && gfirst && m0 + g > 0) ok = em_wait(cx, EM_READ, (m0 + g - 1) & 1u);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        const bool glast = (c + 1) % EM_GCH == 0 || c + 1 == nch;
+        if (lane == 0) {
+          em_issue_chunk(cx, smem_addr(cx.stage) + (uint32_t)(b * 2 * EM_BUF_HALFS), nbp, gfirst);
+          em_commit(cx, EM_FREE + b);
+          if (glast) {
+            em_commit(cx, EM_DONE);
+            em_arrive(cx, EM_DONE, 1);           // (releases the column scales written above)
+          }
+        }
+        __syncwarp();
+        if (glast) ok = drain(g);
+      }
+    } else {
+      // The warps share out the operands in the ratio of their slots (a warp keeps
+      // to one operand): slot q of chunk c is rows 16 q .. of it.  An operand of
+      // sx slots a chunk gets at most 2 sx warps: a warp's next slot then lies at
+      // most two chunks on, and since its own arrival held back the MMAs of the
+      // chunk it staged last, the buffer's barrier is within one phase of the one
+      // it waits for (a parity tells neighbouring phases apart only).
+      const int wa = max(1, min(EM_NT / 32 - 2, ((EM_NT / 32 - 1) * sa + ns / 2) / ns));
+      const bool isA = warp <= wa;
+      const EmOperand o = isA ? oa : ob;
+      const int* tab = isA ? cx.ra : cx.cb;
+      const int ts = isA ? cx.rs : cx.cs, sx = isA ? sa : ns - sa;
+      const int nw = min(isA ? wa : EM_NT / 32 - 1 - wa, 2 * sx), w0 = isA ? warp - 1 : warp - 1 - wa;
+      const int pstride = isA ? EM_A_HALFS : nbp * EM_KC;
+      uint16_t* const planes = cx.stage + (isA ? 0 : EM_S * EM_A_HALFS);
+      int g = 0;
+      int c = w0 >= nw ? nch : 0, q = w0;          // the slot to stage
+      while (q >= sx) q -= sx, ++c;
+      int cn = c, qn = q;                          // the slot to load next
+      double x[8];                                 // its elements, in flight while the slot before is stored
+      int e[2] = {0, 0};                           // and the scales of their rows
+      auto load = [&] {
+        if (cn < nch) {
+          em_load(o, tab + (cn / EM_GCH) * ts, qn * EM_SLOT, K0 + cn * EM_KC, K0 + KS, x, e);
+          qn += nw;
+          while (qn >= sx) qn -= sx, ++cn;
+        }
+      };
+      auto step = [&] {
+        const uint32_t n = n0 + c;
+        const int b = (int)(n & 1u);
+        // the buffer is free once the MMAs of chunk n - 2 are done
+        if (n >= 2 && !em_wait(cx, EM_FREE + b, ((n >> 1) - 1) & 1u)) return false;
+        em_split_slot(o, q * EM_SLOT, x, e, planes + b * EM_BUF_HALFS, pstride);
+        load();
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        // (A's last slot makes up the arrivals of the slots that the product does not have)
+        if (lane == 0) em_arrive(cx, EM_FULL + b, isA && q == sa - 1 ? EM_SLOTS + 1 - ns : 1);
+        q += nw;
+        while (q >= sx) q -= sx, ++c;
+        return true;
+      };
+      load();
+      while (c < nch && ok) {
+        // (one chunk of the next group is staged before this group is drained)
+        const int stop = min(nch, (g + 1) * EM_GCH + 1);
+        while (ok && c < stop) ok = step();
+        if (c < nch && ok) ok = drain(g++);
+      }
+      while (g < ngr && ok) ok = drain(g++);
+    }
+    cx.chunks += nch;
+    cx.groups += ngr;
+    if (__syncthreads_or(!ok)) {                           // uniform: every thread leaves
+      if (threadIdx.x == 0) {
+        *cx.fail = 0;
+        em_commit(cx, EM_LAST);
+      }
+      __syncthreads();
+      if (warp == 0) em_wait(cx, EM_LAST, 0);              // one more bounded wait for the MMAs in flight
+      if (threadIdx.x == 0) *cx.fail = 1;
+      __syncthreads();
+      ok = false;
     }
   }
-  // hi + lo to FP64 with one DADD: the float-to-double widening is done on the
-  // integer pipe (exact bit moves), not as a conversion on the narrow FP64 pipe
-  // (for every row and column: skipping the discarded ones was measured slower)
+  // hi + lo to FP64 (warps whose rows or columns are all discarded leave it out)
+  if ((warp & 3) * 32 < na && c0 < nb) {
 #pragma unroll
-  for (int c = 0; c < 32; ++c) acc.v[c] = em_widen(hi[c]) + em_widen(lo[c]);
-  return true;
+    for (int c = 0; c < EmAcc::NC; ++c) acc.v[c] = em_sum(hi[c], lo[c]);
+  }
+  return ok;
 }
 
 // Row blocks of r rows stacked into one 128-row tile.

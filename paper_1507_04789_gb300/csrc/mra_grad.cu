@@ -47,8 +47,9 @@ __device__ __forceinline__ void store_tile(const TileAcc<TILE>& acc, double* dst
 }
 
 // Phi(Y): lower triangle, halved diagonal, zero above (in place, square n).
+template <int NTH = NT>
 __device__ __forceinline__ void phi_inplace(double* Y, int n, long ld) {
-  for (int t = threadIdx.x; t < n * n; t += NT) {
+  for (int t = threadIdx.x; t < n * n; t += NTH) {
     int i = t / n, j = t - i * n;
     if (j > i) Y[i * ld + j] = 0.0;
     else if (j == i) Y[i * ld + j] *= 0.5;
@@ -56,8 +57,9 @@ __device__ __forceinline__ void phi_inplace(double* Y, int n, long ld) {
   __syncthreads();
 }
 
+template <int NTH = NT>
 __device__ __forceinline__ void lower_inplace(double* Y, int n, long ld) {
-  for (int t = threadIdx.x; t < n * n; t += NT) {
+  for (int t = threadIdx.x; t < n * n; t += NTH) {
     int i = t / n, j = t - i * n;
     if (j > i) Y[i * ld + j] = 0.0;
   }
@@ -139,23 +141,27 @@ __device__ void chol_inverse_adjoint(double* B0, double* B1, double* B2, long ld
 // 128; B0..B2 may live in global or shared memory).  Returns false (uniformly)
 // if a tensor-core wait timed out; the buffers are then incomplete.
 // (pa, pb: the operands' row scales from their producers, one group since n <= 128, or null)
-__device__ inline bool em_store_product(EmCtx& cx, const double* A, long sai, long sak, const double* B, long sbj,
-                                        long sbk, int n, double* C, long ldc, double scale,
-                                        const int* pa = nullptr, const int* pb = nullptr) {
-  TcAcc acc;
+// A call, not inlined: five copies of the engine in one kernel crowd its registers.
+static __device__ __noinline__ bool em_store_product(EmCtx* pcx, const double* A, long sai, long sak, const double* B,
+                                                     long sbj, long sbk, int n, double* C, long ldc, double scale,
+                                                     const int* pa, const int* pb) {
+  EmCtx cx = *pcx;
+  EmAcc acc;
   const int row = acc.row(), c0 = acc.col0();
-  for (int j0 = 0; j0 < n; j0 += TC_N) {
+  bool ok = true;
+  for (int j0 = 0; j0 < n && ok; j0 += TC_N) {
     const int nb = min(TC_N, n - j0);
-    if (!em_mma(cx, acc, A, sai, sak, n, B + (long)j0 * sbj, sbj, sbk, nb, n, pa, 0, pb ? pb + j0 : nullptr, 0))
-      return false;
-    if (row < n) {
+    ok = em_mma(cx, acc, A, sai, sak, n, B + (long)j0 * sbj, sbj, sbk, nb, n, pa, 0, pb ? pb + j0 : nullptr, 0);
+    if (ok && row < n) {
 #pragma unroll
-      for (int c = 0; c < 32; ++c)
+      for (int c = 0; c < EmAcc::NC; ++c)
         if (c0 + c < nb) C[(long)row * ldc + j0 + c0 + c] = scale * acc.v[c];
     }
   }
+  pcx->chunks = cx.chunks;
+  pcx->groups = cx.groups;
   __syncthreads();
-  return true;
+  return ok;
 }
 
 // Optional scale tables (exponents over the n rows or columns, or null): y_r
@@ -165,21 +171,21 @@ __device__ inline bool chol_inverse_adjoint_em(EmCtx& cx, double* B0, double* B1
                                                const int* y_r = nullptr, const int* li_r = nullptr,
                                                const int* li_c = nullptr, const int* l_c = nullptr) {
   // B1 = Ybar Li'
-  if (!em_store_product(cx, B0, ld, 1, Li, ldi, 1, n, B1, ld, 1.0, y_r, li_r)) return false;
+  if (!em_store_product(&cx, B0, ld, 1, Li, ldi, 1, n, B1, ld, 1.0, y_r, li_r)) return false;
   // B2 = lower(-Li' B1) + dlog / L_ii
-  if (!em_store_product(cx, Li, 1, ldi, B1, 1, ld, n, B2, ld, -1.0, li_c)) return false;
-  lower_inplace(B2, n, ld);
+  if (!em_store_product(&cx, Li, 1, ldi, B1, 1, ld, n, B2, ld, -1.0, li_c, nullptr)) return false;
+  lower_inplace<EM_NT>(B2, n, ld);
   if (dlog != 0.0)
-    for (int t = threadIdx.x; t < n; t += NT) B2[t * ld + t] += dlog / L[t * ldl + t];
+    for (int t = threadIdx.x; t < n; t += EM_NT) B2[t * ld + t] += dlog / L[t * ldl + t];
   __syncthreads();
   // B0 = Phi(L' B2)
-  if (!em_store_product(cx, L, 1, ldl, B2, 1, ld, n, B0, ld, 1.0, l_c)) return false;
-  phi_inplace(B0, n, ld);
+  if (!em_store_product(&cx, L, 1, ldl, B2, 1, ld, n, B0, ld, 1.0, l_c, nullptr)) return false;
+  phi_inplace<EM_NT>(B0, n, ld);
   // B1 = B0 Li
-  if (!em_store_product(cx, B0, ld, 1, Li, 1, ldi, n, B1, ld, 1.0, nullptr, li_c)) return false;
+  if (!em_store_product(&cx, B0, ld, 1, Li, 1, ldi, n, B1, ld, 1.0, nullptr, li_c)) return false;
   // B2 = Li' B1, then symmetrise in place
-  if (!em_store_product(cx, Li, 1, ldi, B1, 1, ld, n, B2, ld, 1.0, li_c)) return false;
-  for (int t = threadIdx.x; t < n * n; t += NT) {
+  if (!em_store_product(&cx, Li, 1, ldi, B1, 1, ld, n, B2, ld, 1.0, li_c, nullptr)) return false;
+  for (int t = threadIdx.x; t < n * n; t += EM_NT) {
     int i = t / n, j = t - i * n;
     if (j < i) {
       double v = 0.5 * (B2[i * ld + j] + B2[j * ld + i]);
@@ -198,13 +204,14 @@ __device__ inline bool chol_inverse_adjoint_em(EmCtx& cx, double* B0, double* B1
 // I + Ahat^{m,m} and S^{m,l} = Lti' Gbar^l / 2 on the emulation engine; a
 // timeout sets status.
 template <int TILE, bool EMU>
-__global__ void __launch_bounds__(NT) post_adjoint_kernel(int m, const Desc* __restrict__ D, GradState gs,
+__global__ void __launch_bounds__(EMU ? EM_NT : NT) post_adjoint_kernel(int m, const Desc* __restrict__ D, GradState gs,
                                                           int gb_ready, int* status) {
+  constexpr int NTH = EMU ? EM_NT : NT;
   extern __shared__ __align__(1024) double smem_all[];
-  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ __align__(8) uint64_t mbar[EM_MBARS];
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
-  __shared__ int rexp[EMU ? EM_REXP : 1], cexp[EMU ? EM_CEXP : 1];
+  __shared__ __align__(16) int rexp[EMU ? EM_REXP : 1], cexp[EMU ? EM_CEXP : 1];
   double* smem = smem_all + (EMU ? EM_STAGE_BYTES / sizeof(double) : 0);
   EmCtx cx;
   bool ok = true;
@@ -216,7 +223,7 @@ __global__ void __launch_bounds__(NT) post_adjoint_kernel(int m, const Desc* __r
     cx.fail = &fail;
     em_init(cx, &tmem_slot);
   }
-  TcAcc ea;
+  EmAcc ea;
   const int erow = ea.row(), ec0 = ea.col0();
   const Desc& ds = D[0];
   const Shape sh = ds.sh;
@@ -232,7 +239,7 @@ __global__ void __launch_bounds__(NT) post_adjoint_kernel(int m, const Desc* __r
   double* stg = B2 + MAX_R_DEV * (MAX_R_DEV + 1);
   long anc[MAXL];
   for (int l = 0; l <= m; ++l) anc[l] = ancestor(st, m, i, l);
-  for (int t = threadIdx.x; t < mr; t += NT) {
+  for (int t = threadIdx.x; t < mr; t += NTH) {
     int k = t / r;
     wbar[t] = gs.Obar[k][anc[k] * r + (t - k * r)];
   }
@@ -242,7 +249,7 @@ __global__ void __launch_bounds__(NT) post_adjoint_kernel(int m, const Desc* __r
   const int T = (m + 1) * (m + 2) / 2;
   const double* A = st.Acc[m] + i * (long)T * r * r;
   // gbar = g - G omega~bar
-  for (int q = threadIdx.x; q < r; q += NT) {
+  for (int q = threadIdx.x; q < r; q += NTH) {
     double s = g[q];
     for (int c = 0; c < mr; ++c) s = fma(-G[(long)q * mr + c], wbar[c], s);
     gbar[q] = s;
@@ -250,7 +257,7 @@ __global__ void __launch_bounds__(NT) post_adjoint_kernel(int m, const Desc* __r
   // Gbar^l = -2 sum_k G^k S^{k,l} - g omega~bar^l'   -> gs.GB
   double* GB = gs.GB[m] + i * (long)r * mr;
   TileAcc<TILE> acc;
-  for (int l = 0; l < m && !gb_ready; ++l) {   // (gb_ready: formed by gbar_kernel_em)
+  for (int l = 0; l < m && !EMU && !gb_ready; ++l) {   // (gb_ready: formed by gbar_kernel_em)
     acc.zero();
     for (int k = 0; k < m; ++k) {
       SRef b = sblock(gs, anc, r, k, l);
@@ -268,17 +275,17 @@ __global__ void __launch_bounds__(NT) post_adjoint_kernel(int m, const Desc* __r
   // Ltbar = sum_l Gbar^l (Ahat^{m,l})' + gbar omegahat^m'   -> B0 (lower)
   const double* om = st.Om[m] + (i * (m + 1) + m) * (long)r;
   if (EMU) {   // one product per l, summed in B0 (each thread owns its entries)
-    for (int t = threadIdx.x; t < r * r; t += NT) B0[(t / r) * ld + t % r] = 0.0;
+    for (int t = threadIdx.x; t < r * r; t += NTH) B0[(t / r) * ld + t % r] = 0.0;
     for (int l = 0; l < m && ok; ++l) {
       ok = em_mma(cx, ea, GB + l * r, mr, 1, r, A + (long)tri_index(m, l) * r * r, r, 1, r, r);
       if (ok && erow < r) {
 #pragma unroll
-        for (int c = 0; c < 32; ++c)
+        for (int c = 0; c < EmAcc::NC; ++c)
           if (ec0 + c < r) B0[erow * ld + ec0 + c] += ea.v[c];
       }
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < r * r; t += NT) {
+    for (int t = threadIdx.x; t < r * r; t += NTH) {
       const int row = t / r, col = t % r;
       B0[row * ld + col] = row >= col ? B0[row * ld + col] + gbar[row] * om[col] : 0.0;
     }
@@ -304,7 +311,7 @@ __global__ void __launch_bounds__(NT) post_adjoint_kernel(int m, const Desc* __r
     chol_inverse_adjoint<TILE>(B0, B1, B2, ld, r, Ltf, r, Lti, r, -1.0, stg);
   }
   double* Ab = gs.Abar[m] + i * (long)r * (mr + r);
-  for (int t = threadIdx.x; t < r * r; t += NT) {
+  for (int t = threadIdx.x; t < r * r; t += NTH) {
     int a = t / r, b = t - a * r;
     Ab[(long)a * (mr + r) + mr + b] = B2[a * ld + b];
   }
@@ -316,7 +323,7 @@ __global__ void __launch_bounds__(NT) post_adjoint_kernel(int m, const Desc* __r
       if (ok && erow < min(S, m - l0) * r) {
         const int l = l0 + erow / r, jj = erow % r;
 #pragma unroll
-        for (int c = 0; c < 32; ++c)
+        for (int c = 0; c < EmAcc::NC; ++c)
           if (ec0 + c < r) Ab[(long)(ec0 + c) * (mr + r) + l * r + jj] = 0.5 * ea.v[c];
       }
     }
@@ -328,7 +335,7 @@ __global__ void __launch_bounds__(NT) post_adjoint_kernel(int m, const Desc* __r
     }
   }
   // omegahat^m bar = Lti' gbar
-  for (int q = threadIdx.x; q < r; q += NT) {
+  for (int q = threadIdx.x; q < r; q += NTH) {
     double s = 0.0;
     for (int c = q; c < r; ++c) s = fma(Lti[(long)c * r + q], gbar[c], s);
     gs.Obar[m][i * r + q] = s;
@@ -339,6 +346,78 @@ __global__ void __launch_bounds__(NT) post_adjoint_kernel(int m, const Desc* __r
   }
 }
 
+// Hbar = 2 H S_p + z omegabar' of one leaf (nF x M r), S_p read block by block
+// from the ancestors; a leaf of at most 16 observations in one 16-row tile
+// (sparse leaves: no FMA lanes on empty rows).
+template <int TILE>
+__device__ void leaf_hbar(const GradState& gs, const long* anc, int M, int r, int nF, const double* H, const double* z,
+                          const double* wbar, double* HB, double* stg) {
+  const int Mr = M * r;
+  if (TILE > 16 && nF <= 16) {
+    TileAccR<16, TILE> a16;
+    for (int l = 0; l < M; ++l) {
+      a16.zero();
+      for (int k = 0; k < M; ++k) {
+        SRef b = sblock(gs, anc, r, k, l);
+        tile_mma_r<16, TILE>(a16, H + k * r, Mr, 1, nF, b.p, b.sj, b.sk, r, r, stg);
+      }
+#pragma unroll
+      for (int p = 0; p < TileAccR<16, TILE>::RR; ++p)
+#pragma unroll
+        for (int q = 0; q < TileAccR<16, TILE>::RC; ++q) {
+          const int row = a16.row(p), col = a16.col(q);
+          if (row < nF && col < r) HB[(long)row * Mr + l * r + col] = 2.0 * a16.v[p][q] + z[row] * wbar[l * r + col];
+        }
+    }
+    return;
+  }
+  TileAcc<TILE> acc;
+  for (int rt = 0; rt < (nF + TILE - 1) / TILE; ++rt) {
+    const int nrow = min(TILE, nF - rt * TILE);
+    for (int l = 0; l < M; ++l) {
+      acc.zero();
+      for (int k = 0; k < M; ++k) {
+        SRef b = sblock(gs, anc, r, k, l);
+        tile_mma<TILE>(acc, H + (long)rt * TILE * Mr + k * r, Mr, 1, nrow, b.p, b.sj, b.sk, r, r, stg);
+      }
+#pragma unroll
+      for (int p = 0; p < TileAcc<TILE>::RM; ++p)
+#pragma unroll
+        for (int q = 0; q < TileAcc<TILE>::RM; ++q) {
+          int row = acc.row(p), col = acc.col(q);
+          if (row < nrow && col < r) {
+            int o = rt * TILE + row;
+            HB[(long)o * Mr + l * r + col] = 2.0 * acc.v[p][q] + z[o] * wbar[l * r + col];
+          }
+        }
+    }
+  }
+}
+
+// Hbar of every leaf on the FP64 pipe, for an emulated gradient without its
+// assembled per-parent S (its other adjoints run in kernels of EM_NT threads,
+// the FP64 tiles take NT).  One CTA per leaf.
+__global__ void __launch_bounds__(NT) leaf_hbar_kernel(const Desc* __restrict__ D, GradState gs) {
+  extern __shared__ double smem[];
+  const Desc& ds = D[0];
+  const LeafState& lf = ds.lf;
+  const int M = ds.sh.M, r = ds.sh.r, Mr = M * r;
+  const long F = gs.rbase + blockIdx.x;         // compact leaf id
+  const long Fm = ds.st.mort[M][F], o0 = lf.off[Fm];
+  const int nF = (int)(lf.off[Fm + 1] - o0);
+  if (nF == 0) return;
+  double* wbar = smem;                           // M r
+  double* stg = wbar + MAXL * MAX_R_DEV;
+  long anc[MAXL];
+  for (int l = 0; l < M; ++l) anc[l] = ancestor(ds.st, M, F, l);
+  for (int t = threadIdx.x; t < Mr; t += NT) {
+    const int k = t / r;
+    wbar[t] = gs.Obar[k][anc[k] * r + (t - k * r)];
+  }
+  __syncthreads();
+  leaf_hbar<64>(gs, anc, M, r, nF, lf.H + o0 * Mr, lf.z + o0, wbar, gs.HB + o0 * Mr, stg);
+}
+
 // ---------------------------------------------------------------------------
 // Leaf adjoint: one CTA per leaf.
 // ---------------------------------------------------------------------------
@@ -347,13 +426,14 @@ __global__ void __launch_bounds__(NT) post_adjoint_kernel(int m, const Desc* __r
 // LSi' Hbar, Hbar V_F' and Sigmabar V_F run on the emulation engine (its
 // staging buffers open the dynamic shared memory); a timeout sets status.
 template <int TILE, bool EMU>
-__global__ void __launch_bounds__(NT) leaf_adjoint_kernel(const Desc* __restrict__ D, GradState gs, long slot0,
+__global__ void __launch_bounds__(EMU ? EM_NT : NT) leaf_adjoint_kernel(const Desc* __restrict__ D, GradState gs, long slot0,
                                                            int em_parts, int* status) {
+  constexpr int NTH = EMU ? EM_NT : NT;
   extern __shared__ __align__(1024) double smem_all[];
-  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ __align__(8) uint64_t mbar[EM_MBARS];
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
-  __shared__ int rexp[EMU ? EM_REXP : 1], cexp[EMU ? EM_CEXP : 1];
+  __shared__ __align__(16) int rexp[EMU ? EM_REXP : 1], cexp[EMU ? EM_CEXP : 1];
   // EMU: operand scales formed once per leaf (exponents, |x| < 2^e): rows of Hbar and of V_F per
   // 128-column group, their columns over the leaf's rows, the rows and columns of L_Sigma^{-1}, the
   // columns of L_Sigma, the rows of LSibar and of Sigmabar
@@ -393,16 +473,16 @@ __global__ void __launch_bounds__(NT) leaf_adjoint_kernel(const Desc* __restrict
     cx.fail = &fail;
     em_init(cx, &tmem_slot);
   }
-  TcAcc ea;                                  // EMU: the engine's accumulator
+  EmAcc ea;                                  // EMU: the engine's accumulator
   const int erow = ea.row(), ec0 = ea.col0();
   if (nF > 0) {
     long anc[MAXL];
     for (int l = 0; l < M; ++l) anc[l] = ancestor(st, M, F, l);
-    for (int t = threadIdx.x; t < Mr; t += NT) {
+    for (int t = threadIdx.x; t < Mr; t += NTH) {
       int k = t / r;
       wbar[t] = gs.Obar[k][anc[k] * r + (t - k * r)];
     }
-    for (int t = threadIdx.x; t < nF; t += NT) {
+    for (int t = threadIdx.x; t < nF; t += NTH) {
       sx[t] = lf.xs[o0 + t];
       sy[t] = lf.ys[o0 + t];
     }
@@ -421,47 +501,11 @@ __global__ void __launch_bounds__(NT) leaf_adjoint_kernel(const Desc* __restrict
     double* T3 = T2 + (long)nF * nF;
     const int nrt = (nF + TILE - 1) / TILE;
     TileAcc<TILE> acc;
-    // Hbar = 2 H S_p + z omegabar' (already in HB when the emulated form formed it); a leaf
-    // of at most 16 observations in one 16-row tile (sparse leaves: no FMA lanes on empty rows)
-    if (!(em_parts & 1) && TILE > 16 && nF <= 16) {
-      TileAccR<16, TILE> a16;
-      for (int l = 0; l < M; ++l) {
-        a16.zero();
-        for (int k = 0; k < M; ++k) {
-          SRef b = sblock(gs, anc, r, k, l);
-          tile_mma_r<16, TILE>(a16, H + k * r, Mr, 1, nF, b.p, b.sj, b.sk, r, r, stg);
-        }
-#pragma unroll
-        for (int p = 0; p < TileAccR<16, TILE>::RR; ++p)
-#pragma unroll
-          for (int q = 0; q < TileAccR<16, TILE>::RC; ++q) {
-            const int row = a16.row(p), col = a16.col(q);
-            if (row < nF && col < r) HB[(long)row * Mr + l * r + col] = 2.0 * a16.v[p][q] + z[row] * wbar[l * r + col];
-          }
-      }
-    }
-    for (int rt = 0; rt < nrt && !(em_parts & 1) && !(TILE > 16 && nF <= 16); ++rt) {
-      const int nrow = min(TILE, nF - rt * TILE);
-      for (int l = 0; l < M; ++l) {
-        acc.zero();
-        for (int k = 0; k < M; ++k) {
-          SRef b = sblock(gs, anc, r, k, l);
-          tile_mma<TILE>(acc, H + (long)rt * TILE * Mr + k * r, Mr, 1, nrow, b.p, b.sj, b.sk, r, r, stg);
-        }
-#pragma unroll
-        for (int p = 0; p < TileAcc<TILE>::RM; ++p)
-#pragma unroll
-          for (int q = 0; q < TileAcc<TILE>::RM; ++q) {
-            int row = acc.row(p), col = acc.col(q);
-            if (row < nrow && col < r) {
-              int o = rt * TILE + row;
-              HB[(long)o * Mr + l * r + col] = 2.0 * acc.v[p][q] + z[o] * wbar[l * r + col];
-            }
-          }
-      }
-    }
+    // Hbar = 2 H S_p + z omegabar' (already in HB when em_parts bit 0 is set)
+    if constexpr (!EMU)
+      if (!(em_parts & 1)) leaf_hbar<TILE>(gs, anc, M, r, nF, H, z, wbar, HB, stg);
     // zbar = H omegabar - z
-    for (int t = threadIdx.x; t < nF; t += NT) {
+    for (int t = threadIdx.x; t < nF; t += NTH) {
       double s = -z[t];
       for (int c = 0; c < Mr; ++c) s = fma(H[(long)t * Mr + c], wbar[c], s);
       zb[t] = s;
@@ -470,8 +514,8 @@ __global__ void __launch_bounds__(NT) leaf_adjoint_kernel(const Desc* __restrict
     if (EMU) {   // the operand scales, one pass over Hbar, V_F, L_Sigma^{-1} and L_Sigma
       const int ng = (Mr + EM_KG - 1) / EM_KG;
       const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-      for (int t = threadIdx.x; t < TC_M; t += NT) t1_r[t] = -2000;
-      for (int o = warp; o < TC_M; o += NT / 32)   // rows per group: a warp per row
+      for (int t = threadIdx.x; t < TC_M; t += NTH) t1_r[t] = -2000;
+      for (int o = warp; o < TC_M; o += NTH / 32)   // rows per group: a warp per row
         for (int g = 0; g < ng; ++g) {
           int eh = -2000, ev = -2000;
           if (o < nF)
@@ -486,7 +530,7 @@ __global__ void __launch_bounds__(NT) leaf_adjoint_kernel(const Desc* __restrict
             vf_r[g * TC_M + o] = ev;
           }
         }
-      for (int c = threadIdx.x; c < Mr; c += NT) {   // columns over the leaf's rows: a thread per column
+      for (int c = threadIdx.x; c < Mr; c += NTH) {   // columns over the leaf's rows: a thread per column
         int eh = -2000, ev = -2000;
         for (int o = 0; o < nF; ++o) {
           eh = max(eh, xexp_of(HB[(long)o * Mr + c]));
@@ -495,7 +539,7 @@ __global__ void __launch_bounds__(NT) leaf_adjoint_kernel(const Desc* __restrict
         hb_c[c] = eh;
         vf_c[c] = ev;
       }
-      for (int j = threadIdx.x; j < nF; j += NT) {   // L_Sigma^{-1} (lower) and L_Sigma
+      for (int j = threadIdx.x; j < nF; j += NTH) {   // L_Sigma^{-1} (lower) and L_Sigma
         int er = -2000, ec = -2000, el = -2000;
         for (int q = 0; q < nF; ++q) {
           er = max(er, xexp_of(LSi[(long)j * nF + q]));
@@ -514,7 +558,7 @@ __global__ void __launch_bounds__(NT) leaf_adjoint_kernel(const Desc* __restrict
       if (ok && erow < nF) {
         double* out = VB + (long)erow * Mr + l * r;
 #pragma unroll
-        for (int c = 0; c < 32; ++c)
+        for (int c = 0; c < EmAcc::NC; ++c)
           if (ec0 + c < r) out[ec0 + c] = ea.v[c];
       }
     }
@@ -532,7 +576,7 @@ __global__ void __launch_bounds__(NT) leaf_adjoint_kernel(const Desc* __restrict
       if (ok && erow < nF) {
         int e = -2000;
 #pragma unroll
-        for (int c = 0; c < 32; ++c) {
+        for (int c = 0; c < EmAcc::NC; ++c) {
           const int j = j0 + ec0 + c;
           if (ec0 + c < nb) {
             const double v = erow >= j ? ea.v[c] + zb[erow] * yv[j] : 0.0;
@@ -559,7 +603,7 @@ __global__ void __launch_bounds__(NT) leaf_adjoint_kernel(const Desc* __restrict
             }
           }
         if (bj < bi) {   // zero the mirrored upper block
-          for (int t = threadIdx.x; t < nj * ni; t += NT) {
+          for (int t = threadIdx.x; t < nj * ni; t += NTH) {
             int a = t / ni, b = t - a * ni;
             T1[(long)(bj * TILE + a) * nF + bi * TILE + b] = 0.0;
           }
@@ -571,7 +615,7 @@ __global__ void __launch_bounds__(NT) leaf_adjoint_kernel(const Desc* __restrict
       if (ok) ok = chol_inverse_adjoint_em(cx, T1, T2, T3, nF, nF, LSf, nF, LSi, nF, -1.0, t1_r, li_r, li_c, l_c);
       if (ok) {   // rows of Sigmabar for the product below
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        for (int o = warp; o < TC_M; o += NT / 32) {
+        for (int o = warp; o < TC_M; o += NTH / 32) {
           int e = -2000;
           if (o < nF)
             for (int c = lane; c < nF; c += 32) e = max(e, xexp_of(T3[(long)o * nF + c]));
@@ -583,7 +627,7 @@ __global__ void __launch_bounds__(NT) leaf_adjoint_kernel(const Desc* __restrict
       chol_inverse_adjoint<TILE>(T1, T2, T3, nF, nF, LSf, nF, LSi, nF, -1.0, stg);
     }
     // T3 = Sigmabar (symmetric): C0 and tau2 terms
-    for (int t = threadIdx.x; t < nF * nF; t += NT) {
+    for (int t = threadIdx.x; t < nF * nF; t += NTH) {
       int a = t / nF, b = t - a * nF;
       double sb = T3[t];
       double d1, d2, d3;
@@ -599,7 +643,7 @@ __global__ void __launch_bounds__(NT) leaf_adjoint_kernel(const Desc* __restrict
       if (ok && erow < nF) {
         double* out = VB + (long)erow * Mr + l * r;
 #pragma unroll
-        for (int c = 0; c < 32; ++c)
+        for (int c = 0; c < EmAcc::NC; ++c)
           if (ec0 + c < r) out[ec0 + c] -= 2.0 * ea.v[c];
       }
     }
@@ -623,7 +667,7 @@ __global__ void __launch_bounds__(NT) leaf_adjoint_kernel(const Desc* __restrict
       const double* Lia = st.Li[l] + a * (long)r * r;
       const double* Va = st.V[l] + a * (long)r * (l * r);
       __syncthreads();
-      load_knots(sh, l, st.mort[l][a], ax, ay);
+      load_knots<NTH>(sh, l, st.mort[l][a], ax, ay);
       __syncthreads();
       for (int rt = 0; rt < nrt; ++rt) {
         const int nrow = min(TILE, nF - rt * TILE);
@@ -663,10 +707,10 @@ __global__ void __launch_bounds__(NT) leaf_adjoint_kernel(const Desc* __restrict
     }
   }
   if (EMU) em_release(cx);
-  g_s2 = block_sum(g_s2, red);
-  g_k = block_sum(g_k, red);
-  g_t = block_sum(g_t, red);
-  g_nu = block_sum(g_nu, red);
+  g_s2 = block_sum<NTH>(g_s2, red);
+  g_k = block_sum<NTH>(g_k, red);
+  g_t = block_sum<NTH>(g_t, red);
+  g_nu = block_sum<NTH>(g_nu, red);
   if (EMU && !ok && threadIdx.x == 0) flag_error(status, ST_TIMEOUT, M, F);
   if (threadIdx.x == 0) {
     gs.gpart[GP * (slot0 + F) + 0] = g_s2;
@@ -712,13 +756,14 @@ __global__ void __launch_bounds__(NT) leaf_partial_kernel(const Desc* __restrict
 // emulation engine, whose staging buffers open the dynamic shared memory; a
 // timeout sets status.
 template <int TILE, bool EMU>
-__global__ void __launch_bounds__(NT) prior_adjoint_kernel(int m, const Desc* __restrict__ D, GradState gs,
+__global__ void __launch_bounds__(EMU ? EM_NT : NT) prior_adjoint_kernel(int m, const Desc* __restrict__ D, GradState gs,
                                                            long slot0, int* status) {
+  constexpr int NTH = EMU ? EM_NT : NT;
   extern __shared__ __align__(1024) double smem_all[];
-  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ __align__(8) uint64_t mbar[EM_MBARS];
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
-  __shared__ int rexp[EMU ? EM_REXP : 1], cexp[EMU ? EM_CEXP : 1];
+  __shared__ __align__(16) int rexp[EMU ? EM_REXP : 1], cexp[EMU ? EM_CEXP : 1];
   double* smem = smem_all + (EMU ? EM_STAGE_BYTES / sizeof(double) : 0);
   const Desc& ds = D[0];
   const Shape sh = ds.sh;
@@ -758,7 +803,7 @@ __global__ void __launch_bounds__(NT) prior_adjoint_kernel(int m, const Desc* __
     em_init(cx, &tmem_slot);
   }
   TileAcc<TILE> acc;
-  TcAcc ea;
+  EmAcc ea;
   // f(i, j, P(i, j)) for the r x r product P(i, j) = sum_{c < kk} A(i, c) B(j, c)
   auto product = [&](const double* A, long sai, long sak, const double* B, long sbj, long sbk, int kk, auto&& f) {
     if constexpr (EMU) {
@@ -766,7 +811,7 @@ __global__ void __launch_bounds__(NT) prior_adjoint_kernel(int m, const Desc* __
       const int row = ea.row(), c0 = ea.col0();
       if (ok && row < r) {
 #pragma unroll
-        for (int c = 0; c < 32; ++c)
+        for (int c = 0; c < EmAcc::NC; ++c)
           if (c0 + c < r) f(row, c0 + c, ea.v[c]);
       }
     } else {
@@ -790,18 +835,18 @@ __global__ void __launch_bounds__(NT) prior_adjoint_kernel(int m, const Desc* __
     const int row = ea.row(), c0 = ea.col0();
     if (ok && row < na) {
 #pragma unroll
-      for (int c = 0; c < 32; ++c)
+      for (int c = 0; c < EmAcc::NC; ++c)
         if (c0 + c < r) f(row, c0 + c, ea.v[c]);
     }
   };
   const int S = em_stack(r);
   double g_s2 = 0.0, g_k = 0.0, g_nu = 0.0;
-  load_knots(sh, m, st.mort[m][i], qx, qy);
+  load_knots<NTH>(sh, m, st.mort[m][i], qx, qy);
   const double* L = st.L[m] + i * (long)r * r;
   const double* Li = st.Li[m] + i * (long)r * r;
   const double* V = st.V[m] + i * (long)r * mr;
   // Libar = lower(incoming(m, m) L')  -> B0   (the adjoint of L^{-1} gathered from the subtree)
-  for (int t = threadIdx.x; t < r * r; t += NT) {
+  for (int t = threadIdx.x; t < r * r; t += NTH) {
     int a = t / r, b = t - a * r;
     B1[a * ld + b] = incoming(m, m, a, b);
   }
@@ -813,7 +858,7 @@ __global__ void __launch_bounds__(NT) prior_adjoint_kernel(int m, const Desc* __
   } else {
     chol_inverse_adjoint<TILE>(B0, B1, B2, ld, r, L, r, Li, r, 0.0, stg);
   }
-  for (int t = threadIdx.x; t < r * r; t += NT) {
+  for (int t = threadIdx.x; t < r * r; t += NTH) {
     int a = t / r, b = t - a * r;
     double d1, d2, d3;
     dcov0(cv, qx[a], qy[a], qx[b], qy[b], d1, d2, d3);
@@ -844,7 +889,7 @@ __global__ void __launch_bounds__(NT) prior_adjoint_kernel(int m, const Desc* __
     const double* Lia = st.Li[l] + a * (long)r * r;
     const double* Va = st.V[l] + a * (long)r * (l * r);
     __syncthreads();
-    load_knots(sh, l, st.mort[l][a], ax, ay);
+    load_knots<NTH>(sh, l, st.mort[l][a], ax, ay);
     __syncthreads();
     auto xbar_epi = [&](int row, int col, double xb) {
       XB[(long)row * mr + l * r + col] = xb;
@@ -900,9 +945,9 @@ __global__ void __launch_bounds__(NT) prior_adjoint_kernel(int m, const Desc* __
       }
   }
   if (EMU) em_release(cx);
-  g_s2 = block_sum(g_s2, red);
-  g_k = block_sum(g_k, red);
-  g_nu = block_sum(g_nu, red);
+  g_s2 = block_sum<NTH>(g_s2, red);
+  g_k = block_sum<NTH>(g_k, red);
+  g_nu = block_sum<NTH>(g_nu, red);
   if (threadIdx.x == 0) {
     gs.gpart[GP * (slot0 + i) + 0] = g_s2;
     gs.gpart[GP * (slot0 + i) + 1] = g_k;
@@ -968,7 +1013,7 @@ static cudaError_t launch_leaf_adjoint(int tile, int nleaves, size_t sm, cudaStr
   if ((e = cudaFuncSetAttribute(leaf_adjoint_kernel<T, EMU>, cudaFuncAttributeMaxDynamicSharedMemorySize,     \
                                 (int)sm)))                                                                    \
     return e;                                                                                                 \
-  leaf_adjoint_kernel<T, EMU><<<nleaves, NT, sm, s>>>(d_desc, gs, slot0, em_parts, status);
+  leaf_adjoint_kernel<T, EMU><<<nleaves, EMU ? EM_NT : NT, sm, s>>>(d_desc, gs, slot0, em_parts, status);
   if constexpr (EMU) {   // the emulated instances use 64-wide FP64 tiles only (fewer instantiations)
     MRA_LEAF_ADJ(64)
   } else {
@@ -992,7 +1037,7 @@ static cudaError_t launch_post_adjoint(int tile, int m, int nregions, size_t sm,
   if ((e = cudaFuncSetAttribute(post_adjoint_kernel<T, EMU>, cudaFuncAttributeMaxDynamicSharedMemorySize,    \
                                 (int)sm)))                                                                    \
     return e;                                                                                                 \
-  post_adjoint_kernel<T, EMU><<<nregions, NT, sm, s>>>(m, d_desc, gs, gb_ready, status);
+  post_adjoint_kernel<T, EMU><<<nregions, EMU ? EM_NT : NT, sm, s>>>(m, d_desc, gs, gb_ready, status);
   if constexpr (EMU) {   // the emulated instances use 64-wide FP64 tiles only (fewer instantiations)
     MRA_POST_ADJ(64)
   } else {
@@ -1016,7 +1061,7 @@ static cudaError_t launch_prior_adjoint(int tile, int m, int nregions, size_t sm
   if ((e = cudaFuncSetAttribute(prior_adjoint_kernel<T, EMU>, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
                                 (int)sm)))                                                                    \
     return e;                                                                                                 \
-  prior_adjoint_kernel<T, EMU><<<nregions, NT, sm, s>>>(m, d_desc, gs, slot0, status);
+  prior_adjoint_kernel<T, EMU><<<nregions, EMU ? EM_NT : NT, sm, s>>>(m, d_desc, gs, slot0, status);
   if constexpr (EMU) {   // the emulated instances use 64-wide FP64 tiles only (fewer instantiations)
     MRA_PRIOR_ADJ(64)
   } else {
@@ -1103,9 +1148,15 @@ cudaError_t launch_grad_range(const Desc& hd, const Desc* d_desc, GradState gs, 
     }
     gs.rbase = base(M);
     size_t sm = sizeof(double) * (MAXL * MAX_R_DEV + 3 * 128 + 2 * MAX_R_DEV + 32) + stg;
-    if (emu) {   // (the emulated instance's FP64 tiles are 64 wide: its staging sized for them)
-      sm += EM_STAGE_BYTES + sizeof(double) * 2 * KC * (64 + 2) - stg;
-      if (sm < EM_SOLO_SMEM) sm = EM_SOLO_SMEM;
+    if (emu) {
+      if (!(em_parts & 1)) {
+        const size_t sh = sizeof(double) * (MAXL * MAX_R_DEV + 2 * KC * (64 + 2));
+        if ((e = cudaFuncSetAttribute(leaf_hbar_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh))) return e;
+        leaf_hbar_kernel<<<(unsigned)count(M), NT, sh, s>>>(d_desc, gs);
+        if ((e = cudaGetLastError())) return e;
+        ++*launches;
+      }
+      sm = std::max(sm - stg + EM_STAGE_BYTES, EM_SOLO_SMEM);
       e = launch_leaf_adjoint<true>(tile, (int)count(M), sm, s, d_desc, gs, slot_leaf, em_parts, status);
     } else {
       e = launch_leaf_adjoint<false>(tile, (int)count(M), sm, s, d_desc, gs, slot_leaf, em_parts, status);

@@ -183,9 +183,10 @@ __host__ __device__ __forceinline__ int leaf_bits(const Shape& sh) { return lvl_
 constexpr unsigned long long QUAD_HALVINGS = 0x1111111111110ull;
 
 // Fill sx/sy (shared) with the r knots of region (m, i).
+template <int NTH = NT>
 __device__ __forceinline__ void load_knots(const Shape& sh, int m, long i, double* sx, double* sy) {
   Box b = region_box(sh.bbox, sh.hx, sh.hy, m, i);
-  for (int q = threadIdx.x; q < sh.gx * sh.gy; q += NT) knot_xy(b, sh.gx, sh.gy, q, sx[q], sy[q]);
+  for (int q = threadIdx.x; q < sh.gx * sh.gy; q += NTH) knot_xy(b, sh.gx, sh.gy, q, sx[q], sy[q]);
 }
 
 // Everything a kernel needs about one dataset, in device memory.  A single

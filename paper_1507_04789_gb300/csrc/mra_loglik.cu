@@ -298,13 +298,14 @@ __global__ void __launch_bounds__(NT) leaf_syrk_kernel(const Desc* __restrict__ 
 // EMU: the products G^l = Lt^{-1} Ahat^{m,l} on the emulation engine (its
 // staging buffers open the dynamic shared memory).
 template <int TILE, bool EMU>
-__global__ void __launch_bounds__(NT) post_level_kernel(int m, const Desc* __restrict__ D,
+__global__ void __launch_bounds__(EMU ? EM_NT : NT) post_level_kernel(int m, const Desc* __restrict__ D,
                                                         const int2* __restrict__ work, int* status) {
+  constexpr int NTH = EMU ? EM_NT : NT;
   extern __shared__ __align__(1024) double smem_all[];
-  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ __align__(8) uint64_t mbar[EM_MBARS];
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
-  __shared__ int rexp[EMU ? EM_REXP : 1], cexp[EMU ? EM_CEXP : 1];
+  __shared__ __align__(16) int rexp[EMU ? EM_REXP : 1], cexp[EMU ? EM_CEXP : 1];
   double* smem = smem_all + (EMU ? EM_STAGE_BYTES / sizeof(double) : 0);
   EmCtx cx;
   bool ok = true;
@@ -334,44 +335,44 @@ __global__ void __launch_bounds__(NT) post_level_kernel(int m, const Desc* __res
   if (threadIdx.x == 0) bad = 0;
   const double* A = st.Acc[m] + i * (long)T * r * r;
   const double* Amm = A + (long)tri_index(m, m) * r * r;
-  for (int t = threadIdx.x; t < r * r; t += NT) {
+  for (int t = threadIdx.x; t < r * r; t += NTH) {
     int a = t / r, b = t % r;
     W[a * ldw + b] = Amm[t] + (a == b ? 1.0 : 0.0);
   }
-  chol_smem(W, r, ldw, &bad);
+  chol_smem<NTH>(W, r, ldw, &bad);
   double ld = 0.0;
-  for (int t = threadIdx.x; t < r; t += NT) ld += log(W[t * ldw + t]);
-  ld = 2.0 * block_sum(ld, red);
+  for (int t = threadIdx.x; t < r; t += NTH) ld += log(W[t * ldw + t]);
+  ld = 2.0 * block_sum<NTH>(ld, red);
   if (st.Ltf[m]) {
     double* Lf = st.Ltf[m] + i * (long)r * r;
-    for (int t = threadIdx.x; t < r * r; t += NT) Lf[t] = W[(t / r) * ldw + (t % r)];
+    for (int t = threadIdx.x; t < r * r; t += NTH) Lf[t] = W[(t / r) * ldw + (t % r)];
     __syncthreads();
   }
-  trinv_smem(W, r, ldw, tmp);
+  trinv_smem<NTH>(W, r, ldw, tmp);
   double* Lt = st.Lt[m] + i * (long)r * r;
-  for (int t = threadIdx.x; t < r * r; t += NT) Lt[t] = W[(t / r) * ldw + (t % r)];
+  for (int t = threadIdx.x; t < r * r; t += NTH) Lt[t] = W[(t / r) * ldw + (t % r)];
   // g = Lt^{-1} omegahat^m
   const double* om = st.Om[m] + (i * (m + 1) + m) * (long)r;
   double gg = 0.0;
-  for (int a = threadIdx.x; a < r; a += NT) {
+  for (int a = threadIdx.x; a < r; a += NTH) {
     double s = 0.0;
     for (int b = 0; b <= a; ++b) s = fma(W[a * ldw + b], om[b], s);
     gs[a] = s;
     st.gv[m][i * r + a] = s;
     gg = fma(s, s, gg);
   }
-  gg = block_sum(gg, red);
+  gg = block_sum<NTH>(gg, red);
   // G^l = Lt^{-1} Ahat^{m,l}, l < m.  Ahat^{m,l}(a, b) is stored row-major.
   double* Gr = st.G[m] + i * (long)r * mr;
   if constexpr (EMU) {
-    TcAcc ea;
+    EmAcc ea;
     const int row = ea.row(), c0 = ea.col0();
     for (int l = 0; l < m && ok; ++l) {
       const double* Aml = A + (long)tri_index(m, l) * r * r;
       ok = em_mma(cx, ea, W, ldw, 1, r, Aml, 1, r, r, r);
       if (ok && row < r) {
 #pragma unroll
-        for (int c = 0; c < 32; ++c)
+        for (int c = 0; c < EmAcc::NC; ++c)
           if (c0 + c < r) Gr[(long)row * mr + l * r + c0 + c] = ea.v[c];
       }
     }
@@ -392,7 +393,7 @@ __global__ void __launch_bounds__(NT) post_level_kernel(int m, const Desc* __res
   }
   if (st.gcol[m]) {   // emulation: column scales of G over its r rows, for the aggregation above
     __syncthreads();
-    for (int c = threadIdx.x; c < mr; c += NT) {
+    for (int c = threadIdx.x; c < mr; c += NTH) {
       int e = -2000;
       for (int a = 0; a < r; ++a) e = max(e, xexp_of(Gr[(long)a * mr + c]));
       st.gcol[m][i * (long)mr + c] = e;
@@ -514,7 +515,7 @@ static cudaError_t launch_post_level(bool emu, int tile, int m, int nblocks, cud
     if ((e = cudaFuncSetAttribute(post_level_kernel<T, EMU>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                   (int)sm)))                                                              \
       return e;                                                                                           \
-    post_level_kernel<T, EMU><<<nblocks, NT, sm, s>>>(m, d_desc, work, status);                           \
+    post_level_kernel<T, EMU><<<nblocks, EMU ? EM_NT : NT, sm, s>>>(m, d_desc, work, status);                           \
   }
   if (tile == 16) {
     if (emu) MRA_POST(16, true) else MRA_POST(16, false)

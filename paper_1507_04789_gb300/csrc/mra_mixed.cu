@@ -9,7 +9,7 @@
 //  * MRA_PREC_MIXED: tc_mma (3xTF32 with FP64 accumulation every 64 terms);
 //    the Gram products of the posterior pass (leaf_syrk, aggregate) stay in
 //    the FP64 kernels, since they need more than FP32 accuracy;
-//  * MRA_PREC_EMU: em_mma (bf16-slice FP64 emulation, about 1e-14 relative),
+//  * MRA_PREC_EMU: em_mma (f16-digit FP64 emulation, about 1e-14 relative),
 //    which also runs the two Gram products (leaf_syrk_kernel_em,
 //    aggregate_kernel_em below).
 // The Cholesky factorisations, triangular inverses, log-determinants and the
@@ -23,15 +23,17 @@
 namespace mra {
 
 // The tensor-core engine of a kernel: 3xTF32 (EMU = false) or the FP64-grade
-// bf16-slice emulation (EMU = true); both write the same TcAcc layout.  Every
-// call site zeroes the accumulator first: the 3xTF32 engine adds to it, the
-// emulation engine overwrites it.
+// f16-digit emulation (EMU = true), each with its threads per CTA (NTH) and its
+// accumulator (Acc: row(), col0() and NC columns of the 128 x 64 tile per
+// thread).  Every call site zeroes the accumulator first: the 3xTF32 engine
+// adds to it, the emulation engine overwrites it.
 template <bool EMU>
 struct Engine;
 
 template <>
 struct Engine<false> {
-  static constexpr int STAGE = TC_STAGE_BYTES;
+  static constexpr int STAGE = TC_STAGE_BYTES, NTH = NT, MBARS = 1;
+  using Acc = TcAcc;
   TcCtx cx;
   __device__ void init(unsigned char* stage, uint64_t* mbar, uint32_t* tmem_slot, int* fail, int*, int*) {
     cx = TcCtx{reinterpret_cast<uint32_t*>(stage), mbar, 0, 0, fail};
@@ -46,7 +48,8 @@ struct Engine<false> {
 
 template <>
 struct Engine<true> {
-  static constexpr int STAGE = EM_STAGE_BYTES;
+  static constexpr int STAGE = EM_STAGE_BYTES, NTH = EM_NT, MBARS = EM_MBARS;
+  using Acc = EmAcc;
   EmCtx cx;
   __device__ void init(unsigned char* stage, uint64_t* mbar, uint32_t* tmem_slot, int* fail, int* rexp, int* cexp) {
     cx.stage = reinterpret_cast<uint16_t*>(stage);
@@ -57,7 +60,7 @@ struct Engine<true> {
     em_init(cx, tmem_slot);
   }
   // pa / pb: the operands' row scales from their producers (see em_mma), or null
-  __device__ bool mma(TcAcc& acc, const double* A, long sai, long sak, int na, const double* B, long sbj, long sbk,
+  __device__ bool mma(EmAcc& acc, const double* A, long sai, long sak, int na, const double* B, long sbj, long sbk,
                       int nb, int K, const int* pa = nullptr, int pas = 0, const int* pb = nullptr, int pbs = 0) {
     return em_mma(cx, acc, A, sai, sak, na, B, sbj, sbk, nb, K, pa, pas, pb, pbs);
   }
@@ -73,14 +76,15 @@ constexpr int EM_GMAX = 6;   // 128-column groups of a row of at most MRA_MAX_M 
 // ancestor's V and L^{-1} split once for all of them), and their W blocks are
 // factorised and inverted block by block (chol_seg / trinv_seg, stacked rows).
 template <bool EMU>
-__global__ void __launch_bounds__(NT) prior_level_kernel_tc(int m, const Desc* __restrict__ D,
+__global__ void __launch_bounds__(Engine<EMU>::NTH) prior_level_kernel_tc(int m, const Desc* __restrict__ D,
                                                              const int2* __restrict__ work, int* status,
                                                              const int* __restrict__ gcnt, int rcap) {
+  constexpr int NTH = Engine<EMU>::NTH, NC = Engine<EMU>::Acc::NC;   // threads, columns of the tile per thread
   extern __shared__ __align__(1024) unsigned char dsm[];
-  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ __align__(8) uint64_t mbar[Engine<EMU>::MBARS];
   __shared__ uint32_t tmem_slot;
   __shared__ int fail, bad;
-  __shared__ int rexp[EMU ? EM_REXP : 1], cexp[EMU ? EM_CEXP : 1];
+  __shared__ __align__(16) int rexp[EMU ? EM_REXP : 1], cexp[EMU ? EM_CEXP : 1];
   // emulation: row scales of the stacked V rows per 128-column group, and of the current X^l block
   __shared__ int vsc[EMU ? EM_GMAX * TC_M : 1], xsc[EMU ? TC_M : 1];
   // c0_fast on two knot grids: squared scaled offsets between their columns and
@@ -106,13 +110,13 @@ __global__ void __launch_bounds__(NT) prior_level_kernel_tc(int m, const Desc* _
     if (threadIdx.x == 0) flag_error(status, ST_LIMIT, m, it.i);
     return;
   }
-  for (int q = threadIdx.x; q < r; q += NT) {
+  for (int q = threadIdx.x; q < r; q += NTH) {
     qcol[q] = (unsigned char)(q % gx);
     qrow[q] = (unsigned char)(q / gx);
   }
   if (threadIdx.x <= G) gseg[threadIdx.x] = threadIdx.x * r;
   if (EMU)
-    for (int t = threadIdx.x; t < EM_GMAX * TC_M; t += NT) vsc[t] = -2000;
+    for (int t = threadIdx.x; t < EM_GMAX * TC_M; t += NTH) vsc[t] = -2000;
   const long i = it.i;                          // the first region of the group
   double* qx = reinterpret_cast<double*>(dsm + Engine<EMU>::STAGE);   // the group's knots, rcap each
   double* qy = qx + rcap;
@@ -125,7 +129,7 @@ __global__ void __launch_bounds__(NT) prior_level_kernel_tc(int m, const Desc* _
   // synchronises before and after)
   const int gsz = gx * gx + gy * gy;
   auto grid_offsets = [&](const double* bx, const double* by, bool self) {
-    for (int t = threadIdx.x; t < G * gsz; t += NT) {
+    for (int t = threadIdx.x; t < G * gsz; t += NTH) {
       const int g = t / gsz, u = t - g * gsz;
       const double* ox = qx + g * r;
       const double* oy = qy + g * r;
@@ -140,7 +144,7 @@ __global__ void __launch_bounds__(NT) prior_level_kernel_tc(int m, const Desc* _
         pdy[g * C0_GMAX * C0_GMAX + v] = d * d;
       }
     }
-    for (int t = threadIdx.x; t < G * gx; t += NT) {
+    for (int t = threadIdx.x; t < G * gx; t += NTH) {
       const int g = t / gx, c = t - g * gx;
       pgp[t] = cv.sigma2 * c0_vfac(cv, qx[g * r + c]);
       pgq[t] = c0_vfac(cv, self ? qx[g * r + c] : bx[c]);
@@ -158,18 +162,18 @@ __global__ void __launch_bounds__(NT) prior_level_kernel_tc(int m, const Desc* _
   if (threadIdx.x == 0) bad = 0;
   Engine<EMU> eng;
   eng.init(dsm, mbar, &tmem_slot, &fail, rexp, cexp);
-  for (int g = 0; g < G; ++g) load_knots(sh, m, st.mort[m][i + g], qx + g * r, qy + g * r);
+  for (int g = 0; g < G; ++g) load_knots<NTH>(sh, m, st.mort[m][i + g], qx + g * r, qy + g * r);
   double* Vrow = st.V[m] + i * (long)r * mr;   // the group's rows are consecutive
-  TcAcc acc;
+  typename Engine<EMU>::Acc acc;
   bool ok = true;
   const int row = acc.row(), c0 = acc.col0();
   for (int l = 0; l < m && ok; ++l) {
     const long a = ancestor(st, m, i, l);
     __syncthreads();
-    load_knots(sh, l, st.mort[l][a], ax, ay);
+    load_knots<NTH>(sh, l, st.mort[l][a], ax, ay);
     const double* Vanc = st.V[l] + a * (long)r * (l * r);
     if (EMU)
-      for (int t = threadIdx.x; t < TC_M; t += NT) xsc[t] = -2000;
+      for (int t = threadIdx.x; t < TC_M; t += NTH) xsc[t] = -2000;
     __syncthreads();
     if (fast) {
       grid_offsets(ax, ay, false);
@@ -177,7 +181,7 @@ __global__ void __launch_bounds__(NT) prior_level_kernel_tc(int m, const Desc* _
     }
     // C0(Q_R, Q_{R_l}) into block l, spread over every warp (the FP64 pipe of
     // every SM sub-partition); the product below reads only blocks < l
-    for (int t = threadIdx.x; t < R * r; t += NT) {
+    for (int t = threadIdx.x; t < R * r; t += NTH) {
       const int qi = t / r, qj = t - qi * r;
       const double v = c0_at(qi, qj, ax, ay);
       Vrow[(long)qi * mr + l * r + qj] = v;
@@ -192,7 +196,7 @@ __global__ void __launch_bounds__(NT) prior_level_kernel_tc(int m, const Desc* _
       if (row < R) {
         int e = -2000;
         #pragma unroll
-        for (int c = 0; c < 32; ++c) {
+        for (int c = 0; c < NC; ++c) {
           const int col = c0 + c;
           if (col < r) {
             const double v = Vrow[(long)row * mr + l * r + col] - acc.v[c];
@@ -209,10 +213,10 @@ __global__ void __launch_bounds__(NT) prior_level_kernel_tc(int m, const Desc* _
                  EMU ? st.liexp[l] + a * r : nullptr, 0);
     if (!ok) break;
     if (row < R) {
-      int e0 = -2000, e1 = -2000;       // a thread's 32 columns touch at most two groups
+      int e0 = -2000, e1 = -2000;       // a thread's columns touch at most two groups
       const int gbase = (l * r + c0) / 128;
       #pragma unroll
-      for (int c = 0; c < 32; ++c) {
+      for (int c = 0; c < NC; ++c) {
         const int col = c0 + c;
         if (col < r) {
           Vrow[(long)row * mr + l * r + col] = acc.v[c];
@@ -235,7 +239,7 @@ __global__ void __launch_bounds__(NT) prior_level_kernel_tc(int m, const Desc* _
   }
   // lower triangle of every region's C0(Q_R, Q_R), every warp
   const int T1 = r * (r + 1) / 2;
-  for (int t = threadIdx.x; t < G * T1; t += NT) {
+  for (int t = threadIdx.x; t < G * T1; t += NTH) {
     const int g = t / T1;
     int qi, qj;
     tri_decode(t - g * T1, qi, qj);
@@ -253,7 +257,7 @@ __global__ void __launch_bounds__(NT) prior_level_kernel_tc(int m, const Desc* _
     if (row < R) {
       const int rb = (row / r) * r;           // the row's block
       #pragma unroll
-      for (int c = 0; c < 32; ++c) {
+      for (int c = 0; c < NC; ++c) {
         const int oj = ct * TC_N + c0 + c;
         if (c0 + c < ncol && oj >= rb && oj <= row) W[row * ldw + oj - rb] -= acc.v[c];
       }
@@ -261,26 +265,26 @@ __global__ void __launch_bounds__(NT) prior_level_kernel_tc(int m, const Desc* _
     __syncthreads();
   }
   if (ok) {
-    if (G == 1) chol_smem(W, r, ldw, &bad);
-    else chol_seg<true>(W, ldw, gseg, G, &bad, gpv);
+    if (G == 1) chol_smem<NTH>(W, r, ldw, &bad);
+    else chol_seg<true, NTH>(W, ldw, gseg, G, &bad, gpv);
     if (st.L[m]) {
       double* Lr = st.L[m] + i * (long)r * r;
-      for (int t = threadIdx.x; t < R * r; t += NT) Lr[t] = W[(t / r) * ldw + (t % r)];
+      for (int t = threadIdx.x; t < R * r; t += NTH) Lr[t] = W[(t / r) * ldw + (t % r)];
       __syncthreads();
     }
-    if (G == 1) trinv_smem(W, r, ldw, tmp);
-    else trinv_seg<true>(W, ldw, gseg, G, tmp, gpv);
+    if (G == 1) trinv_smem<NTH>(W, r, ldw, tmp);
+    else trinv_seg<true, NTH>(W, ldw, gseg, G, tmp, gpv);
     double* Li = st.Li[m] + i * (long)r * r;
-    for (int t = threadIdx.x; t < R * r; t += NT) Li[t] = W[(t / r) * ldw + (t % r)];
+    for (int t = threadIdx.x; t < R * r; t += NTH) Li[t] = W[(t / r) * ldw + (t % r)];
     if (EMU) {   // row scales of V_R and L_R^{-1} for the descendants' products
-      for (int t = threadIdx.x; t < R; t += NT) {
+      for (int t = threadIdx.x; t < R; t += NTH) {
         int e = -2000;
         for (int k = 0; k <= t % r; ++k) e = max(e, xexp_of(W[t * ldw + k]));
         st.liexp[m][i * r + t] = e;
       }
       if (m > 0) {
         const int ng = (mr + 127) / 128;
-        for (int t = threadIdx.x; t < ng * R; t += NT) {   // region g = q / r, group t / R, row q % r
+        for (int t = threadIdx.x; t < ng * R; t += NTH) {   // region g = q / r, group t / R, row q % r
           const int grp = t / R, q = t - grp * R, g = q / r;
           st.vexp[m][((i + g) * ng + grp) * (long)r + (q - g * r)] = vsc[grp * TC_M + q];
         }
@@ -304,14 +308,15 @@ __global__ void __launch_bounds__(NT) prior_level_kernel_tc(int m, const Desc* _
 // tile: the levels l < M - 1 (their common ancestors) are one product per
 // level for the whole tile, level M - 1 one product per region on its rows.
 template <bool GRP>
-__global__ void __launch_bounds__(NT) chain_forward_kernel_em(const Desc* __restrict__ D,
+__global__ void __launch_bounds__(EM_NT) chain_forward_kernel_em(const Desc* __restrict__ D,
                                                               const int2* __restrict__ work, int* status,
                                                               const int* __restrict__ gcnt) {
+  constexpr int NTH = EM_NT, NC = EmAcc::NC;
   extern __shared__ __align__(1024) unsigned char dsm[];
-  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ __align__(8) uint64_t mbar[EM_MBARS];
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
-  __shared__ int rexp[EM_REXP], cexp[EM_CEXP];
+  __shared__ __align__(16) int rexp[EM_REXP], cexp[EM_CEXP];
   __shared__ int hsc[EM_GMAX * TC_M], xsc[TC_M];
   __shared__ double sx[TC_M], sy[TC_M], ax[MAX_R_DEV], ay[MAX_R_DEV];
   // c0_fast: squared scaled offsets of the tile's points to the knot grid's
@@ -340,25 +345,25 @@ __global__ void __launch_bounds__(NT) chain_forward_kernel_em(const Desc* __rest
   const int gx = sh.gx, gy = sh.gy;
   const bool fast = c0_fast_ok(cv, gx, gy);
   const double c0s = c0_scale(cv), is2 = 1.0 / cv.sigma2;
-  for (int q = threadIdx.x; q < r; q += NT) {
+  for (int q = threadIdx.x; q < r; q += NTH) {
     qcol[q] = (unsigned char)(q % gx);
     qrow[q] = (unsigned char)(q / gx);
   }
   Engine<true> eng;
   eng.init(dsm, mbar, &tmem_slot, &fail, rexp, cexp);
-  TcAcc acc;
+  EmAcc acc;
   bool ok = true;
   const int row = acc.row(), c0 = acc.col0();
   for (long t0 = row0; t0 < row1 && ok; t0 += TC_M) {
     const int na = (int)min((long)TC_M, row1 - t0);
     double* Hrow = lf.H + t0 * Mr;
     __syncthreads();                             // the previous tile's points and scales are no longer read
-    for (int t = threadIdx.x; t < na; t += NT) {
+    for (int t = threadIdx.x; t < na; t += NTH) {
       sx[t] = lf.xs[t0 + t];
       sy[t] = lf.ys[t0 + t];
       if (fast) c0gp[t] = cv.sigma2 * c0_vfac(cv, sx[t]);
     }
-    for (int t = threadIdx.x; t < EM_GMAX * TC_M; t += NT) hsc[t] = -2000;
+    for (int t = threadIdx.x; t < EM_GMAX * TC_M; t += NTH) hsc[t] = -2000;
     for (int l = 0; l < M && ok; ++l)
     for (int sg = 0; sg < (G > 1 && l == M - 1 ? G : 1) && ok; ++sg) {   // (level M - 1 of a group: per region)
       const bool per = G > 1 && l == M - 1;
@@ -367,23 +372,23 @@ __global__ void __launch_bounds__(NT) chain_forward_kernel_em(const Desc* __rest
       if (nr == 0) continue;                     // (uniform: a region without observations)
       double* Hseg = Hrow + (long)ra * Mr;
       __syncthreads();
-      load_knots(sh, l, st.mort[l][a], ax, ay);
+      load_knots<NTH>(sh, l, st.mort[l][a], ax, ay);
       const double* Vanc = st.V[l] + a * (long)r * (l * r);
-      for (int t = threadIdx.x; t < TC_M; t += NT) xsc[t] = -2000;
+      for (int t = threadIdx.x; t < TC_M; t += NTH) xsc[t] = -2000;
       __syncthreads();
       if (fast) {   // offsets to the knot grid's gx columns and gy rows, knot columns' variance factors
         const int gs = gx + gy;
-        for (int t = threadIdx.x; t < nr * gs; t += NT) {
+        for (int t = threadIdx.x; t < nr * gs; t += NTH) {
           const int fi = ra + t / gs, c = t - (t / gs) * gs;
           const double d = c < gx ? c0s * (sx[fi] - ax[c]) : c0s * (sy[fi] - ay[(c - gx) * gx]);
           (c < gx ? c0dx + fi * gx + c : c0dy + fi * gy + (c - gx))[0] = d * d;
         }
-        for (int c = threadIdx.x; c < gx; c += NT) c0gq[c] = c0_vfac(cv, ax[c]);
+        for (int c = threadIdx.x; c < gx; c += NTH) c0gq[c] = c0_vfac(cv, ax[c]);
         __syncthreads();
       }
       // C0(S_F, Q_l) into block l (the product below reads only blocks < l); in
       // gradient calls with its two derivatives
-      for (int t = threadIdx.x; t < nr * r; t += NT) {
+      for (int t = threadIdx.x; t < nr * r; t += NTH) {
         const int fi = ra + t / r, qj = t - (t / r) * r;
         double v;
         if (fast) {
@@ -415,7 +420,7 @@ __global__ void __launch_bounds__(NT) chain_forward_kernel_em(const Desc* __rest
         if (row < nr) {
           int e = -2000;
 #pragma unroll
-          for (int c = 0; c < 32; ++c) {
+          for (int c = 0; c < NC; ++c) {
             const int col = c0 + c;
             if (col < r) {
               const double v = Hseg[(long)row * Mr + l * r + col] - acc.v[c];
@@ -432,10 +437,10 @@ __global__ void __launch_bounds__(NT) chain_forward_kernel_em(const Desc* __rest
                    st.liexp[l] + a * r, 0);
       if (!ok) break;
       if (row < nr) {
-        int e0 = -2000, e1 = -2000;       // a thread's 32 columns touch at most two groups
+        int e0 = -2000, e1 = -2000;       // a thread's columns touch at most two groups
         const int gbase = (l * r + c0) / 128;
 #pragma unroll
-        for (int c = 0; c < 32; ++c) {
+        for (int c = 0; c < NC; ++c) {
           const int col = c0 + c;
           if (col < r) {
             Hseg[(long)row * Mr + l * r + col] = acc.v[c];
@@ -449,7 +454,7 @@ __global__ void __launch_bounds__(NT) chain_forward_kernel_em(const Desc* __rest
       }
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < na * ng; t += NT) {
+    for (int t = threadIdx.x; t < na * ng; t += NTH) {
       const int i = t / ng, g = t - i * ng;
       lf.hrow[(t0 + i) * ng + g] = hsc[g * TC_M + i];
     }
@@ -457,7 +462,7 @@ __global__ void __launch_bounds__(NT) chain_forward_kernel_em(const Desc* __rest
       for (int g = 0; g < G; ++g) {
         const int ra = G > 1 ? gseg[g] : 0, rb = G > 1 ? gseg[g + 1] : na;
         int32_t* out = lf.vfexp + ((P + g) * 4 + (G > 1 ? 0 : (t0 - row0) / TC_M)) * (long)Mr;
-        for (int c = threadIdx.x; c < Mr; c += NT) {
+        for (int c = threadIdx.x; c < Mr; c += NTH) {
           int e = -2000;
           for (int i = ra; i < rb; ++i) e = max(e, xexp_of(Hrow[(long)i * Mr + c]));
           out[c] = e;
@@ -478,13 +483,14 @@ __global__ void __launch_bounds__(NT) chain_forward_kernel_em(const Desc* __rest
 // inverted block by block (chol_seg, trinv_seg), and H = L^{-1} V_F is one
 // product for all of them (the inverse is zero outside the blocks).
 template <bool EMU>
-__global__ void __launch_bounds__(NT) leaf_kernel_tc(const Desc* __restrict__ D, const int2* __restrict__ work,
+__global__ void __launch_bounds__(Engine<EMU>::NTH) leaf_kernel_tc(const Desc* __restrict__ D, const int2* __restrict__ work,
                                                      int* status, int chain_done, const int* __restrict__ gcnt) {
+  constexpr int NTH = Engine<EMU>::NTH, NC = Engine<EMU>::Acc::NC;   // threads, columns of the tile per thread
   extern __shared__ __align__(1024) unsigned char dsm[];
-  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ __align__(8) uint64_t mbar[Engine<EMU>::MBARS];
   __shared__ uint32_t tmem_slot;
   __shared__ int fail, bad;
-  __shared__ int rexp[EMU ? EM_REXP : 1], cexp[EMU ? EM_CEXP : 1];
+  __shared__ __align__(16) int rexp[EMU ? EM_REXP : 1], cexp[EMU ? EM_CEXP : 1];
   // emulation: row scales of H rows per 128-column group, of the current X^l block, of L_Sigma^{-1}
   __shared__ int hsc[EMU ? EM_GMAX * TC_M : 1], xsc[EMU ? TC_M : 1], ssc[EMU ? TC_M : 1];
   const Item it = work_item(work);
@@ -516,13 +522,13 @@ __global__ void __launch_bounds__(NT) leaf_kernel_tc(const Desc* __restrict__ D,
   double* tmp = sv + nlmax;
   double* ax = tmp + nlmax;
   double* ay = ax + MAX_R_DEV;
-  double* red = ay + MAX_R_DEV;                 // block sums (red[0..7]) or a group's pivots (red[0..3])
-  double* S = red + 32;                         // nlmax x (nlmax + 1)
+  double* red = ay + MAX_R_DEV;                 // block sums (red[0..15]) or a group's pivots (red[0..3])
+  double* S = red + 40;                         // nlmax x (nlmax + 1)
   // a group's leaves: rows gseg[k] .. gseg[k + 1] - 1, and the leaf of every row
-  int* gseg = reinterpret_cast<int*>(red + 8);
-  unsigned char* growb = reinterpret_cast<unsigned char*>(red + 16);
+  int* gseg = reinterpret_cast<int*>(red + 16);
+  unsigned char* growb = reinterpret_cast<unsigned char*>(red + 24);
   static_assert(TC_M <= 16 * sizeof(double) && LGRP_MAX + 1 <= 8 * sizeof(double) / sizeof(int),
-                "the group tables fit in red[8..31]");
+                "the group tables fit in red[16..39]");
   if (threadIdx.x == 0) {
     bad = 0;
     gseg[0] = 0;
@@ -530,24 +536,24 @@ __global__ void __launch_bounds__(NT) leaf_kernel_tc(const Desc* __restrict__ D,
   }
   __syncthreads();
   if (EMU)
-    for (int t = threadIdx.x; t < nF; t += NT) growb[t] = (unsigned char)seg_block(gseg, G, t);
+    for (int t = threadIdx.x; t < nF; t += NTH) growb[t] = (unsigned char)seg_block(gseg, G, t);
   Engine<EMU> eng;
   eng.init(dsm, mbar, &tmem_slot, &fail, rexp, cexp);
-  for (int t = threadIdx.x; t < nF; t += NT) {
+  for (int t = threadIdx.x; t < nF; t += NTH) {
     sx[t] = lf.xs[o0 + t];
     sy[t] = lf.ys[o0 + t];
     sv[t] = lf.yv[o0 + t];
   }
   if (EMU)
-    for (int t = threadIdx.x; t < EM_GMAX * TC_M; t += NT) hsc[t] = -2000;
+    for (int t = threadIdx.x; t < EM_GMAX * TC_M; t += NTH) hsc[t] = -2000;
   double* Hrow = lf.H + o0 * Mr;
-  TcAcc acc;
+  typename Engine<EMU>::Acc acc;
   bool ok = true;
   const int row = acc.row(), c0 = acc.col0();
   if (EMU && chain_done) {
     const int ng = (Mr + EM_KG - 1) / EM_KG;
     __syncthreads();                             // after the reset of hsc above
-    for (int t = threadIdx.x; t < nF * ng; t += NT) {
+    for (int t = threadIdx.x; t < nF * ng; t += NTH) {
       const int i = t / ng, g = t - i * ng;
       hsc[g * TC_M + i] = lf.hrow[(o0 + i) * ng + g];
     }
@@ -556,14 +562,14 @@ __global__ void __launch_bounds__(NT) leaf_kernel_tc(const Desc* __restrict__ D,
   for (int l = 0; l < M && ok && !(EMU && chain_done); ++l) {
     const long a = ancestor(st, M, F, l);
     __syncthreads();
-    load_knots(sh, l, st.mort[l][a], ax, ay);
+    load_knots<NTH>(sh, l, st.mort[l][a], ax, ay);
     const double* Vanc = st.V[l] + a * (long)r * (l * r);
     if (EMU)
-      for (int t = threadIdx.x; t < TC_M; t += NT) xsc[t] = -2000;
+      for (int t = threadIdx.x; t < TC_M; t += NTH) xsc[t] = -2000;
     __syncthreads();
     // C0(S_F, Q_l) into block l, spread over every warp; the product below
     // reads only blocks < l
-    for (int t = threadIdx.x; t < nF * r; t += NT) {
+    for (int t = threadIdx.x; t < nF * r; t += NTH) {
       const int fi = t / r, qj = t - fi * r;
       const double v = cov0(cv, sx[fi], sy[fi], ax[qj], ay[qj]);
       Hrow[(long)fi * Mr + l * r + qj] = v;
@@ -578,7 +584,7 @@ __global__ void __launch_bounds__(NT) leaf_kernel_tc(const Desc* __restrict__ D,
       if (row < nF) {
         int e = -2000;
         #pragma unroll
-        for (int c = 0; c < 32; ++c) {
+        for (int c = 0; c < NC; ++c) {
           const int col = c0 + c;
           if (col < r) {
             const double v = Hrow[(long)row * Mr + l * r + col] - acc.v[c];
@@ -595,10 +601,10 @@ __global__ void __launch_bounds__(NT) leaf_kernel_tc(const Desc* __restrict__ D,
                  EMU ? st.liexp[l] + a * r : nullptr, 0);
     if (!ok) break;
     if (row < nF) {
-      int e0 = -2000, e1 = -2000;       // a thread's 32 columns touch at most two groups
+      int e0 = -2000, e1 = -2000;       // a thread's columns touch at most two groups
       const int gbase = (l * r + c0) / 128;
       #pragma unroll
-      for (int c = 0; c < 32; ++c) {
+      for (int c = 0; c < NC; ++c) {
         const int col = c0 + c;
         if (col < r) {
           Hrow[(long)row * Mr + l * r + col] = acc.v[c];
@@ -621,12 +627,12 @@ __global__ void __launch_bounds__(NT) leaf_kernel_tc(const Desc* __restrict__ D,
   static_assert(TC_M <= 2 * MAX_R_DEV, "the leaf's variance factors reuse ax and ay");
   double* lgq = ax;                              // the points' variance factors (ax, ay: 2 MAX_R_DEV >= nF doubles)
   if (fast && cv.nonstat) {
-    for (int t = threadIdx.x; t < nF; t += NT) lgq[t] = c0_vfac(cv, sx[t]);
+    for (int t = threadIdx.x; t < nF; t += NTH) lgq[t] = c0_vfac(cv, sx[t]);
     __syncthreads();
   }
   int tri_all = 0;                               // lower triangles of the group's diagonal blocks
   for (int k = 0; k < G; ++k) tri_all += (gseg[k + 1] - gseg[k]) * (gseg[k + 1] - gseg[k] + 1) / 2;
-  for (int t = threadIdx.x; t < tri_all; t += NT) {
+  for (int t = threadIdx.x; t < tri_all; t += NTH) {
     int b = 0, u = t;
     for (int c = gseg[1] * (gseg[1] + 1) / 2; u >= c; c = (gseg[b + 1] - gseg[b]) * (gseg[b + 1] - gseg[b] + 1) / 2) {
       u -= c;
@@ -655,7 +661,7 @@ __global__ void __launch_bounds__(NT) leaf_kernel_tc(const Desc* __restrict__ D,
     if (!ok) break;
     if (row < nF)
       #pragma unroll
-      for (int c = 0; c < 32; ++c) {
+      for (int c = 0; c < NC; ++c) {
         const int oj = ct * TC_N + c0 + c;
         if (c0 + c < ncol && oj <= row && (G == 1 || oj >= gseg[growb[row]])) S[row * lds + oj] -= acc.v[c];
       }
@@ -665,7 +671,7 @@ __global__ void __launch_bounds__(NT) leaf_kernel_tc(const Desc* __restrict__ D,
   auto store_blocks = [&](double* dst) {
     int tot = 0;
     for (int k = 0; k < G; ++k) tot += (gseg[k + 1] - gseg[k]) * (gseg[k + 1] - gseg[k]);
-    for (int t = threadIdx.x; t < tot; t += NT) {
+    for (int t = threadIdx.x; t < tot; t += NTH) {
       int b = 0, u = t;
       for (int c = gseg[1] * gseg[1]; u >= c; c = (gseg[b + 1] - gseg[b]) * (gseg[b + 1] - gseg[b])) {
         u -= c;
@@ -684,29 +690,29 @@ __global__ void __launch_bounds__(NT) leaf_kernel_tc(const Desc* __restrict__ D,
   };
   if (ok) {
     if (G == 1) {
-      chol_smem(S, nF, lds, &bad);
-      for (int t = threadIdx.x; t < nF; t += NT) ld += log(S[t * lds + t]);
-      ld = 2.0 * block_sum(ld, red);
+      chol_smem<NTH>(S, nF, lds, &bad);
+      for (int t = threadIdx.x; t < nF; t += NTH) ld += log(S[t * lds + t]);
+      ld = 2.0 * block_sum<NTH>(ld, red);
     } else {
-      chol_seg(S, lds, gseg, G, &bad, red);
-      for (int t = threadIdx.x; t < nF; t += NT) tmp[t] = log(S[t * lds + t]);
+      chol_seg<false, NTH>(S, lds, gseg, G, &bad, red);
+      for (int t = threadIdx.x; t < nF; t += NTH) tmp[t] = log(S[t * lds + t]);
       __syncthreads();
       ld = 2.0 * leaf_sum();
     }
     if (lf.LSf) {
       if (G == 1) {
         double* Lf = lf.LSf + lf.sq_off[Fm];
-        for (int t = threadIdx.x; t < nF * nF; t += NT) Lf[t] = S[(t / nF) * lds + (t % nF)];
+        for (int t = threadIdx.x; t < nF * nF; t += NTH) Lf[t] = S[(t / nF) * lds + (t % nF)];
       } else {
         store_blocks(lf.LSf);
       }
     }
     if (lf.VF)
-      for (long t = threadIdx.x; t < (long)nF * Mr; t += NT) lf.VF[o0 * Mr + t] = Hrow[t];
-    if (G == 1) trinv_smem(S, nF, lds, tmp);
-    else trinv_seg(S, lds, gseg, G, tmp, red);
+      for (long t = threadIdx.x; t < (long)nF * Mr; t += NTH) lf.VF[o0 * Mr + t] = Hrow[t];
+    if (G == 1) trinv_smem<NTH>(S, nF, lds, tmp);
+    else trinv_seg<false, NTH>(S, lds, gseg, G, tmp, red);
     if (EMU) {   // row scales of L_Sigma^{-1} (lower triangular) for the solve below
-      for (int t = threadIdx.x; t < nF; t += NT) {
+      for (int t = threadIdx.x; t < nF; t += NTH) {
         int e = -2000;
         for (int q = G == 1 ? 0 : gseg[growb[t]]; q <= t; ++q) e = max(e, xexp_of(S[t * lds + q]));
         ssc[t] = e;
@@ -714,11 +720,11 @@ __global__ void __launch_bounds__(NT) leaf_kernel_tc(const Desc* __restrict__ D,
     }
     if (G == 1) {
       double* LS = lf.LS + lf.sq_off[Fm];
-      for (int t = threadIdx.x; t < nF * nF; t += NT) LS[t] = S[(t / nF) * lds + (t % nF)];
+      for (int t = threadIdx.x; t < nF * nF; t += NTH) LS[t] = S[(t / nF) * lds + (t % nF)];
     } else {
       store_blocks(lf.LS);
     }
-    for (int t = threadIdx.x; t < nF; t += NT) {
+    for (int t = threadIdx.x; t < nF; t += NTH) {
       double s = 0.0;
       for (int k = G == 1 ? 0 : gseg[growb[t]]; k <= t; ++k) s = fma(S[t * lds + k], sv[k], s);
       lf.z[o0 + t] = s;
@@ -726,7 +732,7 @@ __global__ void __launch_bounds__(NT) leaf_kernel_tc(const Desc* __restrict__ D,
       else tmp[t] = s * s;
     }
     if (G == 1) {
-      zz = block_sum(zz, red);
+      zz = block_sum<NTH>(zz, red);
     } else {
       __syncthreads();
       zz = leaf_sum();
@@ -734,9 +740,9 @@ __global__ void __launch_bounds__(NT) leaf_kernel_tc(const Desc* __restrict__ D,
     // H^l = L_Sigma^{-1} V^l_F (whole block read before it is overwritten)
     int32_t* hcol = EMU ? lf.hcol + F * (long)Mr : nullptr;   // column scales of H_F for the Gram kernel
     if (EMU) {
-      for (int t = threadIdx.x; t < G * Mr; t += NT) hcol[t] = -2000;   // (the group's leaves are consecutive)
+      for (int t = threadIdx.x; t < G * Mr; t += NTH) hcol[t] = -2000;   // (the group's leaves are consecutive)
       // hsc (the V_F row scales) is read no more: it collects the row scales of H_F
-      for (int t = threadIdx.x; t < EM_GMAX * TC_M; t += NT) hsc[t] = -2000;
+      for (int t = threadIdx.x; t < EM_GMAX * TC_M; t += NTH) hsc[t] = -2000;
     }
     for (int cb = 0; cb < Mr && ok; cb += TC_N) {   // 64 columns of H a product (two levels at r = 32)
       const int nbc = min(TC_N, Mr - cb);
@@ -744,10 +750,10 @@ __global__ void __launch_bounds__(NT) leaf_kernel_tc(const Desc* __restrict__ D,
       ok = eng.mma(acc, S, lds, 1, nF, Hrow + cb, 1, Mr, nbc, nF, EMU ? ssc : nullptr, 0);
       if (!ok) break;
       if (row < nF) {
-        int e0 = -2000, e1 = -2000;       // a thread's 32 columns touch at most two groups
+        int e0 = -2000, e1 = -2000;       // a thread's columns touch at most two groups
         const int gbase = (cb + c0) / 128;
         #pragma unroll
-        for (int c = 0; c < 32; ++c) {
+        for (int c = 0; c < NC; ++c) {
           const int col = c0 + c;
           if (col < nbc) {
             Hrow[(long)row * Mr + cb + col] = acc.v[c];
@@ -764,7 +770,7 @@ __global__ void __launch_bounds__(NT) leaf_kernel_tc(const Desc* __restrict__ D,
       if (EMU && G == 1 && ((threadIdx.x >> 5) & 3) * 32 < nF) {   // warp-uniform: the warp holds a kept row
         const int lane = threadIdx.x & 31;
         #pragma unroll
-        for (int c = 0; c < 32; ++c) {
+        for (int c = 0; c < NC; ++c) {
           const int e = __reduce_max_sync(0xffffffffu, row < nF ? xexp_of(acc.v[c]) : -2000);
           if (lane == c && c0 + c < nbc && e > -2000) atomicMax(hcol + cb + c0 + c, e);
         }
@@ -773,7 +779,7 @@ __global__ void __launch_bounds__(NT) leaf_kernel_tc(const Desc* __restrict__ D,
         const int lk = row < nF ? (int)growb[row] : -1;
         const unsigned grp = __match_any_sync(0xffffffffu, lk);
         #pragma unroll
-        for (int c = 0; c < 32; ++c) {
+        for (int c = 0; c < NC; ++c) {
           const int e = __reduce_max_sync(grp, row < nF ? xexp_of(acc.v[c]) : -2000);
           if (lk >= 0 && lane == __ffs(grp) - 1 && c0 + c < nbc && e > -2000)
             atomicMax(hcol + (long)lk * Mr + cb + c0 + c, e);
@@ -783,7 +789,7 @@ __global__ void __launch_bounds__(NT) leaf_kernel_tc(const Desc* __restrict__ D,
     }
     if (EMU && lf.hrow && ok) {   // row scales of H_F per 128-column group (the gradient's Hbar operand)
       const int ng = (Mr + EM_KG - 1) / EM_KG;
-      for (int t = threadIdx.x; t < nF * ng; t += NT) {
+      for (int t = threadIdx.x; t < nF * ng; t += NTH) {
         const int i = t / ng, g = t - i * ng;
         lf.hrow[(o0 + i) * ng + g] = hsc[g * TC_M + i];
       }
@@ -837,13 +843,14 @@ __host__ __device__ inline int em_cblocks(int r) { return r <= 16 ? 4 : (r <= 32
 
 // One column block per tile (r > 32).  (A separate kernel: the same body
 // compiled as a branch of the several-block kernel below ran 10 % slower.)
-__global__ void __launch_bounds__(NT) leaf_syrk_kernel_em1(const Desc* __restrict__ D, const int2* __restrict__ work,
+__global__ void __launch_bounds__(EM_NT) leaf_syrk_kernel_em1(const Desc* __restrict__ D, const int2* __restrict__ work,
                                                           int nt, int* status) {
+  constexpr int NTH = EM_NT, NC = EmAcc::NC;
   extern __shared__ __align__(1024) unsigned char dsm[];
-  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ __align__(8) uint64_t mbar[EM_MBARS];
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
-  __shared__ int rexp[EM_REXP], cexp[EM_CEXP];
+  __shared__ __align__(16) int rexp[EM_REXP], cexp[EM_CEXP];
   int tile;
   const Item it = work_item_tiled(work, nt, tile);
   const Desc& ds = D[it.d];
@@ -864,7 +871,7 @@ __global__ void __launch_bounds__(NT) leaf_syrk_kernel_em1(const Desc* __restric
   // scales per 128-row group of the parent's rows: the largest column scale of
   // the leaves whose rows meet the group (an upper bound of the group's maximum)
   const int ng = (K + EM_KG - 1) / EM_KG;
-  for (int t = threadIdx.x; t < ng * (TC_M + TC_N); t += NT) {
+  for (int t = threadIdx.x; t < ng * (TC_M + TC_N); t += NTH) {
     const bool isA = t < ng * TC_M;
     const int u = isA ? t : t - ng * TC_M;
     const int g = isA ? u / TC_M : u / TC_N, i = isA ? u % TC_M : u % TC_N;
@@ -882,7 +889,7 @@ __global__ void __launch_bounds__(NT) leaf_syrk_kernel_em1(const Desc* __restric
     (isA ? rexp : cexp)[u] = e;
   }
   __syncthreads();
-  TcAcc acc;
+  EmAcc acc;
   acc.zero();
   const bool ok = eng.mma(acc, Hb + k0 * r, 1, Mr, nk * r, Hb + l * r, 1, Mr, r, K, rexp, TC_M, cexp, TC_N);
   const int m = M - 1, T = (m + 1) * (m + 2) / 2;
@@ -891,13 +898,13 @@ __global__ void __launch_bounds__(NT) leaf_syrk_kernel_em1(const Desc* __restric
     const int k = k0 + row / r, ri = row % r;
     double* out = st.Acc[m] + (p * T + tri_index(k, l)) * (long)r * r + (long)ri * r;
 #pragma unroll
-    for (int c = 0; c < 32; ++c)
+    for (int c = 0; c < NC; ++c)
       if (c0 + c < r) out[c0 + c] = acc.v[c];
   }
   eng.release();
   if (k0 == l) {
     double* om = st.Om[m] + (p * (m + 1) + l) * (long)r;
-    for (int a = threadIdx.x; a < r; a += NT) {
+    for (int a = threadIdx.x; a < r; a += NTH) {
       double s = 0.0;
       for (long o = 0; o < K; ++o) s = fma(Hb[o * Mr + l * r + a], lf.z[row0 + o], s);
       om[a] = s;
@@ -908,13 +915,14 @@ __global__ void __launch_bounds__(NT) leaf_syrk_kernel_em1(const Desc* __restric
 
 // Several column blocks per tile (r <= 32).
 template <bool MULTI>
-__global__ void __launch_bounds__(NT) leaf_syrk_kernel_em(const Desc* __restrict__ D, const int2* __restrict__ work,
+__global__ void __launch_bounds__(EM_NT) leaf_syrk_kernel_em(const Desc* __restrict__ D, const int2* __restrict__ work,
                                                           int nt, int* status) {
+  constexpr int NTH = EM_NT, NC = EmAcc::NC;
   extern __shared__ __align__(1024) unsigned char dsm[];
-  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ __align__(8) uint64_t mbar[EM_MBARS];
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
-  __shared__ int rexp[EM_REXP], cexp[EM_CEXP];
+  __shared__ __align__(16) int rexp[EM_REXP], cexp[EM_CEXP];
   int tile;
   const Item it = work_item_tiled(work, nt, tile);
   const Desc& ds = D[it.d];
@@ -936,7 +944,7 @@ __global__ void __launch_bounds__(NT) leaf_syrk_kernel_em(const Desc* __restrict
   // scales per 128-row group of the parent's rows: the largest column scale of
   // the leaves whose rows meet the group (an upper bound of the group's maximum)
   const int ng = (K + EM_KG - 1) / EM_KG;
-  for (int t = threadIdx.x; t < ng * (TC_M + TC_N); t += NT) {
+  for (int t = threadIdx.x; t < ng * (TC_M + TC_N); t += NTH) {
     const bool isA = t < ng * TC_M;
     const int u = isA ? t : t - ng * TC_M;
     const int g = isA ? u / TC_M : u / TC_N, i = isA ? u % TC_M : u % TC_N;
@@ -954,7 +962,7 @@ __global__ void __launch_bounds__(NT) leaf_syrk_kernel_em(const Desc* __restrict
     (isA ? rexp : cexp)[u] = e;
   }
   __syncthreads();
-  TcAcc acc;
+  EmAcc acc;
   acc.zero();
   const bool ok = eng.mma(acc, Hb + k0 * r, 1, Mr, nk * r, Hb + l * r, 1, Mr, nl * r, K, rexp, TC_M, cexp, TC_N);
   const int m = M - 1, T = (m + 1) * (m + 2) / 2;
@@ -964,11 +972,11 @@ __global__ void __launch_bounds__(NT) leaf_syrk_kernel_em(const Desc* __restrict
     if (!MULTI) {                                     // (r > 32: one column block)
       double* out = st.Acc[m] + (p * T + tri_index(k, l)) * (long)r * r + (long)ri * r;
 #pragma unroll
-      for (int c = 0; c < 32; ++c)
+      for (int c = 0; c < NC; ++c)
         if (c0 + c < r) out[c0 + c] = acc.v[c];
     } else {
 #pragma unroll
-      for (int c = 0; c < 32; ++c) {
+      for (int c = 0; c < NC; ++c) {
         const int col = c0 + c, lb = l + col / r;     // column block of this column
         if (col < nl * r && k >= lb)
           st.Acc[m][(p * T + tri_index(k, lb)) * (long)r * r + (long)ri * r + col % r] = acc.v[c];
@@ -979,7 +987,7 @@ __global__ void __launch_bounds__(NT) leaf_syrk_kernel_em(const Desc* __restrict
   if (k0 == l)
     for (int lb = l; lb < l + nl; ++lb) {
       double* om = st.Om[m] + (p * (m + 1) + lb) * (long)r;
-      for (int a = threadIdx.x; a < r; a += NT) {
+      for (int a = threadIdx.x; a < r; a += NTH) {
         double s = 0.0;
         for (long o = 0; o < K; ++o) s = fma(Hb[o * Mr + lb * r + a], lf.z[row0 + o], s);
         om[a] = s;
@@ -989,13 +997,14 @@ __global__ void __launch_bounds__(NT) leaf_syrk_kernel_em(const Desc* __restrict
 }
 
 template <bool MULTI>
-__global__ void __launch_bounds__(NT) aggregate_kernel_em(int m, const Desc* __restrict__ D,
+__global__ void __launch_bounds__(EM_NT) aggregate_kernel_em(int m, const Desc* __restrict__ D,
                                                           const int2* __restrict__ work, int nt, int* status) {
+  constexpr int NTH = EM_NT, NC = EmAcc::NC;
   extern __shared__ __align__(1024) unsigned char dsm[];
-  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ __align__(8) uint64_t mbar[EM_MBARS];
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
-  __shared__ int rexp[EM_REXP], cexp[EM_CEXP];
+  __shared__ __align__(16) int rexp[EM_REXP], cexp[EM_CEXP];
   int tile;
   const Item it = work_item_tiled(work, nt, tile);
   const Desc& ds = D[it.d];
@@ -1015,7 +1024,7 @@ __global__ void __launch_bounds__(NT) aggregate_kernel_em(int m, const Desc* __r
   // scales per 128-row group of the stacked children (r rows each): the
   // largest column scale of the children whose rows meet the group
   const int K = (int)(cc * r), ng = (K + EM_KG - 1) / EM_KG;
-  for (int t = threadIdx.x; t < ng * (TC_M + TC_N); t += NT) {
+  for (int t = threadIdx.x; t < ng * (TC_M + TC_N); t += NTH) {
     const bool isA = t < ng * TC_M;
     const int u = isA ? t : t - ng * TC_M;
     const int g = isA ? u / TC_M : u / TC_N, i = isA ? u % TC_M : u % TC_N;
@@ -1029,7 +1038,7 @@ __global__ void __launch_bounds__(NT) aggregate_kernel_em(int m, const Desc* __r
     (isA ? rexp : cexp)[u] = e;
   }
   __syncthreads();
-  TcAcc acc;
+  EmAcc acc;
   acc.zero();
   const bool ok = eng.mma(acc, Gb + k0 * r, 1, mr, nk * r, Gb + l * r, 1, mr, nl * r, K, rexp, TC_M, cexp, TC_N);
   const int row = acc.row(), c0 = acc.col0();
@@ -1039,7 +1048,7 @@ __global__ void __launch_bounds__(NT) aggregate_kernel_em(int m, const Desc* __r
       const int t = tri_index(k, l);
       double* out = st.Acc[m - 1] + (p * Tp + t) * (long)r * r + (long)ri * r;
 #pragma unroll
-      for (int c = 0; c < 32; ++c) {
+      for (int c = 0; c < NC; ++c) {
         const int col = c0 + c;
         if (col < r) {
           double s = -acc.v[c];
@@ -1049,7 +1058,7 @@ __global__ void __launch_bounds__(NT) aggregate_kernel_em(int m, const Desc* __r
       }
     } else {
 #pragma unroll
-      for (int c = 0; c < 32; ++c) {
+      for (int c = 0; c < NC; ++c) {
         const int col = c0 + c, lb = l + col / r, cj = col % r;   // column block and column
         if (col < nl * r && k >= lb) {
           const int t = tri_index(k, lb);
@@ -1064,7 +1073,7 @@ __global__ void __launch_bounds__(NT) aggregate_kernel_em(int m, const Desc* __r
   if (k0 == l)
     for (int lb = l; lb < l + nl; ++lb) {
       double* om = st.Om[m - 1] + (p * m + lb) * (long)r;
-      for (int a = threadIdx.x; a < r; a += NT) {
+      for (int a = threadIdx.x; a < r; a += NTH) {
         double s = 0.0;
         for (long ci = cf; ci < cf + cc; ++ci) {
           s += st.Om[m][(ci * (m + 1) + lb) * (long)r + a];
@@ -1088,7 +1097,7 @@ static size_t prior_tc_smem(int rcap) {     // knots (2 rcap), ancestor knots, s
 template <bool EMU>
 static size_t leaf_tc_smem(int nlmax) {
   const size_t b =
-      Engine<EMU>::STAGE + sizeof(double) * (4 * (size_t)nlmax + 2 * MAX_R_DEV + 32 + (size_t)nlmax * (nlmax + 1));
+      Engine<EMU>::STAGE + sizeof(double) * (4 * (size_t)nlmax + 2 * MAX_R_DEV + 40 + (size_t)nlmax * (nlmax + 1));
   return EMU ? std::max(b, EM_SOLO_SMEM) : b;
 }
 // Dynamic plus (an upper bound of) static shared memory of the leaf kernel.
@@ -1107,7 +1116,7 @@ cudaError_t launch_prior_tc(int m, const Desc* d_desc, const int2* work, int nbl
     const size_t sm = prior_tc_smem<true>(rcap);
     if ((e = cudaFuncSetAttribute(prior_level_kernel_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))
       return e;
-    prior_level_kernel_tc<true><<<nblocks, NT, sm, s>>>(m, d_desc, work, status, gcnt, rcap);
+    prior_level_kernel_tc<true><<<nblocks, EM_NT, sm, s>>>(m, d_desc, work, status, gcnt, rcap);
   } else {
     const size_t sm = prior_tc_smem<false>(rcap);
     if ((e = cudaFuncSetAttribute(prior_level_kernel_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))
@@ -1128,8 +1137,8 @@ cudaError_t launch_leaf_tc(const Desc* d_desc, const int2* work, int nblocks, in
       if ((e = cudaFuncSetAttribute(gpar ? chain_forward_kernel_em<true> : chain_forward_kernel_em<false>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, EM_SOLO_SMEM)))
         return e;
-      if (gpar) chain_forward_kernel_em<true><<<n_par, NT, EM_SOLO_SMEM, s>>>(d_desc, w_par, status, gpar);
-      else chain_forward_kernel_em<false><<<n_par, NT, EM_SOLO_SMEM, s>>>(d_desc, w_par, status, nullptr);
+      if (gpar) chain_forward_kernel_em<true><<<n_par, EM_NT, EM_SOLO_SMEM, s>>>(d_desc, w_par, status, gpar);
+      else chain_forward_kernel_em<false><<<n_par, EM_NT, EM_SOLO_SMEM, s>>>(d_desc, w_par, status, nullptr);
       if ((e = cudaGetLastError())) return e;
       if (tm) {   // the chain and the leaf kernel are timed as two records
         tm->stop(s);
@@ -1139,7 +1148,7 @@ cudaError_t launch_leaf_tc(const Desc* d_desc, const int2* work, int nblocks, in
     if (gcnt && !chain_done) return cudaErrorInvalidValue;   // (groups need the per-parent chain kernel)
     const size_t sm = leaf_tc_smem<true>(std::max(nlmax, chain_done ? lrows : 0));
     if ((e = cudaFuncSetAttribute(leaf_kernel_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
-    leaf_kernel_tc<true><<<nblocks, NT, sm, s>>>(d_desc, work, status, chain_done, chain_done ? gcnt : nullptr);
+    leaf_kernel_tc<true><<<nblocks, EM_NT, sm, s>>>(d_desc, work, status, chain_done, chain_done ? gcnt : nullptr);
   } else {
     const size_t sm = leaf_tc_smem<false>(nlmax);
     if ((e = cudaFuncSetAttribute(leaf_kernel_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
@@ -1156,8 +1165,8 @@ cudaError_t launch_leaf_syrk_em(const Desc* d_desc, const int2* work, int nblock
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, EM_SOLO_SMEM)))
     return e;
   const int nt = em_tiles(maxM, em_stack(r), em_cblocks(r));
-  if (multi) leaf_syrk_kernel_em<true><<<nblocks * nt, NT, EM_SOLO_SMEM, s>>>(d_desc, work, nt, status);
-  else leaf_syrk_kernel_em1<<<nblocks * nt, NT, EM_SOLO_SMEM, s>>>(d_desc, work, nt, status);
+  if (multi) leaf_syrk_kernel_em<true><<<nblocks * nt, EM_NT, EM_SOLO_SMEM, s>>>(d_desc, work, nt, status);
+  else leaf_syrk_kernel_em1<<<nblocks * nt, EM_NT, EM_SOLO_SMEM, s>>>(d_desc, work, nt, status);
   return cudaGetLastError();
 }
 
@@ -1217,12 +1226,13 @@ __global__ void __launch_bounds__(NT) s_full_kernel(int L, const Desc* __restric
 }
 
 // One CTA per (level-(M-1) region p, column block l), l fastest: column block l of Hbar for all rows under p.
-__global__ void __launch_bounds__(NT) hbar_kernel_em(const Desc* __restrict__ D, GradState gs, int* status) {
+__global__ void __launch_bounds__(EM_NT) hbar_kernel_em(const Desc* __restrict__ D, GradState gs, int* status) {
+  constexpr int NTH = EM_NT, NC = EmAcc::NC;
   extern __shared__ __align__(1024) unsigned char dsm[];
-  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ __align__(8) uint64_t mbar[EM_MBARS];
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
-  __shared__ int rexp[EM_REXP], cexp[EM_CEXP];
+  __shared__ __align__(16) int rexp[EM_REXP], cexp[EM_CEXP];
   __shared__ int hsc[EM_GMAX * TC_M];            // row scales of the current 128 rows of H per group
   __shared__ double wb[MAX_R_DEV];               // omegabar of block l
   const Desc& ds = D[0];
@@ -1235,12 +1245,12 @@ __global__ void __launch_bounds__(NT) hbar_kernel_em(const Desc* __restrict__ D,
   const long pm = st.mort[M - 1][p];
   const long row0 = lf.off[pm << leaf_bits(ds.sh)], row1 = lf.off[(pm + 1) << leaf_bits(ds.sh)];
   const long al = ancestor(st, M - 1, p, l);
-  for (int t = threadIdx.x; t < r; t += NT) wb[t] = gs.Obar[l][al * r + t];
+  for (int t = threadIdx.x; t < r; t += NTH) wb[t] = gs.Obar[l][al * r + t];
   Engine<true> eng;
   eng.init(dsm, mbar, &tmem_slot, &fail, rexp, cexp);
   const double* Sl = gs.SF + p * (long)Mr * Mr + (long)l * r * Mr;
   const int* Se = gs.SFexp + p * (long)ng * Mr + l * r;
-  TcAcc acc;
+  EmAcc acc;
   bool ok = true;
   const int row = acc.row(), c0 = acc.col0();
   for (long t0 = row0; t0 < row1 && ok; t0 += TC_M) {
@@ -1248,12 +1258,12 @@ __global__ void __launch_bounds__(NT) hbar_kernel_em(const Desc* __restrict__ D,
     const double* Ht = lf.H + t0 * Mr;
     __syncthreads();                             // the previous tile's scales are no longer read
     if (lf.hrow) {                               // exported by the leaf kernel
-      for (int t = threadIdx.x; t < TC_M * ng; t += NT) {
+      for (int t = threadIdx.x; t < TC_M * ng; t += NTH) {
         const int i = t / ng, g = t - i * ng;
         hsc[g * TC_M + i] = i < na ? lf.hrow[(t0 + i) * ng + g] : -2000;
       }
     } else {
-      for (int i = warp; i < TC_M; i += NT / 32)
+      for (int i = warp; i < TC_M; i += NTH / 32)
         for (int g = 0; g < ng; ++g) {
           int e = -2000;
           if (i < na)
@@ -1269,7 +1279,7 @@ __global__ void __launch_bounds__(NT) hbar_kernel_em(const Desc* __restrict__ D,
       const double zr = lf.z[t0 + row];
       double* out = gs.HB + (t0 + row) * Mr + l * r;
 #pragma unroll
-      for (int c = 0; c < 32; ++c)
+      for (int c = 0; c < NC; ++c)
         if (c0 + c < r) out[c0 + c] = 2.0 * acc.v[c] + zr * wb[c0 + c];
     }
   }
@@ -1282,12 +1292,13 @@ __global__ void __launch_bounds__(NT) hbar_kernel_em(const Desc* __restrict__ D,
 // (the FP64 leaf_partial_kernel's tiles).  Per column block k, the diagonal
 // tile (operand Vbar) runs alone and the tiles l > k (operand Xbar, adjacent
 // columns) are stacked em_stack(r) high.
-__global__ void __launch_bounds__(NT) leaf_partial_kernel_em(const Desc* __restrict__ D, GradState gs, int* status) {
+__global__ void __launch_bounds__(EM_NT) leaf_partial_kernel_em(const Desc* __restrict__ D, GradState gs, int* status) {
+  constexpr int NTH = EM_NT, NC = EmAcc::NC;
   extern __shared__ __align__(1024) unsigned char dsm[];
-  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ __align__(8) uint64_t mbar[EM_MBARS];
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
-  __shared__ int rexp[EM_REXP], cexp[EM_CEXP];
+  __shared__ __align__(16) int rexp[EM_REXP], cexp[EM_CEXP];
   const Desc& ds = D[0];
   const int M = ds.sh.M, r = ds.sh.r, Mr = M * r, T = M * (M + 1) / 2;
   const LeafState& lf = ds.lf;
@@ -1303,7 +1314,7 @@ __global__ void __launch_bounds__(NT) leaf_partial_kernel_em(const Desc* __restr
   const double* B = lf.VF + row0 * Mr + k * r;
   Engine<true> eng;
   eng.init(dsm, mbar, &tmem_slot, &fail, rexp, cexp);
-  TcAcc acc;
+  EmAcc acc;
   // operand scales per 128-row group from the chain kernels, when they exported them
   const bool tab = gs.VFexp != nullptr;
   const long tb = p * 4 * (long)Mr;
@@ -1316,7 +1327,7 @@ __global__ void __launch_bounds__(NT) leaf_partial_kernel_em(const Desc* __restr
     const double sg = diag ? 1.0 : -1.0;
     double* out = gs.PartLeaf + (p * T + tri_index(l, k)) * (long)r * r + (long)i * r;
 #pragma unroll
-    for (int c = 0; c < 32; ++c)
+    for (int c = 0; c < NC; ++c)
       if (c0 + c < r) out[c0 + c] = sg * acc.v[c];
   }
   eng.release();
@@ -1331,7 +1342,7 @@ cudaError_t launch_leaf_partial_em(const Desc& hd, const Desc* d_desc, const Gra
   cudaError_t e;
   if ((e = cudaFuncSetAttribute(leaf_partial_kernel_em, cudaFuncAttributeMaxDynamicSharedMemorySize, EM_SOLO_SMEM)))
     return e;
-  leaf_partial_kernel_em<<<np * partial_tiles(M, em_stack(r)), NT, EM_SOLO_SMEM, s>>>(d_desc, gs, status);
+  leaf_partial_kernel_em<<<np * partial_tiles(M, em_stack(r)), EM_NT, EM_SOLO_SMEM, s>>>(d_desc, gs, status);
   return cudaGetLastError();
 }
 
@@ -1343,13 +1354,14 @@ cudaError_t launch_leaf_partial_em(const Desc& hd, const Desc* d_desc, const Gra
 // row by row; the ancestors a_l (l < M) are shared by all children of one
 // level-(M-1) region, so one CTA takes the region's contiguous rows in tiles of
 // 128.  Its C0 terms go to gradient slot slot0 + p.
-__global__ void __launch_bounds__(NT) chain_adjoint_kernel_em(const Desc* __restrict__ D, GradState gs, long slot0,
+__global__ void __launch_bounds__(EM_NT) chain_adjoint_kernel_em(const Desc* __restrict__ D, GradState gs, long slot0,
                                                               int* status) {
+  constexpr int NTH = EM_NT, NC = EmAcc::NC;
   extern __shared__ __align__(1024) unsigned char dsm[];
-  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ __align__(8) uint64_t mbar[EM_MBARS];
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
-  __shared__ int rexp[EM_REXP], cexp[EM_CEXP];
+  __shared__ __align__(16) int rexp[EM_REXP], cexp[EM_CEXP];
   __shared__ double ax[MAX_R_DEV], ay[MAX_R_DEV], red[32];
   // row scales (one 64-column block = one group) of the tile's Vbar blocks and of the current Xbar block
   __shared__ int vbsc[MAXL * TC_M], xbsc[TC_M];
@@ -1364,7 +1376,7 @@ __global__ void __launch_bounds__(NT) chain_adjoint_kernel_em(const Desc* __rest
   const long row0 = lf.off[pm << leaf_bits(ds.sh)], row1 = lf.off[(pm + 1) << leaf_bits(ds.sh)];
   Engine<true> eng;
   eng.init(dsm, mbar, &tmem_slot, &fail, rexp, cexp);
-  TcAcc acc;
+  EmAcc acc;
   const int row = acc.row(), c0 = acc.col0();
   double g_s2 = 0.0, g_k = 0.0, g_nu = 0.0;
   bool ok = true;
@@ -1377,7 +1389,7 @@ __global__ void __launch_bounds__(NT) chain_adjoint_kernel_em(const Desc* __rest
     __syncthreads();                             // the previous tile's scales are no longer read
     {   // row scales of Vbar^{M-1} (as the leaf adjoint left it): one warp per row
       const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-      for (int i = warp; i < TC_M; i += NT / 32) {
+      for (int i = warp; i < TC_M; i += NTH / 32) {
         int e = -2000;
         if (i < na)
           for (int c = lane; c < r; c += 32) e = max(e, xexp_of(VB[(long)i * Mr + (M - 1) * r + c]));
@@ -1390,8 +1402,8 @@ __global__ void __launch_bounds__(NT) chain_adjoint_kernel_em(const Desc* __rest
       const double* Lia = st.Li[l] + a * (long)r * r;
       const double* Va = st.V[l] + a * (long)r * (l * r);
       __syncthreads();                           // the previous level's knots and Xbar scales are no longer read
-      load_knots(sh, l, st.mort[l][a], ax, ay);
-      for (int t = threadIdx.x; t < TC_M; t += NT) {
+      load_knots<NTH>(sh, l, st.mort[l][a], ax, ay);
+      for (int t = threadIdx.x; t < TC_M; t += NTH) {
         xbsc[t] = -2000;
         if (l > 0) vbsc[(l - 1) * TC_M + t] = -2000;   // block l - 1 takes its last update at this level
       }
@@ -1400,7 +1412,7 @@ __global__ void __launch_bounds__(NT) chain_adjoint_kernel_em(const Desc* __rest
                    tab ? st.licol[l] + a * r : nullptr, 0);
       if (ok && row < na) {
 #pragma unroll
-        for (int c = 0; c < 32; ++c) {
+        for (int c = 0; c < NC; ++c) {
           const int col = c0 + c;
           if (col < r) {
             const double xb = acc.v[c];
@@ -1420,7 +1432,7 @@ __global__ void __launch_bounds__(NT) chain_adjoint_kernel_em(const Desc* __rest
         }
         int e = -2000;   // row scale of Xbar^l (two threads per row)
 #pragma unroll
-        for (int c = 0; c < 32; ++c)
+        for (int c = 0; c < NC; ++c)
           if (c0 + c < r) e = max(e, xexp_of(acc.v[c]));
         atomicMax(xbsc + row, e);
       }
@@ -1432,7 +1444,7 @@ __global__ void __launch_bounds__(NT) chain_adjoint_kernel_em(const Desc* __rest
           double* out = VB + (long)row * Mr + k * r;
           int e = -2000;
 #pragma unroll
-          for (int c = 0; c < 32; ++c)
+          for (int c = 0; c < NC; ++c)
             if (c0 + c < r) {
               const double v = out[c0 + c] - acc.v[c];
               out[c0 + c] = v;
@@ -1445,7 +1457,7 @@ __global__ void __launch_bounds__(NT) chain_adjoint_kernel_em(const Desc* __rest
     if (ok && gs.VBexp) {   // column scales of the final Vbar_F and Xbar_F over the tile (leaf partials)
       __syncthreads();
       const long base = (p * 4 + (t0 - row0) / TC_M) * (long)Mr;
-      for (int c = threadIdx.x; c < 2 * Mr; c += NT) {
+      for (int c = threadIdx.x; c < 2 * Mr; c += NTH) {
         const double* X = c < Mr ? VB : XB;
         const int cc = c < Mr ? c : c - Mr;
         int e = -2000;
@@ -1455,9 +1467,9 @@ __global__ void __launch_bounds__(NT) chain_adjoint_kernel_em(const Desc* __rest
     }
   }
   eng.release();
-  g_s2 = block_sum(g_s2, red);
-  g_k = block_sum(g_k, red);
-  g_nu = block_sum(g_nu, red);
+  g_s2 = block_sum<NTH>(g_s2, red);
+  g_k = block_sum<NTH>(g_k, red);
+  g_nu = block_sum<NTH>(g_nu, red);
   if (threadIdx.x == 0) {
     gs.gpart[GP * (slot0 + p) + 0] = g_s2;
     gs.gpart[GP * (slot0 + p) + 1] = g_k;
@@ -1475,7 +1487,7 @@ cudaError_t launch_chain_adjoint_em(const Desc& hd, const Desc* d_desc, const Gr
   cudaError_t e;
   if ((e = cudaFuncSetAttribute(chain_adjoint_kernel_em, cudaFuncAttributeMaxDynamicSharedMemorySize, EM_SOLO_SMEM)))
     return e;
-  chain_adjoint_kernel_em<<<np, NT, EM_SOLO_SMEM, s>>>(d_desc, gs, slot0, status);
+  chain_adjoint_kernel_em<<<np, EM_NT, EM_SOLO_SMEM, s>>>(d_desc, gs, slot0, status);
   return cudaGetLastError();
 }
 
@@ -1498,7 +1510,7 @@ cudaError_t launch_hbar_em(const Desc& hd, const Desc* d_desc, const GradState& 
   cudaError_t e;
   if ((e = launch_s_full(M - 1, hd, d_desc, gs, s, np))) return e;
   if ((e = cudaFuncSetAttribute(hbar_kernel_em, cudaFuncAttributeMaxDynamicSharedMemorySize, EM_SOLO_SMEM))) return e;
-  hbar_kernel_em<<<np * M, NT, EM_SOLO_SMEM, s>>>(d_desc, gs, status);
+  hbar_kernel_em<<<np * M, EM_NT, EM_SOLO_SMEM, s>>>(d_desc, gs, status);
   *launches += 2;
   return cudaGetLastError();
 }
@@ -1507,12 +1519,13 @@ cudaError_t launch_hbar_em(const Desc& hd, const Desc* d_desc, const GradState& 
 //     Gbar^l = -2 sum_k G^k S^{k,l} - g omegabar^l',  l < m,
 // for all children of each level-(m-1) region P at once (they share P's chain
 // S and omegabar; their rows of G are contiguous), from St_P assembled first.
-__global__ void __launch_bounds__(NT) gbar_kernel_em(int m, const Desc* __restrict__ D, GradState gs, int* status) {
+__global__ void __launch_bounds__(EM_NT) gbar_kernel_em(int m, const Desc* __restrict__ D, GradState gs, int* status) {
+  constexpr int NTH = EM_NT, NC = EmAcc::NC;
   extern __shared__ __align__(1024) unsigned char dsm[];
-  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ __align__(8) uint64_t mbar[EM_MBARS];
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
-  __shared__ int rexp[EM_REXP], cexp[EM_CEXP];
+  __shared__ __align__(16) int rexp[EM_REXP], cexp[EM_CEXP];
   __shared__ int gsc[EM_GMAX * TC_M];            // row scales of the current 128 rows of G per group
   __shared__ double wb[MAX_R_DEV];
   const Desc& ds = D[0];
@@ -1523,19 +1536,19 @@ __global__ void __launch_bounds__(NT) gbar_kernel_em(int m, const Desc* __restri
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long row0 = (long)st.cfirst[m - 1][P] * r, row1 = row0 + (long)st.ccnt[m - 1][P] * r;
   const long al = ancestor(st, m - 1, P, l);
-  for (int t = threadIdx.x; t < r; t += NT) wb[t] = gs.Obar[l][al * r + t];
+  for (int t = threadIdx.x; t < r; t += NTH) wb[t] = gs.Obar[l][al * r + t];
   Engine<true> eng;
   eng.init(dsm, mbar, &tmem_slot, &fail, rexp, cexp);
   const double* Sl = gs.SF + P * (long)mr * mr + (long)l * r * mr;
   const int* Se = gs.SFexp + P * (long)ng * mr + l * r;
-  TcAcc acc;
+  EmAcc acc;
   bool ok = true;
   const int row = acc.row(), c0 = acc.col0();
   for (long t0 = row0; t0 < row1 && ok; t0 += TC_M) {
     const int na = (int)min((long)TC_M, row1 - t0);
     const double* Gt = st.G[m] + t0 * mr;
     __syncthreads();                             // the previous tile's scales are no longer read
-    for (int i = warp; i < TC_M; i += NT / 32)
+    for (int i = warp; i < TC_M; i += NTH / 32)
       for (int g = 0; g < ng; ++g) {
         int e = -2000;
         if (i < na)
@@ -1549,7 +1562,7 @@ __global__ void __launch_bounds__(NT) gbar_kernel_em(int m, const Desc* __restri
       const double gr = st.gv[m][t0 + row];
       double* out = gs.GB[m] + (t0 + row) * mr + l * r;
 #pragma unroll
-      for (int c = 0; c < 32; ++c)
+      for (int c = 0; c < NC; ++c)
         if (c0 + c < r) out[c0 + c] = -2.0 * acc.v[c] - gr * wb[c0 + c];
     }
   }
@@ -1564,7 +1577,7 @@ cudaError_t launch_gbar_em(int m, const Desc& hd, const Desc* d_desc, const Grad
   cudaError_t e;
   if ((e = launch_s_full(m - 1, hd, d_desc, gs, s, np))) return e;
   if ((e = cudaFuncSetAttribute(gbar_kernel_em, cudaFuncAttributeMaxDynamicSharedMemorySize, EM_SOLO_SMEM))) return e;
-  gbar_kernel_em<<<np * m, NT, EM_SOLO_SMEM, s>>>(m, d_desc, gs, status);
+  gbar_kernel_em<<<np * m, EM_NT, EM_SOLO_SMEM, s>>>(m, d_desc, gs, status);
   *launches += 2;
   return cudaGetLastError();
 }
@@ -1577,8 +1590,8 @@ cudaError_t launch_aggregate_em(int m, int r, const Desc* d_desc, const int2* wo
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, EM_SOLO_SMEM)))
     return e;
   const int nt = em_tiles(m, em_stack(r), em_cblocks(r));
-  if (multi) aggregate_kernel_em<true><<<nblocks * nt, NT, EM_SOLO_SMEM, s>>>(m, d_desc, work, nt, status);
-  else aggregate_kernel_em<false><<<nblocks * nt, NT, EM_SOLO_SMEM, s>>>(m, d_desc, work, nt, status);
+  if (multi) aggregate_kernel_em<true><<<nblocks * nt, EM_NT, EM_SOLO_SMEM, s>>>(m, d_desc, work, nt, status);
+  else aggregate_kernel_em<false><<<nblocks * nt, EM_NT, EM_SOLO_SMEM, s>>>(m, d_desc, work, nt, status);
   return cudaGetLastError();
 }
 

@@ -64,6 +64,7 @@ struct TcCtx {
 // Output ownership: thread (warp w, lane l) holds row 32 (w % 4) + l and the
 // 32 columns starting at 32 (w / 4) of the 128 x 64 tile.
 struct TcAcc {
+  static constexpr int NC = 32;
   double v[32];
   __device__ __forceinline__ void zero() {
 #pragma unroll
