@@ -12,19 +12,21 @@
 //    f16 (integers to 2048);
 //  * d_p d_q products are exact and the FP32 sums of every pair with the same
 //    weight t = p + q over a group stay at or below 128 (2 256 128 + 4 128^2)
-//    = 2^24, so the tensor-memory accumulation is exact too; the 21 pairs with
-//    t <= S + 1 go to 6 accumulators (one per t, up to 64 TMEM columns each);
-//  * every group is drained: the 6 accumulators of a column are combined in
+//    = 2^24, so the tensor-memory accumulation is exact too; the 26 pairs with
+//    t <= 8 go to 7 accumulators (one per t, up to 64 TMEM columns each);
+//  * every group is drained: the 7 accumulators of a column are combined in
 //    units of the leading weight (double-float, Fast2Sum for the two largest
 //    corrections), scaled by 2^(e_i + f_j - 16) (exact) and added to a
 //    double-float register accumulator, converted to FP64 once at the end.
 //
 // Signed digits carry 8 bits a slice where sign-and-magnitude slices of the
-// same magnitude (|a| < 128) carry 7: 6 slices and 21 products hold what took
-// 7 and 28, the operand error (at most 2^-49 of the group's largest element)
-// is rounded instead of truncated, and the dropped pairs (t = 8) have random
-// signs.  So a product matches FP64 to about 1e-14 relative to sum |a b| while
-// running on the tensor cores; the FP64 pipe only does the final conversion.
+// same magnitude (|a| < 128) carry 7: 6 slices and 26 products against 7 and 28,
+// with the operand error (at most 2^-49 of the group's largest element) rounded
+// instead of truncated.  The pairs of weight 8 matter: without them (21 products,
+// 2 % of an evaluation) the squares d_4^2 a Gram product drops are all positive,
+// and the gradient at n = 2^16 is off by 2e-11 to 3e-10 instead of 6e-13 to 3e-12.
+// So a product matches FP64 to about 1e-15 relative to sum |a b| while running on
+// the tensor cores; only rare sums touch the FP64 pipe.
 // Range: the running sums are FP32 pairs, so |results| < 2^127, and a group
 // whose scale product 2^(e_i + f_j) is below 2^-110 is dropped.
 //
@@ -42,6 +44,8 @@ namespace mra {
 
 constexpr int EM_NT = 512;                    // threads per CTA of the engine's kernels
 constexpr int EM_S = 6;                       // digits per operand
+constexpr int EM_T = EM_S + 2;                // digit pairs (p, q) with p + q <= EM_T are formed
+constexpr int EM_NA = EM_T - 1;               // accumulators, one per p + q
 constexpr int EM_KC = 16;                     // staged K chunk (f16 elements) = one MMA K-step
 constexpr int EM_KG = 128;                    // K group sharing one scale per row (drain period)
 constexpr int EM_GCH = EM_KG / EM_KC;         // chunks per group
@@ -64,8 +68,8 @@ enum : int { EM_FULL = 0, EM_FREE = 2, EM_DONE = 4, EM_READ = 5, EM_LAST = 6, EM
 // half of the SM's shared memory so that a second CTA is never resident (it
 // would only wait in tcgen05.alloc).
 constexpr size_t EM_SOLO_SMEM = 116 * 1024;
-static_assert(EM_KG * (2 * 256 * 128 + (EM_S - 2) * 128 * 128) <= (1 << 24), "group sums must stay exact in FP32");
-static_assert(EM_S * TC_N <= (int)EM_TMEM_COLS, "accumulators exceed the tensor-memory allocation");
+static_assert(EM_KG * (2 * 256 * 128 + 4 * 128 * 128) <= (1 << 24), "group sums (but the least significant) must stay exact in FP32");
+static_assert(EM_NA * TC_N <= (int)EM_TMEM_COLS, "accumulators exceed the tensor-memory allocation");
 
 // kind::f16 instruction descriptor: D = F32, A = B = F16, both K-major, 128 x n.
 __device__ __forceinline__ uint32_t em_idesc(int n) {
@@ -388,22 +392,25 @@ __device__ __forceinline__ void em_issue(uint32_t tmem, uint64_t da, uint64_t db
 // Issue the digit-pair products of one staged chunk (one thread; stage: the
 // buffer's shared-memory address).  The B planes of nbp rows follow each other,
 // and so do the accumulators of nbp columns: digit p of A times the digits
-// 1 .. 7 - p of B is one product of nbp (7 - p) columns into the accumulators
-// p .. 6, cut at 256 columns.  So 8 MMAs of up to 256 columns do the work of 21
-// of 64, which took the issuing thread 86 cycles each on a busy SM and read A
-// from shared memory 21 times.
+// 1 .. min(6, 8 - p) of B is one product of that many times nbp columns into the
+// accumulators from p on, cut at 256 columns.  So 10 MMAs of up to 256 columns do
+// the work of 26 of 64, which took the issuing thread 86 cycles each on a busy
+// SM and read A from shared memory 26 times.  (A group's first chunk sets the
+// accumulators: the last one, which digit 2 is the first to touch, by its own MMA.)
 __device__ __forceinline__ void em_issue_chunk(const EmCtx& cx, uint32_t stage, int nbp, bool gfirst) {
   // plane descriptors differ only in the start-address field (addr >> 4, 14 bits; shared memory
   // addresses stay below 2^18, so the offsets below never carry out of the field)
   const uint64_t da0 = em_desc(stage), db0 = em_desc(stage + 2 * EM_S * EM_A_HALFS);
 #pragma unroll
   for (int p = 1; p <= EM_S; ++p) {
-    const int cols = nbp * (EM_S + 1 - p);
     const uint64_t da = da0 + (uint64_t)(((p - 1) * EM_A_HALFS * 2) >> 4);
     const uint32_t dt = cx.tmem + (uint32_t)((p - 1) * nbp), ac = gfirst && p == 1 ? 0u : 1u;
+    const bool own = gfirst && p == EM_T - EM_S;
+    const int cols = nbp * (min(EM_S, EM_T - p) - (own ? 1 : 0));
     em_issue(dt, da, db0, ac, em_idesc(min(cols, 256)));
-    if (p < 3 && cols > 256)                       // (a row of a plane is 32 bytes)
+    if (p <= EM_T - 5 && cols > 256)               // (a row of a plane is 32 bytes)
       em_issue(dt + 256, da, db0 + 256 * 2, ac, em_idesc(cols - 256));
+    if (own) em_issue(dt + cols, da, db0 + (uint64_t)(cols * 2), 0u, em_idesc(nbp));
   }
 }
 
@@ -432,9 +439,9 @@ __device__ inline void em_drain(const EmCtx& cx, const int* cexp, int ei, int c0
 #pragma unroll
   for (int cb = 0; cb < EmAcc::NC; cb += 8) {
     if (c0 + cb >= nb) break;                        // warp-uniform
-    uint32_t v[EM_S][8];
+    uint32_t v[EM_NA][8];
 #pragma unroll
-    for (int t = 0; t < EM_S; ++t) em_ld8(base + (uint32_t)(t * nbp + c0 + cb), v[t]);
+    for (int t = 0; t < EM_NA; ++t) em_ld8(base + (uint32_t)(t * nbp + c0 + cb), v[t]);
     int f[8];
     *reinterpret_cast<int4*>(f) = *reinterpret_cast<const int4*>(cexp + c0 + cb);
     *reinterpret_cast<int4*>(f + 4) = *reinterpret_cast<const int4*>(cexp + c0 + cb + 4);
@@ -447,8 +454,9 @@ __device__ inline void em_drain(const EmCtx& cx, const int* cexp, int ei, int c0
       const float v0 = __uint_as_float(v[0][c]), v1 = __uint_as_float(v[1][c]), v2 = __uint_as_float(v[2][c]);
       const float s1 = fmaf(v1, 0x1p-8f, v0), r1 = fmaf(v1, 0x1p-8f, -(s1 - v0));
       const float gh = fmaf(v2, 0x1p-16f, s1), r2 = fmaf(v2, 0x1p-16f, -(gh - s1));
-      const float tail = fmaf(fmaf(__uint_as_float(v[5][c]), 0x1p-8f, __uint_as_float(v[4][c])), 0x1p-8f,
-                              __uint_as_float(v[3][c]));
+      float tail = __uint_as_float(v[EM_NA - 1][c]);
+#pragma unroll
+      for (int t = EM_NA - 2; t >= 3; --t) tail = fmaf(tail, 0x1p-8f, __uint_as_float(v[t][c]));
       const float gl = fmaf(tail, 0x1p-24f, r1 + r2);
       const int e = ei + f[c] + (127 - 16);
       const float s = (uint32_t)(e - 1) < 254u ? __int_as_float(e << 23) : 0.0f;
