@@ -593,9 +593,6 @@ __device__ void tile_mma_r(TileAccR<TR, TC>& acc, const double* A, long sai, lon
 }
 
 // ---- factorisations in shared memory ----------------------------------------
-// Lower Cholesky factor in place (A = L L'); the strict upper triangle is set
-// to zero.  A non-positive (or NaN) pivot sets *bad and is replaced by 1 so
-// the factorisation stays finite.  Returns nothing; ends with __syncthreads.
 // Packed lower-triangle index t -> (i, k), k <= i, t = i (i + 1) / 2 + k.
 __device__ __forceinline__ void tri_decode(int t, int& i, int& k) {
   int ii = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
@@ -605,47 +602,230 @@ __device__ __forceinline__ void tri_decode(int t, int& i, int& k) {
   k = t - ii * (ii + 1) / 2;
 }
 
-template <int NTH = NT>
-__device__ inline void chol_smem(double* A, int n, int lda, int* bad) {
-  // The pivot of column j (L_jj = d rsqrt(d), and rsqrt(d) to scale the
-  // column; long sequences on this chip's narrow FP64 pipe) is formed by
-  // thread 0 alone, right after it has
-  // applied the previous column's update to A_jj (element t = 0 of the
-  // trailing update is always its own), while the other threads update the
-  // rest of the trailing block.
-  __shared__ double piv;
-  __syncthreads();
-  if (threadIdx.x == 0 && n > 0) {
-    const double d = A[0];
-    const bool ok = d > 0.0;
-    const double rs = ok ? rsqrt(d) : 1.0;
-    if (!ok) *bad = 1;
-    A[0] = ok ? d * rs : 1.0;
-    piv = rs;
+// A DFMA instruction holds an SM sub-partition's FP64 unit for 64 cycles however
+// few of its lanes are active, dependent or not (measured), and a double rsqrt
+// for about five of them.  What these routines can save is therefore the
+// serial chain around the FP64 work, not the work: with one column at a time
+// (scale, barrier, rank-1 update with every element's index decoded again,
+// barrier) a 64 x 64 Cholesky factor took 64 us and its inverse 55 us, against
+// 11 us each of FP64 time on four units.  They go by panels of FB = 4 columns:
+// two barriers and one index decoding per four columns, and the next panel's
+// diagonal block is updated and factorised by one warp while the others update
+// the rest.  Every entry sees the same operations in the same order as with one
+// column at a time, so the factors are the same to the bit.
+constexpr int FB = 4;
+constexpr int LGRP_MAX = 4;        // blocks of one block-diagonal matrix (leaves or regions of one group)
+constexpr int FAC_MAX_N = 128;     // largest order (of all blocks together)
+constexpr int FAC_SCRATCH = FAC_MAX_N * (1 + 2 * FB);   // doubles of shared scratch of the inverse (idle staging)
+
+// The nb diagonal blocks of A start at rows seg[0] = 0 <= seg[1] <= ... <=
+// seg[nb] (= the order of A); ONE: a single block of order n1.  The panels of
+// all blocks run together.  STK (stacked storage): row i holds only its
+// block's columns, entry (i, k) of block b at A[i lda + k - seg[b]], lda >= the
+// largest block.
+template <bool STK, bool ONE>
+struct Blocks {
+  double* A;
+  int lda;
+  const int* seg;
+  int nb, n1;
+  __device__ __forceinline__ int count() const { return ONE ? 1 : nb; }
+  __device__ __forceinline__ int start(int b) const { return ONE ? 0 : seg[b]; }
+  __device__ __forceinline__ int len(int b) const { return ONE ? n1 : seg[b + 1] - seg[b]; }
+  __device__ __forceinline__ int longest() const {
+    int n = 0;
+    for (int b = 0; b < count(); ++b) n = max(n, len(b));
+    return n;
   }
-  __syncthreads();
-  for (int j = 0; j < n; ++j) {
-    const double inv = piv;
-    for (int i = j + 1 + threadIdx.x; i < n; i += NTH) A[i * lda + j] *= inv;
-    __syncthreads();                       // column j scaled; piv read by every thread
-    const int m = n - j - 1;
-    for (int t = threadIdx.x; t < m * (m + 1) / 2; t += NTH) {   // lower triangle of the trailing block
-      int ii, kk;
-      tri_decode(t, ii, kk);
-      const int i = j + 1 + ii, k = j + 1 + kk;
-      const double v = fma(-A[i * lda + j], A[k * lda + j], A[i * lda + k]);
-      if (t == 0) {                        // A_{j+1,j+1}: the next pivot
-        const bool ok = v > 0.0;
-        const double rs = ok ? rsqrt(v) : 1.0;
+  // entry (i, k) of block b, both counted from the block's start
+  __device__ __forceinline__ double* at(int b, int i, int k) const {
+    const int s0 = start(b);
+    return A + (s0 + i) * lda + k + (STK ? 0 : s0);
+  }
+  // item t of the concatenated per-block counts cnt(b): its block, t becomes the item within it
+  template <typename F>
+  __device__ __forceinline__ int find(int& t, F&& cnt) const {
+    int b = 0;
+    if (!ONE)
+      for (int c = cnt(0); t >= c; c = cnt(b)) {
+        t -= c;
+        ++b;
+      }
+    return b;
+  }
+  template <typename F>
+  __device__ __forceinline__ int total(F&& cnt) const {
+    int s = 0;
+    for (int b = 0; b < count(); ++b) s += cnt(b);
+    return s;
+  }
+};
+
+// Lower Cholesky factor of every block in place; a non-positive (or NaN) pivot
+// sets *bad and is replaced by 1 so the factorisation stays finite.
+template <bool STK, bool ONE, int NTH>
+__device__ inline void chol_panels(const Blocks<STK, ONE> M, int* bad) {
+  __shared__ double pinv[LGRP_MAX][FB];        // reciprocal square roots of the panel's pivots
+  static_assert(FB == 4, "the diagonal block's lanes and the solve below are written for four columns");
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nb = M.count();
+  // lane e < 10 holds entry (er, ec) of a 4 x 4 lower triangle, e = er (er + 1) / 2 + ec
+  const int er = lane < 1 ? 0 : (lane < 3 ? 1 : (lane < 6 ? 2 : 3)), ec = lane - er * (er + 1) / 2;
+  // one warp: the diagonal block at row j of block b, first (upd) updated with the panel before it
+  auto diagonal = [&](int b, int j, bool upd) {
+    const int w = min(FB, M.len(b) - j);
+    const bool in = lane < 10 && er < w;
+    double* const p = M.at(b, j + er, j + ec);
+    double x = in ? *p : 1.0;
+    if (upd && in)
+      for (int q = j - FB; q < j; ++q) x = fma(-*M.at(b, j + er, q), *M.at(b, j + ec, q), x);
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < FB; ++c) {
+      const double d = __shfl_sync(0xffffffffu, x, c * (c + 1) / 2 + c);
+      const bool ok = d > 0.0;
+      const double rs = ok ? rsqrt(d) : 1.0;
+      if (c < w && lane == 0) {
         if (!ok) *bad = 1;
-        A[i * lda + k] = ok ? v * rs : 1.0;
-        piv = rs;
-      } else {
-        A[i * lda + k] = v;
+        pinv[b][c] = rs;
+      }
+      if (ec == c) x = ok || er != c ? x * rs : 1.0;
+      const double xr = __shfl_sync(0xffffffffu, x, (er * (er + 1) / 2 + c) & 31);
+      const double xc = __shfl_sync(0xffffffffu, x, (ec * (ec + 1) / 2 + c) & 31);
+      if (ec > c) x = fma(-xr, xc, x);
+    }
+    if (in) *p = x;
+  };
+  __syncthreads();
+  if (warp < nb && M.len(warp) > 0) diagonal(warp, 0, false);
+  __syncthreads();
+  const int nmax = M.longest();
+  for (int j = 0; j + FB < nmax; j += FB) {
+    auto below = [&](int b) { return max(0, M.len(b) - j - FB); };
+    // the panel's rows below its diagonal block
+    const int rows = M.total(below);
+    for (int t = threadIdx.x; t < rows; t += NTH) {
+      int u = t;
+      const int b = M.find(u, below);
+      const double *L1 = M.at(b, j + 1, j), *L2 = M.at(b, j + 2, j), *L3 = M.at(b, j + 3, j);
+      double* a = M.at(b, j + FB + u, j);
+      const double l0 = a[0] * pinv[b][0];
+      const double l1 = fma(-l0, L1[0], a[1]) * pinv[b][1];
+      const double l2 = fma(-l1, L2[1], fma(-l0, L2[0], a[2])) * pinv[b][2];
+      const double l3 = fma(-l2, L3[2], fma(-l1, L3[1], fma(-l0, L3[0], a[3]))) * pinv[b][3];
+      a[0] = l0;
+      a[1] = l1;
+      a[2] = l2;
+      a[3] = l3;
+    }
+    __syncthreads();
+    // the trailing lower triangles; their first rows (the next diagonal blocks) by warp b, and while the
+    // rest is less than that chain takes, the other warps of its sub-partition leave it the FP64 unit
+    auto rest = [&](int b) {
+      const int m = below(b);
+      return m < FB ? 0 : m * (m + 1) / 2 - FB * (FB + 1) / 2;
+    };
+    const int tot = M.total(rest);
+    const bool leave = nb < 4 && tot < 900;
+    if (warp < nb) {
+      if (below(warp) > 0) diagonal(warp, j + FB, true);
+    } else if (!leave || (warp & 3) >= nb) {
+      const int id = leave ? (warp >> 2) * (4 - nb) + (warp & 3) - nb : warp - nb;
+      const int cnt = leave ? (NTH / 128) * (4 - nb) : NTH / 32 - nb;
+      for (int t = id * 32 + lane; t < tot; t += cnt * 32) {
+        int u = t, ii, kk;
+        const int b = M.find(u, rest);
+        tri_decode(u + FB * (FB + 1) / 2, ii, kk);
+        const double *x = M.at(b, j + FB + ii, j), *y = M.at(b, j + FB + kk, j);
+        double* p = M.at(b, j + FB + ii, j + FB + kk);
+        double v = *p;
+#pragma unroll
+        for (int q = 0; q < FB; ++q) v = fma(-x[q], y[q], v);
+        *p = v;
       }
     }
     __syncthreads();
   }
+}
+
+// Lower-triangular L of every block in place -> L^{-1}, by forward substitution
+// on the rows of the identity, four rows at a time: the panel's rows are
+// finished column by column (one thread a column), then their multiples are
+// subtracted from every row below.
+template <bool STK, bool ONE, int NTH>
+__device__ inline void trinv_panels(const Blocks<STK, ONE> M, double* scr) {
+  double* const rinv = scr;                            // 1 / L_ii
+  double* const lps = scr + FAC_MAX_N;                 // the panel's columns of L, before they are overwritten: two panels
+  auto save = [&](int j, int buf) {                    // rows j .. of columns j .. j + 3 of every block
+    auto cnt = [&](int b) { return max(0, M.len(b) - j) * FB; };
+    const int n = M.total(cnt);
+    for (int t = threadIdx.x; t < n; t += NTH) {
+      int u = t;
+      const int b = M.find(u, cnt);
+      const int i = j + u / FB, q = u % FB;
+      lps[buf * FAC_MAX_N * FB + (M.start(b) + i) * FB + q] = j + q <= i ? *M.at(b, i, j + q) : 0.0;
+    }
+  };
+  __syncthreads();
+  {
+    auto cnt = [&](int b) { return M.len(b); };
+    const int n = M.total(cnt);
+    for (int t = threadIdx.x; t < n; t += NTH) {
+      int u = t;
+      const int b = M.find(u, cnt);
+      rinv[t] = 1.0 / *M.at(b, u, u);
+    }
+  }
+  save(0, 0);
+  __syncthreads();
+  const int nmax = M.longest();
+  for (int j = 0, buf = 0; j < nmax; j += FB, buf ^= 1) {
+    // rows j .. j + w - 1: X_ik = (X_ik - sum_{s < i} L_is X_sk) / L_ii, one thread a column
+    auto width = [&](int b) { return min(FB, max(0, M.len(b) - j)); };
+    auto cols = [&](int b) { return width(b) ? j + width(b) : 0; };
+    const int nc = M.total(cols);
+    for (int t = threadIdx.x; t < nc; t += NTH) {
+      int k = t;
+      const int b = M.find(k, cols), w = width(b);
+      const double *l = lps + buf * FAC_MAX_N * FB + (M.start(b) + j) * FB, *ri = rinv + M.start(b) + j;
+      double x[FB];
+#pragma unroll
+      for (int q = 0; q < FB; ++q)
+        if (q < w) {
+          double* p = M.at(b, j + q, k);
+          double v = k < j ? *p : 0.0;
+#pragma unroll
+          for (int s = 0; s < q; ++s)
+            if (k <= j + s) v = fma(-l[q * FB + s], x[s], v);
+          x[q] = k < j + q ? v * ri[q] : ri[q];
+          if (k <= j + q) *p = x[q];
+        }
+    }
+    __syncthreads();
+    // X_ik -= sum_q L_iq X_qk for the rows below (the panel's own columns start from 0)
+    auto upd = [&](int b) { return max(0, M.len(b) - j - FB) * (j + FB); };
+    const int tot = M.total(upd), w = j + FB;
+    for (int t = threadIdx.x; t < tot; t += NTH) {
+      int u = t;
+      const int b = M.find(u, upd);
+      const int ii = u / w, k = u - ii * w, i = j + FB + ii;
+      const double* l = lps + buf * FAC_MAX_N * FB + (M.start(b) + i) * FB;
+      double* p = M.at(b, i, k);
+      double v = k < j ? *p : 0.0;
+#pragma unroll
+      for (int q = 0; q < FB; ++q)
+        if (k <= j + q) v = fma(-l[q], *M.at(b, j + q, k), v);
+      *p = v;
+    }
+    save(j + FB, buf ^ 1);
+    __syncthreads();
+  }
+}
+
+// Lower Cholesky factor in place (A = L L'); the strict upper triangle is set
+// to zero.  Ends with a barrier.
+template <int NTH = NT>
+__device__ inline void chol_smem(double* A, int n, int lda, int* bad) {
+  chol_panels<false, true, NTH>(Blocks<false, true>{A, lda, nullptr, 1, n}, bad);
   for (int t = threadIdx.x; t < n * n; t += NTH) {
     int i = t / n, k = t - i * n;
     if (k > i) A[i * lda + k] = 0.0;
@@ -653,19 +833,16 @@ __device__ inline void chol_smem(double* A, int n, int lda, int* bad) {
   __syncthreads();
 }
 
-// ---- block-diagonal factorisations (a group of leaves in one CTA) ---------
-// The nb diagonal blocks of A start at rows seg[0] = 0 <= seg[1] <= ... <=
-// seg[nb] (= the order of A).  chol_seg factorises every block in place as
-// chol_smem factorises one matrix and leaves every entry outside the blocks'
-// lower triangles zero; trinv_seg inverts every block's lower triangle as
-// trinv_smem does (the same operations per entry, so a block's factors are
-// those of the single-matrix routines).  The steps of all blocks run together,
-// so the barriers are those of the largest block alone.  pv: nb doubles of
-// shared memory (the blocks' pivots), tmp: seg[nb] doubles.  STK (stacked
-// storage): row i holds only its block's columns, entry (i, k) of block b at
-// A[i lda + k - seg[b]], lda >= the largest block.
-constexpr int LGRP_MAX = 4;        // leaves of one group (the children of one parent)
+// L^{-1} of the lower triangle in place (n <= FAC_MAX_N; scr: FAC_SCRATCH doubles).
+template <int NTH = NT>
+__device__ inline void trinv_smem(double* A, int n, int lda, double* scr) {
+  trinv_panels<false, true, NTH>(Blocks<false, true>{A, lda, nullptr, 1, n}, scr);
+}
 
+// ---- block-diagonal factorisations (a group of leaves in one CTA) ---------
+// chol_seg factorises every block in place as chol_smem factorises one matrix
+// and leaves every entry outside the blocks' lower triangles zero; trinv_seg
+// inverts every block's lower triangle as trinv_smem does.
 __device__ __forceinline__ int seg_block(const int* seg, int nb, int i) {   // block of row i
   int b = 0;
   while (b + 1 < nb && i >= seg[b + 1]) ++b;
@@ -673,59 +850,8 @@ __device__ __forceinline__ int seg_block(const int* seg, int nb, int i) {   // b
 }
 
 template <bool STK = false, int NTH = NT>
-__device__ inline void chol_seg(double* A, int lda, const int* seg, int nb, int* bad, double* pv) {
-  __syncthreads();
-  int nmax = 0;
-  for (int b = 0; b < nb; ++b) nmax = max(nmax, seg[b + 1] - seg[b]);
-  if (threadIdx.x < nb && seg[threadIdx.x + 1] > seg[threadIdx.x]) {
-    const int s0 = seg[threadIdx.x], cs = STK ? s0 : 0;
-    const double d = A[s0 * lda + s0 - cs];
-    const bool ok = d > 0.0;
-    const double rs = ok ? rsqrt(d) : 1.0;
-    if (!ok) *bad = 1;
-    A[s0 * lda + s0 - cs] = ok ? d * rs : 1.0;
-    pv[threadIdx.x] = rs;
-  }
-  __syncthreads();
-  for (int j = 0; j < nmax; ++j) {
-    int tot = 0, tri = 0;
-    for (int b = 0; b < nb; ++b) {
-      const int m = max(0, seg[b + 1] - seg[b] - j - 1);
-      tot += m;
-      tri += m * (m + 1) / 2;
-    }
-    for (int t = threadIdx.x; t < tot; t += NTH) {   // column j of every block scaled
-      int b = 0, u = t;
-      for (int m = max(0, seg[1] - seg[0] - j - 1); u >= m; m = max(0, seg[b + 1] - seg[b] - j - 1)) {
-        u -= m;
-        ++b;
-      }
-      const int s0 = seg[b], cs = STK ? s0 : 0;
-      A[(s0 + j + 1 + u) * lda + s0 + j - cs] *= pv[b];
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < tri; t += NTH) {   // trailing lower triangles; element 0: the next pivot
-      int b = 0, u = t;
-      for (int m = max(0, seg[1] - seg[0] - j - 1); u >= m * (m + 1) / 2; m = max(0, seg[b + 1] - seg[b] - j - 1)) {
-        u -= m * (m + 1) / 2;
-        ++b;
-      }
-      int ii, kk;
-      tri_decode(u, ii, kk);
-      const int s0 = seg[b], cs = STK ? s0 : 0, jc = s0 + j, i = jc + 1 + ii, k = jc + 1 + kk;
-      const double v = fma(-A[i * lda + jc - cs], A[k * lda + jc - cs], A[i * lda + k - cs]);
-      if (u == 0) {
-        const bool ok = v > 0.0;
-        const double rs = ok ? rsqrt(v) : 1.0;
-        if (!ok) *bad = 1;
-        A[i * lda + k - cs] = ok ? v * rs : 1.0;
-        pv[b] = rs;
-      } else {
-        A[i * lda + k - cs] = v;
-      }
-    }
-    __syncthreads();
-  }
+__device__ inline void chol_seg(double* A, int lda, const int* seg, int nb, int* bad) {
+  chol_panels<STK, false, NTH>(Blocks<STK, false>{A, lda, seg, nb, 0}, bad);
   const int n = seg[nb];
   if (STK) {                                   // (stacked: row i holds its block's columns only, lda of them)
     for (int t = threadIdx.x; t < n * lda; t += NTH) {
@@ -742,87 +868,8 @@ __device__ inline void chol_seg(double* A, int lda, const int* seg, int nb, int*
 }
 
 template <bool STK = false, int NTH = NT>
-__device__ inline void trinv_seg(double* A, int lda, const int* seg, int nb, double* tmp, double* pv) {
-  __syncthreads();
-  int nmax = 0;
-  for (int b = 0; b < nb; ++b) nmax = max(nmax, seg[b + 1] - seg[b]);
-  if (threadIdx.x < nb && seg[threadIdx.x + 1] > seg[threadIdx.x]) {
-    const int s0 = seg[threadIdx.x];
-    pv[threadIdx.x] = 1.0 / A[s0 * lda + (STK ? 0 : s0)];
-  }
-  __syncthreads();
-  for (int k = 0; k < nmax; ++k) {
-    // phase 1, every block with k < n_b: row k scaled by 1 / L_kk (X_kk = 1 / L_kk), and
-    // column k below the diagonal saved
-    int tot = 0, upd = 0;
-    for (int b = 0; b < nb; ++b) {
-      const int nbk = seg[b + 1] - seg[b];
-      if (k < nbk) {
-        tot += nbk;
-        upd += (nbk - k - 1) * (k + 1);
-      }
-    }
-    for (int t = threadIdx.x; t < tot; t += NTH) {
-      int b = 0, u = t;
-      for (int c = k < seg[1] - seg[0] ? seg[1] - seg[0] : 0; u >= c;
-           c = k < seg[b + 1] - seg[b] ? seg[b + 1] - seg[b] : 0) {
-        u -= c;
-        ++b;
-      }
-      const int s0 = seg[b], cs = STK ? s0 : 0, gk = s0 + k;
-      if (u <= k) A[gk * lda + s0 + u - cs] = u < k ? A[gk * lda + s0 + u - cs] * pv[b] : pv[b];
-      else tmp[s0 + u] = A[(s0 + u) * lda + gk - cs];
-    }
-    __syncthreads();
-    if (threadIdx.x < nb) {   // the next step's reciprocals (diagonal entries phase 2 does not write)
-      const int s0 = seg[threadIdx.x], cs = STK ? s0 : 0;
-      if (k + 1 < seg[threadIdx.x + 1] - s0) pv[threadIdx.x] = 1.0 / A[(s0 + k + 1) * lda + s0 + k + 1 - cs];
-    }
-    // phase 2: X_ij -= L_ik X_kj for i > k, j <= k, within every block
-    const int w = k + 1;
-    for (int t = threadIdx.x; t < upd; t += NTH) {
-      int b = 0, u = t;
-      for (int c = k < seg[1] - seg[0] ? (seg[1] - seg[0] - k - 1) * w : 0; u >= c;
-           c = k < seg[b + 1] - seg[b] ? (seg[b + 1] - seg[b] - k - 1) * w : 0) {
-        u -= c;
-        ++b;
-      }
-      const int s0 = seg[b], cs = STK ? s0 : 0, ii = u / w, j = u - ii * w, i = s0 + k + 1 + ii;
-      const double x0 = j == k ? 0.0 : A[i * lda + s0 + j - cs];
-      A[i * lda + s0 + j - cs] = fma(-tmp[i], A[(s0 + k) * lda + s0 + j - cs], x0);
-    }
-    __syncthreads();
-  }
-}
-
-// Lower-triangular L in place -> L^{-1}, by forward substitution on the rows
-// of the identity (right-looking): step k scales row k by 1 / L_kk and
-// subtracts L_ik times it from every row i > k.  Each step is a rank-1 update
-// over all threads, so the FP64 work is spread over every warp (the pipe of
-// every SM sub-partition).  tmp: n doubles of shared scratch.
-template <int NTH = NT>
-__device__ inline void trinv_smem(double* A, int n, int lda, double* tmp) {
-  __shared__ double piv;
-  __syncthreads();
-  if (threadIdx.x == 0 && n > 0) piv = 1.0 / A[0];
-  __syncthreads();
-  for (int k = 0; k < n; ++k) {
-    // phase 1: row k of X (columns < k) scaled by 1 / L_kk, X_kk = 1 / L_kk;
-    // column k of L below the diagonal saved before it is overwritten
-    const double rk = piv;
-    for (int t = threadIdx.x; t <= k; t += NTH) A[k * lda + t] = t < k ? A[k * lda + t] * rk : rk;
-    for (int i = k + 1 + threadIdx.x; i < n; i += NTH) tmp[i] = A[i * lda + k];
-    __syncthreads();
-    if (threadIdx.x == 0 && k + 1 < n) piv = 1.0 / A[(k + 1) * lda + k + 1];   // next step's reciprocal
-    // phase 2: X_ij -= L_ik X_kj for i > k, j <= k (X_ik starts from 0)
-    const int w = k + 1, nr = n - k - 1;
-    for (int t = threadIdx.x; t < nr * w; t += NTH) {
-      const int ii = t / w, j = t - ii * w, i = k + 1 + ii;
-      const double x0 = j == k ? 0.0 : A[i * lda + j];
-      A[i * lda + j] = fma(-tmp[i], A[k * lda + j], x0);
-    }
-    __syncthreads();
-  }
+__device__ inline void trinv_seg(double* A, int lda, const int* seg, int nb, double* scr) {
+  trinv_panels<STK, false, NTH>(Blocks<STK, false>{A, lda, seg, nb, 0}, scr);
 }
 
 // ---- reductions --------------------------------------------------------------

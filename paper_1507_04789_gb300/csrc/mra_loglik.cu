@@ -35,8 +35,7 @@ __global__ void __launch_bounds__(NT) prior_level_kernel(int m, const Desc* __re
   double* qy = qx + MAX_R_DEV;
   double* ax = qy + MAX_R_DEV;       // ancestor knots
   double* ay = ax + MAX_R_DEV;
-  double* tmp = ay + MAX_R_DEV;
-  double* red = tmp + MAX_R_DEV;
+  double* red = ay + MAX_R_DEV;
   double* W = red + 32;              // r x (r + 1)
   double* stg = W + MAX_R_DEV * (MAX_R_DEV + 1);
   __shared__ int bad;
@@ -88,7 +87,7 @@ __global__ void __launch_bounds__(NT) prior_level_kernel(int m, const Desc* __re
     for (int t = threadIdx.x; t < r * r; t += NT) Lr[t] = W[(t / r) * ldw + (t % r)];
     __syncthreads();
   }
-  trinv_smem(W, r, ldw, tmp);
+  trinv_smem(W, r, ldw, stg);
   double* Li = st.Li[m] + i * (long)r * r;
   for (int t = threadIdx.x; t < r * r; t += NT) Li[t] = W[(t / r) * ldw + (t % r)];
   if (threadIdx.x == 0 && bad) flag_error(status, ST_NOT_PD, m, i);
@@ -123,8 +122,7 @@ __global__ void __launch_bounds__(NT) leaf_kernel(const Desc* __restrict__ D, co
   double* sx = smem;
   double* sy = sx + nlmax;
   double* sv = sy + nlmax;
-  double* tmp = sv + nlmax;
-  double* ax = tmp + nlmax;
+  double* ax = sv + nlmax;
   double* ay = ax + MAX_R_DEV;
   double* red = ay + MAX_R_DEV;
   double* S = red + 32;                       // nlmax x (nlmax + 1)
@@ -207,7 +205,7 @@ __global__ void __launch_bounds__(NT) leaf_kernel(const Desc* __restrict__ D, co
   if (lf.VF) {
     for (long t = threadIdx.x; t < (long)nF * Mr; t += NT) lf.VF[o0 * Mr + t] = Hrow[t];
   }
-  trinv_smem(S, nF, lds, tmp);
+  trinv_smem(S, nF, lds, stg);
   double* LS = lf.LS + lf.sq_off[Fm];
   for (int t = threadIdx.x; t < nF * nF; t += NT) LS[t] = S[(t / nF) * lds + (t % nF)];
   // z = L_Sigma^{-1} y
@@ -326,8 +324,7 @@ __global__ void __launch_bounds__(EMU ? EM_NT : NT) post_level_kernel(int m, con
   const long i = it.i;
   const int T = (m + 1) * (m + 2) / 2;
   const int ldw = r + 1;
-  double* tmp = smem;
-  double* red = tmp + MAX_R_DEV;
+  double* red = smem;
   double* gs = red + 32;
   double* W = gs + MAX_R_DEV;
   double* stg = W + MAX_R_DEV * (MAX_R_DEV + 1);
@@ -348,7 +345,7 @@ __global__ void __launch_bounds__(EMU ? EM_NT : NT) post_level_kernel(int m, con
     for (int t = threadIdx.x; t < r * r; t += NTH) Lf[t] = W[(t / r) * ldw + (t % r)];
     __syncthreads();
   }
-  trinv_smem<NTH>(W, r, ldw, tmp);
+  trinv_smem<NTH>(W, r, ldw, EMU ? smem_all : stg);   // (the engine's staging is idle)
   double* Lt = st.Lt[m] + i * (long)r * r;
   for (int t = threadIdx.x; t < r * r; t += NTH) Lt[t] = W[(t / r) * ldw + (t % r)];
   // g = Lt^{-1} omegahat^m
@@ -474,17 +471,18 @@ __global__ void __launch_bounds__(NT) aggregate_kernel(int m, const Desc* __rest
 // ---------------------------------------------------------------------------
 // Host launchers
 // ---------------------------------------------------------------------------
+static_assert(2 * KC * (16 + 2) >= FAC_SCRATCH, "the inverse's scratch fits the smallest tile staging");
 static int tile_for(int r) { return r <= 16 ? 16 : (r <= 32 ? 32 : 64); }
 
 static size_t prior_smem(int tile) {
-  return sizeof(double) * (5 * MAX_R_DEV + 32 + MAX_R_DEV * (MAX_R_DEV + 1) + 2 * KC * (tile + 2));
+  return sizeof(double) * (4 * MAX_R_DEV + 32 + MAX_R_DEV * (MAX_R_DEV + 1) + 2 * KC * (tile + 2));
 }
 static size_t leaf_smem(int tile, int nlmax) {
-  return sizeof(double) * (4 * (size_t)nlmax + 2 * MAX_R_DEV + 32 + (size_t)nlmax * (nlmax + 1) +
+  return sizeof(double) * (3 * (size_t)nlmax + 2 * MAX_R_DEV + 32 + (size_t)nlmax * (nlmax + 1) +
                            2 * KC * (tile + 2));
 }
 static size_t post_smem(int tile) {
-  return sizeof(double) * (2 * MAX_R_DEV + 32 + MAX_R_DEV * (MAX_R_DEV + 1) + 2 * KC * (tile + 2));
+  return sizeof(double) * (MAX_R_DEV + 32 + MAX_R_DEV * (MAX_R_DEV + 1) + 2 * KC * (tile + 2));
 }
 static size_t syrk_smem(int tile) { return sizeof(double) * 2 * KC * (tile + 2); }
 

@@ -94,7 +94,6 @@ __global__ void __launch_bounds__(Engine<EMU>::NTH) prior_level_kernel_tc(int m,
   __shared__ double pgp[LGRP_MAX * C0_GMAX], pgq[LGRP_MAX * C0_GMAX];
   __shared__ unsigned char qcol[MAX_R_DEV], qrow[MAX_R_DEV];
   __shared__ int gseg[LGRP_MAX + 1];
-  __shared__ double gpv[LGRP_MAX];
   const Item it = work_item(work);
   const Desc& ds = D[it.d];
   const Shape sh = ds.sh;
@@ -122,8 +121,7 @@ __global__ void __launch_bounds__(Engine<EMU>::NTH) prior_level_kernel_tc(int m,
   double* qy = qx + rcap;
   double* ax = qy + rcap;
   double* ay = ax + MAX_R_DEV;
-  double* tmp = ay + MAX_R_DEV;                 // rcap
-  double* W = tmp + rcap;                       // rcap x (r + 1): region g's block in rows g r .. g r + r - 1
+  double* W = ay + MAX_R_DEV;                       // rcap x (r + 1): region g's block in rows g r .. g r + r - 1
   // offsets between every stacked region's knot grid (qx, qy) + g r and the grid
   // (bx, by), or (self) the region's own grid (all threads; the caller
   // synchronises before and after)
@@ -265,15 +263,16 @@ __global__ void __launch_bounds__(Engine<EMU>::NTH) prior_level_kernel_tc(int m,
     __syncthreads();
   }
   if (ok) {
+    double* scr = reinterpret_cast<double*>(dsm);   // (the engine's staging is idle)
     if (G == 1) chol_smem<NTH>(W, r, ldw, &bad);
-    else chol_seg<true, NTH>(W, ldw, gseg, G, &bad, gpv);
+    else chol_seg<true, NTH>(W, ldw, gseg, G, &bad);
     if (st.L[m]) {
       double* Lr = st.L[m] + i * (long)r * r;
       for (int t = threadIdx.x; t < R * r; t += NTH) Lr[t] = W[(t / r) * ldw + (t % r)];
       __syncthreads();
     }
-    if (G == 1) trinv_smem<NTH>(W, r, ldw, tmp);
-    else trinv_seg<true, NTH>(W, ldw, gseg, G, tmp, gpv);
+    if (G == 1) trinv_smem<NTH>(W, r, ldw, scr);
+    else trinv_seg<true, NTH>(W, ldw, gseg, G, scr);
     double* Li = st.Li[m] + i * (long)r * r;
     for (int t = threadIdx.x; t < R * r; t += NTH) Li[t] = W[(t / r) * ldw + (t % r)];
     if (EMU) {   // row scales of V_R and L_R^{-1} for the descendants' products
@@ -694,7 +693,7 @@ __global__ void __launch_bounds__(Engine<EMU>::NTH) leaf_kernel_tc(const Desc* _
       for (int t = threadIdx.x; t < nF; t += NTH) ld += log(S[t * lds + t]);
       ld = 2.0 * block_sum<NTH>(ld, red);
     } else {
-      chol_seg<false, NTH>(S, lds, gseg, G, &bad, red);
+      chol_seg<false, NTH>(S, lds, gseg, G, &bad);
       for (int t = threadIdx.x; t < nF; t += NTH) tmp[t] = log(S[t * lds + t]);
       __syncthreads();
       ld = 2.0 * leaf_sum();
@@ -709,8 +708,9 @@ __global__ void __launch_bounds__(Engine<EMU>::NTH) leaf_kernel_tc(const Desc* _
     }
     if (lf.VF)
       for (long t = threadIdx.x; t < (long)nF * Mr; t += NTH) lf.VF[o0 * Mr + t] = Hrow[t];
-    if (G == 1) trinv_smem<NTH>(S, nF, lds, tmp);
-    else trinv_seg<false, NTH>(S, lds, gseg, G, tmp, red);
+    double* scr = reinterpret_cast<double*>(dsm);   // (the engine's staging is idle)
+    if (G == 1) trinv_smem<NTH>(S, nF, lds, scr);
+    else trinv_seg<false, NTH>(S, lds, gseg, G, scr);
     if (EMU) {   // row scales of L_Sigma^{-1} (lower triangular) for the solve below
       for (int t = threadIdx.x; t < nF; t += NTH) {
         int e = -2000;
@@ -1089,8 +1089,8 @@ __global__ void __launch_bounds__(EM_NT) aggregate_kernel_em(int m, const Desc* 
 
 
 template <bool EMU>
-static size_t prior_tc_smem(int rcap) {     // knots (2 rcap), ancestor knots, scratch (rcap), W (rcap x (r + 1))
-  const size_t b = Engine<EMU>::STAGE + sizeof(double) * (3 * (size_t)rcap + 2 * MAX_R_DEV +
+static size_t prior_tc_smem(int rcap) {     // knots (2 rcap), ancestor knots, W (rcap x (r + 1))
+  const size_t b = Engine<EMU>::STAGE + sizeof(double) * (2 * (size_t)rcap + 2 * MAX_R_DEV +
                                                           (size_t)rcap * (MAX_R_DEV + 1));
   return EMU ? std::max(b, EM_SOLO_SMEM) : b;
 }
