@@ -592,6 +592,62 @@ __device__ void tile_mma_r(TileAccR<TR, TC>& acc, const double* A, long sai, lon
   __syncthreads();
 }
 
+// f(i, j, sum_k A(i, k) B(j, k)) for i < na <= 64, j < nb <= TC, in a tile of na
+// rows rounded up to 16.  The FP64 unit takes 64 cycles for a DFMA instruction
+// whatever its lanes do, so rows that only fill a tile cost as much as kept ones,
+// while a thread's loads (one or two a DFMA even at one output row a thread)
+// stay far below the shared-memory rate: leaves of 66 observations on 64-row
+// tiles paid for 128.  Opens and ends with a barrier; smem: KC (64 + TC + 4) doubles.
+template <int TR, int TC, typename F>
+__device__ __forceinline__ void mma_rows_tile(const double* A, long sai, long sak, int na, const double* B, long sbj,
+                                              long sbk, int nb, int K, double* smem, F&& f) {
+  TileAccR<TR, TC> acc;
+  acc.zero();
+  tile_mma_r<TR, TC>(acc, A, sai, sak, na, B, sbj, sbk, nb, K, smem);
+#pragma unroll
+  for (int p = 0; p < TileAccR<TR, TC>::RR; ++p)
+#pragma unroll
+    for (int q = 0; q < TileAccR<TR, TC>::RC; ++q) {
+      const int row = acc.row(p), col = acc.col(q);
+      if (row < na && col < nb) f(row, col, acc.v[p][q]);
+    }
+}
+template <int TC, typename F>
+__device__ __forceinline__ void mma_rows(const double* A, long sai, long sak, int na, const double* B, long sbj,
+                                         long sbk, int nb, int K, double* smem, F&& f) {
+  if (na <= 16) mma_rows_tile<16, TC>(A, sai, sak, na, B, sbj, sbk, nb, K, smem, f);
+  else if (na <= 32) mma_rows_tile<32, TC>(A, sai, sak, na, B, sbj, sbk, nb, K, smem, f);
+  else if (na <= 48) mma_rows_tile<48, TC>(A, sai, sak, na, B, sbj, sbk, nb, K, smem, f);
+  else mma_rows_tile<64, TC>(A, sai, sak, na, B, sbj, sbk, nb, K, smem, f);
+}
+constexpr int mma_rows_smem(int tc) { return KC * (64 + 2 + tc + 2); }
+
+// f(i, j, sum_k X(i, k) L(j, k)) for i < na <= 64, j < n <= 64 with L lower
+// triangular (L(j, k) = 0 for k > j): 16 columns at a time over the k they have,
+// 5/8 of the full product at n = 64.  The columns are taken from the last, so f
+// may overwrite X(i, j): the columns still to come read X(., k <= j) only.
+template <typename F>
+__device__ __forceinline__ void mma_lower_t(const double* X, long sxi, long sxk, int na, const double* L, long slj,
+                                            long slk, int n, double* smem, F&& f) {
+  for (int c0 = ((n - 1) >> 4) << 4; c0 >= 0; c0 -= 16) {
+    const int nb = min(16, n - c0);
+    mma_rows<16>(X, sxi, sxk, na, L + c0 * slj, slj, slk, nb, c0 + nb, smem,
+                 [&](int i, int j, double v) { f(i, c0 + j, v); });
+  }
+}
+
+// f(i, j, sum_k A(i, k) A(j, k)) for j <= i < n: the lower triangle of a Gram
+// product, 16 columns at a time over the rows from their first on.
+template <typename F>
+__device__ __forceinline__ void mma_gram_lower(const double* A, long si, long sk, int n, int K, double* smem, F&& f) {
+  for (int c0 = 0; c0 < n; c0 += 16)
+    for (int r0 = c0; r0 < n; r0 += 64)
+      mma_rows<16>(A + r0 * si, si, sk, min(64, n - r0), A + c0 * si, si, sk, min(16, n - c0), K, smem,
+                   [&](int i, int j, double v) {
+                     if (c0 + j <= r0 + i) f(r0 + i, c0 + j, v);
+                   });
+}
+
 // ---- factorisations in shared memory ----------------------------------------
 // Packed lower-triangle index t -> (i, k), k <= i, t = i (i + 1) / 2 + k.
 __device__ __forceinline__ void tri_decode(int t, int& i, int& k) {

@@ -42,45 +42,23 @@ __global__ void __launch_bounds__(NT) prior_level_kernel(int m, const Desc* __re
   if (threadIdx.x == 0) bad = 0;
   load_knots(sh, m, st.mort[m][i], qx, qy);
   double* Vrow = st.V[m] + i * (long)r * mr;
-  TileAcc<TILE> acc;
   for (int l = 0; l < m; ++l) {
     const long a = ancestor(st, m, i, l);
     __syncthreads();
     load_knots(sh, l, st.mort[l][a], ax, ay);
     const double* Vanc = st.V[l] + a * (long)r * (l * r);
-    acc.zero();
-    if (l > 0) tile_mma<TILE>(acc, Vrow, mr, 1, r, Vanc, l * r, 1, r, l * r, stg);
+    mma_rows<TILE>(Vrow, mr, 1, r, Vanc, l * r, 1, r, l * r, stg, [&](int row, int col, double v) {
+      Vrow[(long)row * mr + l * r + col] = cov0(cv, qx[row], qy[row], ax[col], ay[col]) - v;
+    });
     __syncthreads();
-#pragma unroll
-    for (int p = 0; p < TileAcc<TILE>::RM; ++p)
-#pragma unroll
-      for (int q = 0; q < TileAcc<TILE>::RM; ++q) {
-        int row = acc.row(p), col = acc.col(q);
-        if (row < r && col < r)
-          Vrow[(long)row * mr + l * r + col] = cov0(cv, qx[row], qy[row], ax[col], ay[col]) - acc.v[p][q];
-      }
-    __syncthreads();
-    acc.zero();
-    tile_mma<TILE>(acc, Vrow + l * r, mr, 1, r, st.Li[l] + a * (long)r * r, r, 1, r, r, stg);
-#pragma unroll
-    for (int p = 0; p < TileAcc<TILE>::RM; ++p)
-#pragma unroll
-      for (int q = 0; q < TileAcc<TILE>::RM; ++q) {
-        int row = acc.row(p), col = acc.col(q);
-        if (row < r && col < r) Vrow[(long)row * mr + l * r + col] = acc.v[p][q];
-      }
+    mma_lower_t(Vrow + l * r, mr, 1, r, st.Li[l] + a * (long)r * r, r, 1, r, stg,
+                [&](int row, int col, double v) { Vrow[(long)row * mr + l * r + col] = v; });
   }
   __syncthreads();
-  acc.zero();
-  if (m > 0) tile_mma<TILE>(acc, Vrow, mr, 1, r, Vrow, mr, 1, r, mr, stg);
   const int ldw = r + 1;
-#pragma unroll
-  for (int p = 0; p < TileAcc<TILE>::RM; ++p)
-#pragma unroll
-    for (int q = 0; q < TileAcc<TILE>::RM; ++q) {
-      int row = acc.row(p), col = acc.col(q);
-      if (row < r && col < r) W[row * ldw + col] = cov0(cv, qx[row], qy[row], qx[col], qy[col]) - acc.v[p][q];
-    }
+  mma_gram_lower(Vrow, mr, 1, r, mr, stg, [&](int row, int col, double v) {
+    W[row * ldw + col] = cov0(cv, qx[row], qy[row], qx[col], qy[col]) - v;
+  });
   chol_smem(W, r, ldw, &bad);
   if (st.L[m]) {
     double* Lr = st.L[m] + i * (long)r * r;
@@ -135,9 +113,6 @@ __global__ void __launch_bounds__(NT) leaf_kernel(const Desc* __restrict__ D, co
     sv[t] = lf.yv[o0 + t];
   }
   double* Hrow = lf.H + o0 * Mr;
-  const int nrt = (nF + TILE - 1) / TILE;
-  TileAcc<TILE> acc;
-  constexpr int RM = TileAcc<TILE>::RM;
   // chain: V^l_F = (C0(S_F, Q_l) - sum_{k<l} V^k_F V^k_{R_l}') L_l^{-T}
   for (int l = 0; l < M; ++l) {
     const long a = ancestor(st, M, F, l);
@@ -145,55 +120,23 @@ __global__ void __launch_bounds__(NT) leaf_kernel(const Desc* __restrict__ D, co
     load_knots(sh, l, st.mort[l][a], ax, ay);
     const double* Vanc = st.V[l] + a * (long)r * (l * r);
     __syncthreads();
-    for (int rt = 0; rt < nrt; ++rt) {
-      const int nrow = min(TILE, nF - rt * TILE);
-      acc.zero();
-      if (l > 0) tile_mma<TILE>(acc, Hrow + (long)rt * TILE * Mr, Mr, 1, nrow, Vanc, l * r, 1, r, l * r, stg);
-#pragma unroll
-      for (int p = 0; p < RM; ++p)
-#pragma unroll
-        for (int q = 0; q < RM; ++q) {
-          int row = acc.row(p), col = acc.col(q);
-          if (row < nrow && col < r) {
-            int o = rt * TILE + row;
-            Hrow[(long)o * Mr + l * r + col] = cov0(cv, sx[o], sy[o], ax[col], ay[col]) - acc.v[p][q];
-          }
-        }
-    }
+    for (int r0 = 0; r0 < nF; r0 += 64)
+      mma_rows<TILE>(Hrow + (long)r0 * Mr, Mr, 1, min(64, nF - r0), Vanc, l * r, 1, r, l * r, stg,
+                     [&](int row, int col, double v) {
+                       const int o = r0 + row;
+                       Hrow[(long)o * Mr + l * r + col] = cov0(cv, sx[o], sy[o], ax[col], ay[col]) - v;
+                     });
     __syncthreads();
-    for (int rt = 0; rt < nrt; ++rt) {
-      const int nrow = min(TILE, nF - rt * TILE);
-      acc.zero();
-      tile_mma<TILE>(acc, Hrow + (long)rt * TILE * Mr + l * r, Mr, 1, nrow, st.Li[l] + a * (long)r * r, r, 1, r, r, stg);
-#pragma unroll
-      for (int p = 0; p < RM; ++p)
-#pragma unroll
-        for (int q = 0; q < RM; ++q) {
-          int row = acc.row(p), col = acc.col(q);
-          if (row < nrow && col < r) Hrow[(long)(rt * TILE + row) * Mr + l * r + col] = acc.v[p][q];
-        }
-    }
+    for (int r0 = 0; r0 < nF; r0 += 64)
+      mma_lower_t(Hrow + (long)r0 * Mr + l * r, Mr, 1, min(64, nF - r0), st.Li[l] + a * (long)r * r, r, 1, r, stg,
+                  [&](int row, int col, double v) { Hrow[(long)(r0 + row) * Mr + l * r + col] = v; });
   }
   __syncthreads();
-  // Sigma_F = C0(S_F, S_F) - V_F V_F' + tau2 I  (lower blocks)
-  for (int bi = 0; bi < nrt; ++bi)
-    for (int bj = 0; bj <= bi; ++bj) {
-      const int ni = min(TILE, nF - bi * TILE), nj = min(TILE, nF - bj * TILE);
-      acc.zero();
-      if (M > 0) tile_mma<TILE>(acc, Hrow + (long)bi * TILE * Mr, Mr, 1, ni, Hrow + (long)bj * TILE * Mr, Mr, 1, nj, Mr, stg);
-#pragma unroll
-      for (int p = 0; p < RM; ++p)
-#pragma unroll
-        for (int q = 0; q < RM; ++q) {
-          int row = acc.row(p), col = acc.col(q);
-          if (row < ni && col < nj) {
-            int oi = bi * TILE + row, oj = bj * TILE + col;
-            double v = cov0(cv, sx[oi], sy[oi], sx[oj], sy[oj]) - acc.v[p][q];
-            if (oi == oj) v += tau2;
-            S[oi * lds + oj] = v;
-          }
-        }
-    }
+  // Sigma_F = C0(S_F, S_F) - V_F V_F' + tau2 I  (lower triangle)
+  mma_gram_lower(Hrow, Mr, 1, nF, Mr, stg, [&](int oi, int oj, double v) {
+    const double c = cov0(cv, sx[oi], sy[oi], sx[oj], sy[oj]) - v;
+    S[oi * lds + oj] = oi == oj ? c + tau2 : c;
+  });
   chol_smem(S, nF, lds, &bad);
   double ld = 0.0;
   for (int t = threadIdx.x; t < nF; t += NT) ld += log(S[t * lds + t]);
@@ -222,23 +165,12 @@ __global__ void __launch_bounds__(NT) leaf_kernel(const Desc* __restrict__ D, co
     lf.u[F] = zz;
     if (bad) flag_error(status, ST_NOT_PD, M, F);
   }
-  // H^l = L_Sigma^{-1} V^l_F, in place: row tiles from the last, since row
-  // tile t only reads rows below its end (L_Sigma^{-1} is lower triangular).
+  // H^l = L_Sigma^{-1} V^l_F, in place: 16-row tiles from the last, since a row
+  // only reads the rows up to its own (L_Sigma^{-1} is lower triangular).
   for (int l = 0; l < M; ++l)
-    for (int rt = nrt - 1; rt >= 0; --rt) {
-      const int nrow = min(TILE, nF - rt * TILE);
-      const int kend = rt * TILE + nrow;
-      acc.zero();
-      tile_mma<TILE>(acc, S + rt * TILE * lds, lds, 1, nrow, Hrow + l * r, 1, Mr, r, kend, stg);
-#pragma unroll
-      for (int p = 0; p < RM; ++p)
-#pragma unroll
-        for (int q = 0; q < RM; ++q) {
-          int row = acc.row(p), col = acc.col(q);
-          if (row < nrow && col < r) Hrow[(long)(rt * TILE + row) * Mr + l * r + col] = acc.v[p][q];
-        }
-      __syncthreads();
-    }
+    for (int r0 = ((nF - 1) >> 4) << 4; r0 >= 0; r0 -= 16)
+      mma_rows_tile<16, TILE>(S + r0 * lds, lds, 1, min(16, nF - r0), Hrow + l * r, 1, Mr, r, min(r0 + 16, nF), stg,
+                              [&](int row, int col, double v) { Hrow[(long)(r0 + row) * Mr + l * r + col] = v; });
 }
 
 // ---------------------------------------------------------------------------
@@ -265,19 +197,17 @@ __global__ void __launch_bounds__(NT) leaf_syrk_kernel(const Desc* __restrict__ 
   const long row0 = lf.off[pm << leaf_bits(ds.sh)], row1 = lf.off[(pm + 1) << leaf_bits(ds.sh)];
   const int K = (int)(row1 - row0);
   const double* Hb = lf.H + row0 * Mr;
-  TileAcc<TILE> acc;
-  acc.zero();
-  tile_mma<TILE>(acc, Hb + k * r, 1, Mr, r, Hb + l * r, 1, Mr, r, K, smem);
   const int m = M - 1;
   const int T = (m + 1) * (m + 2) / 2;
   double* out = st.Acc[m] + (p * T + t) * (long)r * r;
-#pragma unroll
-  for (int a = 0; a < TileAcc<TILE>::RM; ++a)
-#pragma unroll
-    for (int b = 0; b < TileAcc<TILE>::RM; ++b) {
-      int row = acc.row(a), col = acc.col(b);
-      if (row < r && col < r) out[row * r + col] = acc.v[a][b];
-    }
+  if (k == l)                                    // symmetric: the lower triangle, mirrored
+    mma_gram_lower(Hb + k * r, 1, Mr, r, K, smem, [&](int row, int col, double v) {
+      out[row * r + col] = v;
+      out[col * r + row] = v;
+    });
+  else
+    mma_rows<TILE>(Hb + k * r, 1, Mr, r, Hb + l * r, 1, Mr, r, K, smem,
+                   [&](int row, int col, double v) { out[row * r + col] = v; });
   if (k == l) {
     double* om = st.Om[m] + (p * (m + 1) + k) * (long)r;
     for (int a = threadIdx.x; a < r; a += NT) {
@@ -374,18 +304,12 @@ __global__ void __launch_bounds__(EMU ? EM_NT : NT) post_level_kernel(int m, con
       }
     }
   } else {
-    TileAcc<TILE> acc;
+    // 16 rows at a time over the k they have (Lt^{-1} is lower triangular)
     for (int l = 0; l < m; ++l) {
       const double* Aml = A + (long)tri_index(m, l) * r * r;
-      acc.zero();
-      tile_mma<TILE>(acc, W, ldw, 1, r, Aml, 1, r, r, r, stg);
-#pragma unroll
-      for (int a = 0; a < TileAcc<TILE>::RM; ++a)
-#pragma unroll
-        for (int b = 0; b < TileAcc<TILE>::RM; ++b) {
-          int row = acc.row(a), col = acc.col(b);
-          if (row < r && col < r) Gr[(long)row * mr + l * r + col] = acc.v[a][b];
-        }
+      for (int r0 = 0; r0 < r; r0 += 16)
+        mma_rows_tile<16, TILE>(W + r0 * ldw, ldw, 1, min(16, r - r0), Aml, 1, r, r, min(r0 + 16, r), stg,
+                                [&](int row, int col, double v) { Gr[(long)(r0 + row) * mr + l * r + col] = v; });
     }
   }
   if (st.gcol[m]) {   // emulation: column scales of G over its r rows, for the aggregation above
@@ -438,21 +362,21 @@ __global__ void __launch_bounds__(NT) aggregate_kernel(int m, const Desc* __rest
   const int Tp = m * (m + 1) / 2;         // blocks per parent (level m-1)
   const long cf = st.cfirst[m - 1][p], cc = st.ccnt[m - 1][p];   // children: compact ids cf..cf+cc-1
   const double* Gb = st.G[m] + cf * (long)r * mr;
-  TileAcc<TILE> acc;
-  acc.zero();
-  tile_mma<TILE>(acc, Gb + k * r, 1, mr, r, Gb + l * r, 1, mr, r, (int)(cc * r), smem);
   double* out = st.Acc[m - 1] + (p * Tp + t) * (long)r * r;
-#pragma unroll
-  for (int a = 0; a < TileAcc<TILE>::RM; ++a)
-#pragma unroll
-    for (int b = 0; b < TileAcc<TILE>::RM; ++b) {
-      int row = acc.row(a), col = acc.col(b);
-      if (row < r && col < r) {
-        double s = -acc.v[a][b];
-        for (long c = cf; c < cf + cc; ++c) s += st.Acc[m][(c * Tc + t) * (long)r * r + row * r + col];
-        out[row * r + col] = s;
-      }
-    }
+  auto sum = [&](int e, double v) {
+    double s = -v;
+    for (long c = cf; c < cf + cc; ++c) s += st.Acc[m][(c * Tc + t) * (long)r * r + e];
+    return s;
+  };
+  if (k == l)                                    // symmetric: the lower triangle, mirrored
+    mma_gram_lower(Gb + k * r, 1, mr, r, (int)(cc * r), smem, [&](int row, int col, double v) {
+      const double s = sum(row * r + col, v);
+      out[row * r + col] = s;
+      out[col * r + row] = s;
+    });
+  else
+    mma_rows<TILE>(Gb + k * r, 1, mr, r, Gb + l * r, 1, mr, r, (int)(cc * r), smem,
+                   [&](int row, int col, double v) { out[row * r + col] = sum(row * r + col, v); });
   if (k == l) {
     double* om = st.Om[m - 1] + (p * m + k) * (long)r;
     for (int a = threadIdx.x; a < r; a += NT) {
@@ -471,20 +395,20 @@ __global__ void __launch_bounds__(NT) aggregate_kernel(int m, const Desc* __rest
 // ---------------------------------------------------------------------------
 // Host launchers
 // ---------------------------------------------------------------------------
-static_assert(2 * KC * (16 + 2) >= FAC_SCRATCH, "the inverse's scratch fits the smallest tile staging");
+static_assert(mma_rows_smem(16) >= FAC_SCRATCH, "the inverse's scratch fits the smallest tile staging");
 static int tile_for(int r) { return r <= 16 ? 16 : (r <= 32 ? 32 : 64); }
 
 static size_t prior_smem(int tile) {
-  return sizeof(double) * (4 * MAX_R_DEV + 32 + MAX_R_DEV * (MAX_R_DEV + 1) + 2 * KC * (tile + 2));
+  return sizeof(double) * (4 * MAX_R_DEV + 32 + MAX_R_DEV * (MAX_R_DEV + 1) + mma_rows_smem(tile));
 }
 static size_t leaf_smem(int tile, int nlmax) {
   return sizeof(double) * (3 * (size_t)nlmax + 2 * MAX_R_DEV + 32 + (size_t)nlmax * (nlmax + 1) +
-                           2 * KC * (tile + 2));
+                           mma_rows_smem(tile));
 }
 static size_t post_smem(int tile) {
-  return sizeof(double) * (MAX_R_DEV + 32 + MAX_R_DEV * (MAX_R_DEV + 1) + 2 * KC * (tile + 2));
+  return sizeof(double) * (MAX_R_DEV + 32 + MAX_R_DEV * (MAX_R_DEV + 1) + mma_rows_smem(tile));
 }
-static size_t syrk_smem(int tile) { return sizeof(double) * 2 * KC * (tile + 2); }
+static size_t syrk_smem(int tile) { return sizeof(double) * mma_rows_smem(tile); }
 
 #define MRA_LAUNCH_ONE(T, KERNEL, grid, smem, stream, ...)                \
   {                                                                      \
