@@ -1788,9 +1788,14 @@ int mra_predict(mra_handle* h, const mra_params* theta, const double* plocs, int
   mra::PredState ps = pred_state(h);
   ps.mean = where == MRA_DEVICE ? mean_out : h->p_mean;
   ps.var = where == MRA_DEVICE ? var_out : h->p_var;
+  const int lb = M > 0 ? mra::leaf_bits(h->hd.sh) : 0;
+  auto launch = [&](long nleaf) {                // the points of nleaf leaves from ps.leaf0
+    if (h->cfg.precision == MRA_PREC_EMU && mra::predict_on_engine(M, r, lb, maxp, nleaf))
+      return mra::launch_predict_em(h->d_desc, lb, h->nlmax, ps, maxp, nleaf, h->status, h->stream, &g_launches, &h->timer);
+    return mra::launch_predict(h->d_desc, M, r, h->nlmax, ps, maxp, h->status, h->stream, &g_launches, &h->timer, nleaf);
+  };
   if (!h->s_lvl) {
-    if ((e = mra::launch_predict(h->d_desc, M, r, h->nlmax, ps, maxp, h->status, h->stream, &g_launches, &h->timer)))
-      return cuda_fail(e, "predict launch");
+    if ((e = launch(ps.nleaves))) return cuda_fail(e, "predict launch");
   } else {
     // Streamed: the coarse factors (levels <= s) are resident from the
     // evaluation; each chunk's own factors are formed again from them (its
@@ -1802,8 +1807,7 @@ int mra_predict(mra_handle* h, const mra_params* theta, const double* plocs, int
       ps.desc = (int)g;
       ps.leaf0 = (long)c.f0;
       if ((e = mra::launch_loglik(c.plan, h->d_desc, h->status, h->stream, &g_launches, &h->timer)) ||
-          (e = mra::launch_predict(h->d_desc, M, r, h->nlmax, ps, maxp, h->status, h->stream, &g_launches, &h->timer,
-                                   (long)c.nf)))
+          (e = launch((long)c.nf)))
         return cuda_fail(e, "predict launch");
     }
   }

@@ -639,6 +639,68 @@ __device__ inline bool em_mma(EmCtx& cx, EmAcc& acc, const double* A, long sai, 
   return ok;
 }
 
+// A product and what becomes of it, for kernels with many products: one call,
+// since inlined at every product the engine's state and the kernel's own crowd
+// each other out of the 128 registers a thread has.
+//   out(i, j) = P(i, j)  or, with sub, out(i, j) -= P(i, j),  i < na, j < nb,
+// row-major with stride ldo; the exponents of the results' rows go to xe[i]
+// (columns j >= xe0; null: none), and per 128-column group, counted from column
+// gcol for j = 0, to ge[group * TC_M + i] (null: none).
+struct EmRows {
+  const double* A;
+  long sai, sak;
+  int na;
+  const double* B;
+  long sbj, sbk;
+  int nb, K;
+  const int* pa;
+  int pas;
+  const int* pb;
+  int pbs;
+  double* out;
+  long ldo;
+  bool sub;
+  int* xe;
+  int xe0;
+  int* ge;
+  int gcol;
+};
+static __device__ __noinline__ bool em_rows(EmCtx* pcx, const EmRows* pq) {
+  EmCtx cx = *pcx;
+  EmAcc acc;
+  const bool ok = em_mma(cx, acc, pq->A, pq->sai, pq->sak, pq->na, pq->B, pq->sbj, pq->sbk, pq->nb, pq->K, pq->pa,
+                         pq->pas, pq->pb, pq->pbs);
+  pcx->chunks = cx.chunks;
+  pcx->groups = cx.groups;
+  const int row = acc.row(), c0 = acc.col0(), nb = pq->nb;
+  if (ok && row < pq->na && c0 < nb) {
+    double* const o = pq->out + (long)row * pq->ldo + c0;
+    if (pq->sub) {
+#pragma unroll
+      for (int c = 0; c < EmAcc::NC; ++c)
+        if (c0 + c < nb) acc.v[c] = o[c] - acc.v[c];
+    }
+    int e0 = -2000, e1 = -2000, ex = -2000;      // a thread's columns touch at most two groups
+    const int x0 = pq->xe0 - c0, g0 = EM_KG - ((pq->gcol + c0) & (EM_KG - 1));
+#pragma unroll
+    for (int c = 0; c < EmAcc::NC; ++c)
+      if (c0 + c < nb) {
+        o[c] = acc.v[c];
+        const int e = xexp_of(acc.v[c]);
+        if (c < g0) e0 = max(e0, e);
+        else e1 = max(e1, e);
+        if (c >= x0) ex = max(ex, e);
+      }
+    if (pq->xe && ex > -2000) atomicMax(pq->xe + row, ex);
+    if (pq->ge) {
+      int* const g = pq->ge + ((pq->gcol + c0) / EM_KG) * TC_M + row;
+      if (e0 > -2000) atomicMax(g, e0);
+      if (e1 > -2000) atomicMax(g + TC_M, e1);
+    }
+  }
+  return ok;
+}
+
 // Row blocks of r rows stacked into one 128-row tile.
 __host__ __device__ inline int em_stack(int r) { return r > 64 ? 1 : TC_M / r; }
 

@@ -109,6 +109,12 @@ cudaError_t launch_aggregate_em(int m, int r, const Desc* d_desc, const int2* wo
 cudaError_t launch_predict(const Desc* d_desc, int M, int r, int nlmax, const PredState& ps, int max_per_leaf,
                            int* status, cudaStream_t s, int64_t* launches, Timer* tm, long nleaf = 0);
 size_t predict_smem_bytes(int r, int nlmax);
+// The same for an emulated handle, on the emulation engine (lb = leaf_bits, the
+// leaves [ps.leaf0, ps.leaf0 + nleaf) whole regions of level M - 1), and whether
+// a prediction takes it.
+bool predict_on_engine(int M, int r, int lb, int max_per_leaf, long nleaf);
+cudaError_t launch_predict_em(const Desc* d_desc, int lb, int nlmax, const PredState& ps, int max_per_leaf, long nleaf,
+                              int* status, cudaStream_t s, int64_t* launches, Timer* tm);
 // Joint posterior predictive (Prop. 2): mode 1 keeps D and the Y_l for the
 // covariance, mode 2 chol(D) and the Y_l for simulation (at most JOINT_TILE
 // points per leaf); then the covariance tiles or the draws.
