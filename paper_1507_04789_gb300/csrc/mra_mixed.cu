@@ -1005,6 +1005,9 @@ __global__ void __launch_bounds__(EM_NT) aggregate_kernel_em(int m, const Desc* 
   __shared__ uint32_t tmem_slot;
   __shared__ int fail;
   __shared__ __align__(16) int rexp[EM_REXP], cexp[EM_CEXP];
+  // row scales per 128-row group of the children's rows: up to 16 children of MAX_R_DEV rows
+  constexpr int AGG_G = 16 * MAX_R_DEV / EM_KG;
+  __shared__ int rsc[AGG_G * TC_M], csc[AGG_G * TC_N];
   int tile;
   const Item it = work_item_tiled(work, nt, tile);
   const Desc& ds = D[it.d];
@@ -1035,12 +1038,12 @@ __global__ void __launch_bounds__(EM_NT) aggregate_kernel_em(int m, const Desc* 
         if (ch * r < (long)(g + 1) * EM_KG && (ch + 1) * r > (long)g * EM_KG)
           e = max(e, st.gcol[m][(cf + ch) * (long)mr + col]);
     }
-    (isA ? rexp : cexp)[u] = e;
+    (isA ? rsc : csc)[u] = e;
   }
   __syncthreads();
   EmAcc acc;
   acc.zero();
-  const bool ok = eng.mma(acc, Gb + k0 * r, 1, mr, nk * r, Gb + l * r, 1, mr, nl * r, K, rexp, TC_M, cexp, TC_N);
+  const bool ok = eng.mma(acc, Gb + k0 * r, 1, mr, nk * r, Gb + l * r, 1, mr, nl * r, K, rsc, TC_M, csc, TC_N);
   const int row = acc.row(), c0 = acc.col0();
   if (ok && row < nk * r) {
     const int k = k0 + row / r, ri = row % r;
