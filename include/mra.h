@@ -69,8 +69,9 @@ extern "C" {
 #define MRA_PREC_FP64     0 /* every step in binary64 */
 #define MRA_PREC_MIXED    1 /* prior chain, leaf covariance and leaf solve products on the
                                tensor cores (tcgen05, 3xTF32 with FP64 accumulation every 64
-                               terms); factorisations, log-determinants, quadratic forms and
-                               the Gram products of the posterior pass in binary64 */
+                               terms); factorisations, log-determinants and quadratic forms
+                               in binary64; the Gram products of the posterior pass in the
+                               FP64-grade emulation below (r > 16 and J_M <= 4, else binary64) */
 #define MRA_PREC_EMU      2 /* every large contraction (prior chain, leaf covariance and solve,
                                leaf and child-to-parent Gram products, posterior G, and in
                                mra_loglik_grad the adjoint's products) on the tensor cores as an

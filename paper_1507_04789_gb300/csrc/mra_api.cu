@@ -147,6 +147,17 @@ int check_config(const mra_config* cfg) {
   return MRA_OK;
 }
 
+// Whether the 3xTF32 form forms its Gram products (leaf_syrk, aggregate) on the
+// emulation engine: they need more than FP32 accuracy, and on the FP64 pipe they
+// took 18.6 of the 39 ms of an evaluation at n = 100003, r = 49.  Not for r <= 16
+// (an FP64 tile takes less than the engine's fixed time), and the engine's leaf
+// Gram kernel holds the column scales of at most four 128-row groups of a
+// parent's observations.
+static bool gram_on_engine(const mra_config& cfg) {
+  const int JM = cfg.J_level[0] ? cfg.J_level[cfg.M > 0 ? cfg.M - 1 : 0] : 4;
+  return cfg.precision == MRA_PREC_MIXED && cfg.M > 0 && cfg.r > 16 && JM <= 4;
+}
+
 // Host tree tables (Sec. 2.2): active regions of every level in region-id order
 // (the per-level child digits; Morton order for the quadtree).
 struct Tables {
@@ -359,6 +370,7 @@ struct mra_handle {
   int64_t scount[MRA_MAX_M + 1][MRA_STAGES] = {};
   int64_t nevals = 0;
   std::vector<int32_t> leaf_counts;   // observations per leaf (Morton order), for mra_stats
+  bool gram_em = false;               // 3xTF32 form: Gram products on the emulation engine (gram_on_engine)
   // emulated form: groups of leaves for the leaf kernel (work item (chunk, first
   // compact leaf), leaf count), per chunk from goff[g]; device copies with room
   // for one group per leaf; lrows = the rows of the kernel's layout (0: none)
@@ -454,6 +466,7 @@ void single_plan(mra_handle* h) {
   p.tile = mra::tile_for_r(h->r);
   p.r = h->r;
   p.mixed = h->cfg.precision == MRA_PREC_MIXED ? 1 : (h->cfg.precision == MRA_PREC_EMU ? 2 : 0);
+  p.gram_em = h->gram_em;
   p.nlmax = h->nlmax;
   for (int m = 0; m < h->M; ++m) {
     p.n_lvl[m] = h->tab.nreg[m];
@@ -708,6 +721,8 @@ int mra_build(const mra_config* cfg, const double* locs, const double* y, int64_
   }
   const std::vector<int32_t>& nreg = h->tab.nreg;
   const bool emu = cfg->precision == MRA_PREC_EMU;
+  h->gram_em = gram_on_engine(*cfg);
+  const bool gram = emu || h->gram_em;   // column scales of H and G for the Gram products
   // ---- subtree streaming: the level s and the chunks (one per level-s region) ----
   int s_lvl = 0;
   if (cfg->stream_level > 0) {
@@ -820,9 +835,9 @@ int mra_build(const mra_config* cfg, const double* locs, const double* y, int64_
     B.want(&h->st.uu[m], (int64_t)nreg[m]);
     if (emu) {
       if (m > 0) B.want(&h->st.vexp[m], R * ((int64_t)(m * r + 127) / 128) * r);
-      if (m > 0) B.want(&h->st.gcol[m], R * (int64_t)m * r);
       B.want(&h->st.liexp[m], R * r);
     }
+    if (gram && m > 0) B.want(&h->st.gcol[m], R * (int64_t)m * r);
   }
   double *H, *z, *LS, *d, *u;
   B.want(&H, obs_cap * (int64_t)M * r);
@@ -831,8 +846,8 @@ int mra_build(const mra_config* cfg, const double* locs, const double* y, int64_
   B.want(&d, nreg[M]);
   B.want(&u, nreg[M]);
   int32_t *hcol = nullptr, *hrow = nullptr;
+  if (gram) B.want(&hcol, cap[M] * (int64_t)M * r);
   if (emu) {
-    B.want(&hcol, cap[M] * (int64_t)M * r);
     B.want(&hrow, obs_cap * (int64_t)((M * r + 127) / 128));
   }
   B.want(&h->d_desc, ndesc);
@@ -975,6 +990,7 @@ int mra_build(const mra_config* cfg, const double* locs, const double* y, int64_
       p.tile = mra::tile_for_r(r);
       p.r = r;
       p.mixed = cfg->precision == MRA_PREC_MIXED ? 1 : (emu ? 2 : 0);
+      p.gram_em = h->gram_em;
       p.nlmax = h->nlmax;
       p.prior_lo = p.post_lo = s_lvl + 1;
       const int2* at[mra::MAXL + 1];
@@ -2119,12 +2135,15 @@ int mra_build_batch(const mra_config* cfgs, const double* const* locs, const dou
                        (e = cudaMemcpy(d_bpc, bpc.data(), sizeof(int) * bpc.size(), cudaMemcpyHostToDevice)))) {
     mra_free(h); return cuda_fail(e, "prior groups");
   }
+  h->gram_em = true;
+  for (int k = 0; k < ndata; ++k) h->gram_em = h->gram_em && gram_on_engine(cfgs[k]);
   mra::Plan& p = h->plan;
   p = mra::Plan();
   p.maxM = maxM;
   p.tile = mra::tile_for_r(h->r);
   p.r = h->r;
   p.mixed = h->cfg.precision == MRA_PREC_MIXED ? 1 : (h->cfg.precision == MRA_PREC_EMU ? 2 : 0);
+  p.gram_em = h->gram_em;
   p.nlmax = h->nlmax;
   int li = 0;
   for (int m = 0; m < maxM; ++m, ++li) { p.n_lvl[m] = lists[li].first; p.w_lvl[m] = d_items + lists[li].second; }

@@ -50,6 +50,7 @@ cudaError_t launch_gather_y(const double* y, const int64_t* perm, int64_t n, dou
 struct Plan {
   int maxM = 0, tile = 64, mixed = 0, nlmax = 1;   // mixed: 0 FP64, 1 3xTF32, 2 FP64 emulation
   int r = 0;
+  bool gram_em = false;   // the Gram products on the emulation engine (always with mixed = 2; see gram_on_engine)
   // the part of the pass this plan runs (subtree streaming splits a pass in
   // three): prior levels [prior_lo, prior_hi), the leaves, and posterior
   // levels [post_lo, post_hi) with the aggregation of each such level m > 0

@@ -494,7 +494,7 @@ cudaError_t launch_loglik(const Plan& pl, const Desc* d_desc, int* status, cudaS
   if (pl.leaves && pl.n_syrk > 0) {
     dim3 grid(pl.n_syrk, pl.t_syrk);
     tm->start(2, s, 3, pl.maxM);
-    if (pl.mixed == 2) {
+    if (pl.mixed == 2 || pl.gram_em) {
       if ((e = launch_leaf_syrk_em(d_desc, pl.w_syrk, pl.n_syrk, pl.maxM, pl.r, status, s))) return e;
     } else {
       MRA_LAUNCH(tile, leaf_syrk_kernel, grid, syrk_smem(tile), s, d_desc, pl.w_syrk);
@@ -516,7 +516,7 @@ cudaError_t launch_loglik(const Plan& pl, const Desc* d_desc, int* status, cudaS
     if (m > 0 && pl.n_agg[m] > 0) {
       dim3 g2(pl.n_agg[m], m * (m + 1) / 2);
       tm->start(4, s, 5, m);
-      if (pl.mixed == 2) {
+      if (pl.mixed == 2 || pl.gram_em) {
         if ((e = launch_aggregate_em(m, pl.r, d_desc, pl.w_agg[m], pl.n_agg[m], status, s))) return e;
       } else {
         MRA_LAUNCH(tile, aggregate_kernel, g2, syrk_smem(tile), s, m, d_desc, pl.w_agg[m]);

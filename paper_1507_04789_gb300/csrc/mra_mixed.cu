@@ -7,8 +7,9 @@
 // the leaf covariance C - V_F V_F' and the leaf solve L_Sigma^{-1} V_F -- on the
 // tensor cores, through one of two engines:
 //  * MRA_PREC_MIXED: tc_mma (3xTF32 with FP64 accumulation every 64 terms);
-//    the Gram products of the posterior pass (leaf_syrk, aggregate) stay in
-//    the FP64 kernels, since they need more than FP32 accuracy;
+//    the Gram products of the posterior pass (leaf_syrk, aggregate) need more
+//    than FP32 accuracy: they run on the emulation engine below (r > 16), else
+//    in the FP64 kernels;
 //  * MRA_PREC_EMU: em_mma (f16-digit FP64 emulation, about 1e-14 relative),
 //    which also runs the two Gram products (leaf_syrk_kernel_em,
 //    aggregate_kernel_em below).
@@ -786,6 +787,13 @@ __global__ void __launch_bounds__(Engine<EMU>::NTH) leaf_kernel_tc(const Desc* _
         }
       }
       __syncthreads();
+    }
+    if (!EMU && lf.hcol && ok) {   // 3xTF32 form: column scales of H_F for its Gram products on the emulation engine
+      for (int c = threadIdx.x; c < Mr; c += NTH) {
+        int e = -2000;
+        for (int i = 0; i < nF; ++i) e = max(e, xexp_of(Hrow[(long)i * Mr + c]));
+        lf.hcol[F * (long)Mr + c] = e;
+      }
     }
     if (EMU && lf.hrow && ok) {   // row scales of H_F per 128-column group (the gradient's Hbar operand)
       const int ng = (Mr + EM_KG - 1) / EM_KG;
