@@ -636,6 +636,24 @@ __device__ __forceinline__ void mma_lower_t(const double* X, long sxi, long sxk,
   }
 }
 
+// f(i, j, sum_{k0 <= k < k1} A(i, k) B(j, k)) for i < na, j < nb, any sizes, in
+// TR-row tiles (16: k0 = lo(first row), k1 = hi(first row + rows) trim the sum to
+// the k a triangular A has in those rows; 64: rows rounded up to 16 per tile).
+template <int TR, int TC, typename LO, typename HI, typename F>
+__device__ __forceinline__ void mma_tiles(const double* A, long sai, long sak, int na, const double* B, long sbj,
+                                          long sbk, int nb, LO&& lo, HI&& hi, double* smem, F&& f) {
+  static_assert(TR == 16 || TR == 64, "row tiles of 16, or of up to 64");
+  for (int r0 = 0; r0 < na; r0 += TR) {
+    const int nr = min(TR, na - r0), k0 = lo(r0), k1 = hi(r0 + nr);
+    for (int c0 = 0; c0 < nb; c0 += TC) {
+      auto g = [&](int i, int j, double v) { f(r0 + i, c0 + j, v); };
+      const double *a = A + r0 * sai + k0 * sak, *b = B + c0 * sbj + k0 * sbk;
+      if constexpr (TR == 16) mma_rows_tile<16, TC>(a, sai, sak, nr, b, sbj, sbk, min(TC, nb - c0), k1 - k0, smem, g);
+      else mma_rows<TC>(a, sai, sak, nr, b, sbj, sbk, min(TC, nb - c0), k1 - k0, smem, g);
+    }
+  }
+}
+
 // f(i, j, sum_k A(i, k) A(j, k)) for j <= i < n: the lower triangle of a Gram
 // product, 16 columns at a time over the rows from their first on.
 template <typename F>

@@ -34,6 +34,11 @@
 
 namespace mra {
 
+template <int V>
+struct IntC {
+  static constexpr int value = V;
+};
+
 template <int TILE>
 __device__ __forceinline__ void store_tile(const TileAcc<TILE>& acc, double* dst, long ld, int nr, int nc,
                                            double scale) {
@@ -71,60 +76,32 @@ __device__ __forceinline__ void lower_inplace(double* Y, int n, long ld) {
 //   global or shared), diag term dlog (adjoint of each log L_ii, 0 if none):
 //   Lbar = lower(-Li' Ybar Li') + dlog / L_ii;  S = sym(Li' Phi(L' Lbar) Li)
 // Result S in B2 (full, symmetric).  B0, B1, B2: n x ld shared buffers.
-template <int TILE>
-__device__ void chol_inverse_adjoint(double* B0, double* B1, double* B2, long ld, int n, const double* L, long ldl,
-                                     const double* Li, long ldi, double dlog, double* stg) {
-  TileAcc<TILE> acc;
-  const int nt = (n + TILE - 1) / TILE;
-  // B1 = Ybar Li'
-  for (int bi = 0; bi < nt; ++bi)
-    for (int bj = 0; bj < nt; ++bj) {
-      acc.zero();
-      tile_mma<TILE>(acc, B0 + bi * TILE * ld, ld, 1, min(TILE, n - bi * TILE), Li + bj * TILE * ldi, ldi, 1,
-                     min(TILE, n - bj * TILE), n, stg);
-      store_tile<TILE>(acc, B1 + bi * TILE * ld + bj * TILE, ld, min(TILE, n - bi * TILE), min(TILE, n - bj * TILE), 1.0);
-    }
+// The products keep to the triangles of their operands and results (16 rows at
+// a time; the terms left out are zeros).
+__device__ inline void chol_inverse_adjoint(double* B0, double* B1, double* B2, long ld, int n, const double* L, long ldl,
+                                            const double* Li, long ldi, double dlog, double* stg) {
+  auto zero = [](int) { return 0; };
+  auto first = [](int r0) { return r0; };
+  auto end = [](int r1) { return r1; };
+  auto all = [&](int) { return n; };
+  // B1 = Ybar Li'   (Ybar lower)
+  mma_tiles<16, 64>(B0, ld, 1, n, Li, ldi, 1, n, zero, end, stg, [&](int i, int j, double v) { B1[i * ld + j] = v; });
   __syncthreads();
   // B2 = lower(-Li' B1) + dlog / L_ii
-  for (int bi = 0; bi < nt; ++bi)
-    for (int bj = 0; bj < nt; ++bj) {
-      acc.zero();
-      tile_mma<TILE>(acc, Li + bi * TILE, 1, ldi, min(TILE, n - bi * TILE), B1 + bj * TILE, 1, ld,
-                     min(TILE, n - bj * TILE), n, stg);
-      store_tile<TILE>(acc, B2 + bi * TILE * ld + bj * TILE, ld, min(TILE, n - bi * TILE), min(TILE, n - bj * TILE), -1.0);
-    }
-  __syncthreads();
-  lower_inplace(B2, n, ld);
-  if (dlog != 0.0)
-    for (int t = threadIdx.x; t < n; t += NT) B2[t * ld + t] += dlog / L[t * ldl + t];
+  mma_tiles<16, 64>(Li, 1, ldi, n, B1, 1, ld, n, first, all, stg, [&](int i, int j, double v) {
+    B2[i * ld + j] = j > i ? 0.0 : (j == i && dlog != 0.0 ? -v + dlog / L[i * ldl + i] : -v);
+  });
   __syncthreads();
   // B0 = Phi(L' B2)
-  for (int bi = 0; bi < nt; ++bi)
-    for (int bj = 0; bj < nt; ++bj) {
-      acc.zero();
-      tile_mma<TILE>(acc, L + bi * TILE, 1, ldl, min(TILE, n - bi * TILE), B2 + bj * TILE, 1, ld,
-                     min(TILE, n - bj * TILE), n, stg);
-      store_tile<TILE>(acc, B0 + bi * TILE * ld + bj * TILE, ld, min(TILE, n - bi * TILE), min(TILE, n - bj * TILE), 1.0);
-    }
+  mma_tiles<16, 64>(L, 1, ldl, n, B2, 1, ld, n, first, all, stg, [&](int i, int j, double v) {
+    B0[i * ld + j] = j > i ? 0.0 : (j == i ? 0.5 * v : v);
+  });
   __syncthreads();
-  phi_inplace(B0, n, ld);
-  // B1 = B0 Li
-  for (int bi = 0; bi < nt; ++bi)
-    for (int bj = 0; bj < nt; ++bj) {
-      acc.zero();
-      tile_mma<TILE>(acc, B0 + bi * TILE * ld, ld, 1, min(TILE, n - bi * TILE), Li + bj * TILE, 1, ldi,
-                     min(TILE, n - bj * TILE), n, stg);
-      store_tile<TILE>(acc, B1 + bi * TILE * ld + bj * TILE, ld, min(TILE, n - bi * TILE), min(TILE, n - bj * TILE), 1.0);
-    }
+  // B1 = B0 Li   (lower)
+  mma_tiles<16, 64>(B0, ld, 1, n, Li, 1, ldi, n, zero, end, stg, [&](int i, int j, double v) { B1[i * ld + j] = v; });
   __syncthreads();
   // B2 = Li' B1, then symmetrise in place
-  for (int bi = 0; bi < nt; ++bi)
-    for (int bj = 0; bj < nt; ++bj) {
-      acc.zero();
-      tile_mma<TILE>(acc, Li + bi * TILE, 1, ldi, min(TILE, n - bi * TILE), B1 + bj * TILE, 1, ld,
-                     min(TILE, n - bj * TILE), n, stg);
-      store_tile<TILE>(acc, B2 + bi * TILE * ld + bj * TILE, ld, min(TILE, n - bi * TILE), min(TILE, n - bj * TILE), 1.0);
-    }
+  mma_tiles<16, 64>(Li, 1, ldi, n, B1, 1, ld, n, first, all, stg, [&](int i, int j, double v) { B2[i * ld + j] = v; });
   __syncthreads();
   for (int t = threadIdx.x; t < n * n; t += NT) {
     int i = t / n, j = t - i * n;
@@ -308,7 +285,7 @@ __global__ void __launch_bounds__(EMU ? EM_NT : NT) post_adjoint_kernel(int m, c
   if (EMU) {
     if (ok) ok = chol_inverse_adjoint_em(cx, B0, B1, B2, ld, r, Ltf, r, Lti, r, -1.0);
   } else {
-    chol_inverse_adjoint<TILE>(B0, B1, B2, ld, r, Ltf, r, Lti, r, -1.0, stg);
+    chol_inverse_adjoint(B0, B1, B2, ld, r, Ltf, r, Lti, r, -1.0, stg);
   }
   double* Ab = gs.Abar[m] + i * (long)r * (mr + r);
   for (int t = threadIdx.x; t < r * r; t += NTH) {
@@ -347,50 +324,38 @@ __global__ void __launch_bounds__(EMU ? EM_NT : NT) post_adjoint_kernel(int m, c
 }
 
 // Hbar = 2 H S_p + z omegabar' of one leaf (nF x M r), S_p read block by block
-// from the ancestors; a leaf of at most 16 observations in one 16-row tile
-// (sparse leaves: no FMA lanes on empty rows).
+// from the ancestors, in tiles of the rows there are (rounded up to 16).
 template <int TILE>
 __device__ void leaf_hbar(const GradState& gs, const long* anc, int M, int r, int nF, const double* H, const double* z,
                           const double* wbar, double* HB, double* stg) {
   const int Mr = M * r;
-  if (TILE > 16 && nF <= 16) {
-    TileAccR<16, TILE> a16;
-    for (int l = 0; l < M; ++l) {
-      a16.zero();
-      for (int k = 0; k < M; ++k) {
-        SRef b = sblock(gs, anc, r, k, l);
-        tile_mma_r<16, TILE>(a16, H + k * r, Mr, 1, nF, b.p, b.sj, b.sk, r, r, stg);
-      }
-#pragma unroll
-      for (int p = 0; p < TileAccR<16, TILE>::RR; ++p)
-#pragma unroll
-        for (int q = 0; q < TileAccR<16, TILE>::RC; ++q) {
-          const int row = a16.row(p), col = a16.col(q);
-          if (row < nF && col < r) HB[(long)row * Mr + l * r + col] = 2.0 * a16.v[p][q] + z[row] * wbar[l * r + col];
+  for (int r0 = 0; r0 < nF; r0 += 64) {
+    const int nr = min(64, nF - r0);
+    auto tile = [&](auto tr) {
+      constexpr int TR = decltype(tr)::value;
+      TileAccR<TR, TILE> acc;
+      for (int l = 0; l < M; ++l) {
+        acc.zero();
+        for (int k = 0; k < M; ++k) {
+          SRef b = sblock(gs, anc, r, k, l);
+          tile_mma_r<TR, TILE>(acc, H + (long)r0 * Mr + k * r, Mr, 1, nr, b.p, b.sj, b.sk, r, r, stg);
         }
-    }
-    return;
-  }
-  TileAcc<TILE> acc;
-  for (int rt = 0; rt < (nF + TILE - 1) / TILE; ++rt) {
-    const int nrow = min(TILE, nF - rt * TILE);
-    for (int l = 0; l < M; ++l) {
-      acc.zero();
-      for (int k = 0; k < M; ++k) {
-        SRef b = sblock(gs, anc, r, k, l);
-        tile_mma<TILE>(acc, H + (long)rt * TILE * Mr + k * r, Mr, 1, nrow, b.p, b.sj, b.sk, r, r, stg);
-      }
 #pragma unroll
-      for (int p = 0; p < TileAcc<TILE>::RM; ++p)
+        for (int p = 0; p < TileAccR<TR, TILE>::RR; ++p)
 #pragma unroll
-        for (int q = 0; q < TileAcc<TILE>::RM; ++q) {
-          int row = acc.row(p), col = acc.col(q);
-          if (row < nrow && col < r) {
-            int o = rt * TILE + row;
-            HB[(long)o * Mr + l * r + col] = 2.0 * acc.v[p][q] + z[o] * wbar[l * r + col];
+          for (int q = 0; q < TileAccR<TR, TILE>::RC; ++q) {
+            const int row = acc.row(p), col = acc.col(q);
+            if (row < nr && col < r) {
+              const int o = r0 + row;
+              HB[(long)o * Mr + l * r + col] = 2.0 * acc.v[p][q] + z[o] * wbar[l * r + col];
+            }
           }
-        }
-    }
+      }
+    };
+    if (nr <= 16) tile(IntC<16>());
+    else if (nr <= 32) tile(IntC<32>());
+    else if (nr <= 48) tile(IntC<48>());
+    else tile(IntC<64>());
   }
 }
 
@@ -499,8 +464,6 @@ __global__ void __launch_bounds__(EMU ? EM_NT : NT) leaf_adjoint_kernel(const De
     double* T1 = gs.T + 3 * lf.sq_off[Fm];     // three nF x nF scratch blocks per leaf
     double* T2 = T1 + (long)nF * nF;
     double* T3 = T2 + (long)nF * nF;
-    const int nrt = (nF + TILE - 1) / TILE;
-    TileAcc<TILE> acc;
     // Hbar = 2 H S_p + z omegabar' (already in HB when em_parts bit 0 is set)
     if constexpr (!EMU)
       if (!(em_parts & 1)) leaf_hbar<TILE>(gs, anc, M, r, nF, H, z, wbar, HB, stg);
@@ -562,13 +525,10 @@ __global__ void __launch_bounds__(EMU ? EM_NT : NT) leaf_adjoint_kernel(const De
           if (ec0 + c < r) out[ec0 + c] = ea.v[c];
       }
     }
-    for (int l = 0; l < M && !EMU; ++l)
-      for (int rt = 0; rt < nrt; ++rt) {
-        const int nrow = min(TILE, nF - rt * TILE);
-        acc.zero();
-        tile_mma<TILE>(acc, LSi + rt * TILE, 1, nF, nrow, HB + l * r, 1, Mr, r, nF, stg);
-        store_tile<TILE>(acc, VB + (long)rt * TILE * Mr + l * r, Mr, nrow, r, 1.0);
-      }
+    if constexpr (!EMU)   // (LSi' is upper triangular: rows i take the observations from i on)
+      for (int l = 0; l < M; ++l)
+        mma_tiles<16, TILE>(LSi, 1, nF, nF, HB + l * r, 1, Mr, r, [](int r0) { return r0; }, [&](int) { return nF; }, stg,
+                            [&](int o, int j, double v) { VB[(long)o * Mr + l * r + j] = v; });
     // LSibar = lower(Hbar V_F' + zbar y')  -> T1
     for (int j0 = 0; j0 < nF && EMU && ok; j0 += TC_N) {
       const int nb = min(TC_N, nF - j0);
@@ -587,28 +547,17 @@ __global__ void __launch_bounds__(EMU ? EM_NT : NT) leaf_adjoint_kernel(const De
         atomicMax(t1_r + erow, e);   // rows of LSibar, the Cholesky adjoint's first operand
       }
     }
-    for (int bi = 0; bi < nrt && !EMU; ++bi)
-      for (int bj = 0; bj <= bi; ++bj) {
-        const int ni = min(TILE, nF - bi * TILE), nj = min(TILE, nF - bj * TILE);
-        acc.zero();
-        tile_mma<TILE>(acc, HB + (long)bi * TILE * Mr, Mr, 1, ni, VF + (long)bj * TILE * Mr, Mr, 1, nj, Mr, stg);
-#pragma unroll
-        for (int p = 0; p < TileAcc<TILE>::RM; ++p)
-#pragma unroll
-          for (int q = 0; q < TileAcc<TILE>::RM; ++q) {
-            int row = acc.row(p), col = acc.col(q);
-            if (row < ni && col < nj) {
-              int oi = bi * TILE + row, oj = bj * TILE + col;
-              T1[(long)oi * nF + oj] = oi >= oj ? acc.v[p][q] + zb[oi] * yv[oj] : 0.0;
-            }
-          }
-        if (bj < bi) {   // zero the mirrored upper block
-          for (int t = threadIdx.x; t < nj * ni; t += NTH) {
-            int a = t / ni, b = t - a * ni;
-            T1[(long)(bj * TILE + a) * nF + bi * TILE + b] = 0.0;
-          }
-        }
-      }
+    if constexpr (!EMU) {
+      for (int t = threadIdx.x; t < nF * nF; t += NTH)
+        if (t % nF > t / nF) T1[t] = 0.0;
+      for (int c0 = 0; c0 < nF; c0 += 16)
+        for (int r0 = c0; r0 < nF; r0 += 64)
+          mma_rows<16>(HB + (long)r0 * Mr, Mr, 1, min(64, nF - r0), VF + (long)c0 * Mr, Mr, 1, min(16, nF - c0), Mr, stg,
+                       [&](int i, int j, double v) {
+                         const int oi = r0 + i, oj = c0 + j;
+                         if (oi >= oj) T1[(long)oi * nF + oj] = v + zb[oi] * yv[oj];
+                       });
+    }
     __syncthreads();
     // Cholesky/inverse adjoint of Sigma_F in the leaf's global scratch: T3 = Sigmabar
     if (EMU) {
@@ -624,7 +573,7 @@ __global__ void __launch_bounds__(EMU ? EM_NT : NT) leaf_adjoint_kernel(const De
         }
       }
     } else {
-      chol_inverse_adjoint<TILE>(T1, T2, T3, nF, nF, LSf, nF, LSi, nF, -1.0, stg);
+      chol_inverse_adjoint(T1, T2, T3, nF, nF, LSf, nF, LSi, nF, -1.0, stg);
     }
     // T3 = Sigmabar (symmetric): C0 and tau2 terms
     for (int t = threadIdx.x; t < nF * nF; t += NTH) {
@@ -647,63 +596,35 @@ __global__ void __launch_bounds__(EMU ? EM_NT : NT) leaf_adjoint_kernel(const De
           if (ec0 + c < r) out[ec0 + c] -= 2.0 * ea.v[c];
       }
     }
-    for (int l = 0; l < M && !EMU; ++l)
-      for (int rt = 0; rt < nrt; ++rt) {
-        const int nrow = min(TILE, nF - rt * TILE);
-        acc.zero();
-        tile_mma<TILE>(acc, T3 + (long)rt * TILE * nF, nF, 1, nrow, VF + l * r, 1, Mr, r, nF, stg);
-#pragma unroll
-        for (int p = 0; p < TileAcc<TILE>::RM; ++p)
-#pragma unroll
-          for (int q = 0; q < TileAcc<TILE>::RM; ++q) {
-            int row = acc.row(p), col = acc.col(q);
-            if (row < nrow && col < r) VB[(long)(rt * TILE + row) * Mr + l * r + col] -= 2.0 * acc.v[p][q];
-          }
-      }
+    if constexpr (!EMU)
+      for (int l = 0; l < M; ++l)
+        mma_tiles<64, TILE>(T3, nF, 1, nF, VF + l * r, 1, Mr, r, [](int) { return 0; }, [&](int) { return nF; }, stg,
+                            [&](int o, int j, double v) { VB[(long)o * Mr + l * r + j] -= 2.0 * v; });
     __syncthreads();
     // chain adjoint, l = M-1..0: Xbar^l = Vbar^l Li_a ; Vbar^k -= Xbar^l V^k_a (k < l)
-    for (int l = M - 1; l >= 0 && !(em_parts & 2); --l) {
+    for (int l = M - 1; l >= 0 && !EMU && !(em_parts & 2); --l) {
       const long a = anc[l];
       const double* Lia = st.Li[l] + a * (long)r * r;
       const double* Va = st.V[l] + a * (long)r * (l * r);
       __syncthreads();
       load_knots<NTH>(sh, l, st.mort[l][a], ax, ay);
       __syncthreads();
-      for (int rt = 0; rt < nrt; ++rt) {
-        const int nrow = min(TILE, nF - rt * TILE);
-        acc.zero();
-        tile_mma<TILE>(acc, VB + (long)rt * TILE * Mr + l * r, Mr, 1, nrow, Lia, 1, r, r, r, stg);
-#pragma unroll
-        for (int p = 0; p < TileAcc<TILE>::RM; ++p)
-#pragma unroll
-          for (int q = 0; q < TileAcc<TILE>::RM; ++q) {
-            int row = acc.row(p), col = acc.col(q);
-            if (row < nrow && col < r) {
-              int o = rt * TILE + row;
-              double xb = acc.v[p][q];
-              XB[(long)o * Mr + l * r + col] = xb;
-              double d1, d2, d3;
-              dcov0(cv, sx[o], sy[o], ax[col], ay[col], d1, d2, d3);
-              g_s2 = fma(xb, d1, g_s2);
-              g_k = fma(xb, d2, g_k);
-              g_nu = fma(xb, d3, g_nu);
-            }
-          }
-      }
+      // (L^{-1} is lower triangular: 16 columns j at a time over k >= j)
+      for (int c0 = 0; c0 < r; c0 += 16)
+        mma_tiles<64, 16>(VB + l * r + c0, Mr, 1, nF, Lia + c0 * r + c0, 1, r, min(16, r - c0), [](int) { return 0; },
+                          [&](int) { return r - c0; }, stg, [&](int o, int j, double xb) {
+          const int col = c0 + j;
+          XB[(long)o * Mr + l * r + col] = xb;
+          double d1, d2, d3;
+          dcov0(cv, sx[o], sy[o], ax[col], ay[col], d1, d2, d3);
+          g_s2 = fma(xb, d1, g_s2);
+          g_k = fma(xb, d2, g_k);
+          g_nu = fma(xb, d3, g_nu);
+        });
       __syncthreads();
       for (int k = 0; k < l; ++k)
-        for (int rt = 0; rt < nrt; ++rt) {
-          const int nrow = min(TILE, nF - rt * TILE);
-          acc.zero();
-          tile_mma<TILE>(acc, XB + (long)rt * TILE * Mr + l * r, Mr, 1, nrow, Va + k * r, 1, l * r, r, r, stg);
-#pragma unroll
-          for (int p = 0; p < TileAcc<TILE>::RM; ++p)
-#pragma unroll
-            for (int q = 0; q < TileAcc<TILE>::RM; ++q) {
-              int row = acc.row(p), col = acc.col(q);
-              if (row < nrow && col < r) VB[(long)(rt * TILE + row) * Mr + k * r + col] -= acc.v[p][q];
-            }
-        }
+        mma_tiles<64, TILE>(XB + l * r, Mr, 1, nF, Va + k * r, 1, l * r, r, [](int) { return 0; }, [&](int) { return r; },
+                            stg, [&](int o, int j, double v) { VB[(long)o * Mr + k * r + j] -= v; });
     }
   }
   if (EMU) em_release(cx);
@@ -856,7 +777,7 @@ __global__ void __launch_bounds__(EMU ? EM_NT : NT) prior_adjoint_kernel(int m, 
   if (EMU) {
     if (ok) ok = chol_inverse_adjoint_em(cx, B0, B1, B2, ld, r, L, r, Li, r, 0.0);   // B2 = Wbar
   } else {
-    chol_inverse_adjoint<TILE>(B0, B1, B2, ld, r, L, r, Li, r, 0.0, stg);
+    chol_inverse_adjoint(B0, B1, B2, ld, r, L, r, Li, r, 0.0, stg);
   }
   for (int t = threadIdx.x; t < r * r; t += NTH) {
     int a = t / r, b = t - a * r;
@@ -1102,7 +1023,7 @@ cudaError_t launch_grad_range(const Desc& hd, const Desc* d_desc, GradState gs, 
   const int M = hd.sh.M;
   const LevelState& st = hd.st;
   cudaError_t e;
-  const size_t stg = sizeof(double) * 2 * KC * (tile + 2);
+  const size_t stg = sizeof(double) * mma_rows_smem(64);
   const size_t sq = sizeof(double) * 3 * MAX_R_DEV * (MAX_R_DEV + 1);
   const int post_hi = R.post_hi < 0 ? M : R.post_hi, prior_hi = R.prior_hi < 0 ? M : R.prior_hi;
   auto base = [&](int m) { return R.count[m] < 0 ? 0L : R.base[m]; };

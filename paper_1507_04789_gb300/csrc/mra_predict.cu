@@ -86,25 +86,12 @@ __global__ void __launch_bounds__(NT) predict_kernel(const Desc* __restrict__ D,
     __syncthreads();
     load_knots(sh, l, st.mort[l][a], ax, ay);
     __syncthreads();
-    acc.zero();
-    if (l > 0) tile_mma_r<TP, TILE>(acc, U, Mr, 1, nP, st.V[l] + a * (long)r * (l * r), l * r, 1, r, l * r, stg);
-#pragma unroll
-    for (int p = 0; p < RR; ++p)
-#pragma unroll
-      for (int q = 0; q < RC; ++q) {
-        int row = acc.row(p), col = acc.col(q);
-        if (row < nP && col < r) U[(long)row * Mr + l * r + col] = cov0(cv, px[row], py[row], ax[col], ay[col]) - acc.v[p][q];
-      }
+    mma_rows<TILE>(U, Mr, 1, nP, st.V[l] + a * (long)r * (l * r), l * r, 1, r, l * r, stg, [&](int row, int col, double v) {
+      U[(long)row * Mr + l * r + col] = cov0(cv, px[row], py[row], ax[col], ay[col]) - v;
+    });
     __syncthreads();
-    acc.zero();
-    tile_mma_r<TP, TILE>(acc, U + l * r, Mr, 1, nP, st.Li[l] + a * (long)r * r, r, 1, r, r, stg);
-#pragma unroll
-    for (int p = 0; p < RR; ++p)
-#pragma unroll
-      for (int q = 0; q < RC; ++q) {
-        int row = acc.row(p), col = acc.col(q);
-        if (row < nP && col < r) U[(long)row * Mr + l * r + col] = acc.v[p][q];
-      }
+    mma_lower_t(U + l * r, Mr, 1, nP, st.Li[l] + a * (long)r * r, r, 1, r, stg,
+                [&](int row, int col, double v) { U[(long)row * Mr + l * r + col] = v; });
   }
   __syncthreads();
   // ---- prior variance v^P = C0(s, s) - |Uhat row|^2 --------------------------
@@ -123,27 +110,21 @@ __global__ void __launch_bounds__(NT) predict_kernel(const Desc* __restrict__ D,
       Cs[i * ldc + k] = cov0(cv, px[i], py[i], lf.xs[o0 + k], lf.ys[o0 + k]);
     }
     __syncthreads();
-    const int nct = (nF + TILE - 1) / TILE;
-    for (int ct = 0; ct < nct; ++ct) {
-      const int ncol = min(TILE, nF - ct * TILE);
-      acc.zero();
-      tile_mma_r<TP, TILE>(acc, Cs, ldc, 1, nP, LS + (long)ct * TILE * nF, nF, 1, ncol, nF, stg);
-      if (M > 0) {
-        TileAccR<TP, TILE> sub;
-        sub.zero();
-        tile_mma_r<TP, TILE>(sub, U, Mr, 1, nP, HF + (long)ct * TILE * Mr, Mr, 1, ncol, Mr, stg);
-#pragma unroll
-        for (int p = 0; p < RR; ++p)
-#pragma unroll
-          for (int q = 0; q < RC; ++q) acc.v[p][q] -= sub.v[p][q];
+    // (L_Sigma^{-1} is lower triangular: 16 columns at a time over the observations they have; then the
+    // columns of Uhat H_F' in tiles as wide as are full, and 16)
+    for (int c0 = 0; c0 < nF; c0 += 16)
+      mma_rows<16>(Cs, ldc, 1, nP, LS + (long)c0 * nF, nF, 1, min(16, nF - c0), min(c0 + 16, nF), stg,
+                   [&](int row, int col, double v) { Ps[row * ldp + c0 + col] = v; });
+    auto sub = [&](int c0, int row, int col, double v) { Ps[row * ldp + c0 + col] -= v; };
+    for (int c0 = 0; c0 < nF && M > 0;) {
+      const double* Hc = HF + (long)c0 * Mr;
+      if (nF - c0 >= TILE) {
+        mma_rows<TILE>(U, Mr, 1, nP, Hc, Mr, 1, TILE, Mr, stg, [&](int i, int j, double v) { sub(c0, i, j, v); });
+        c0 += TILE;
+      } else {
+        mma_rows<16>(U, Mr, 1, nP, Hc, Mr, 1, min(16, nF - c0), Mr, stg, [&](int i, int j, double v) { sub(c0, i, j, v); });
+        c0 += 16;
       }
-#pragma unroll
-      for (int p = 0; p < RR; ++p)
-#pragma unroll
-        for (int q = 0; q < RC; ++q) {
-          int row = acc.row(p), col = acc.col(q);
-          if (row < nP && col < ncol) Ps[row * ldp + ct * TILE + col] = acc.v[p][q];
-        }
     }
     __syncthreads();
     for (int t = threadIdx.x; t < nP; t += NT) {
@@ -189,30 +170,16 @@ __global__ void __launch_bounds__(NT) predict_kernel(const Desc* __restrict__ D,
     __syncthreads();
     // Bhat^{M,k} = Uhat^k - P H^k_F  (in place in U)
     for (int k = 0; k < M; ++k) {
-      acc.zero();
-      tile_mma_r<TP, TILE>(acc, Ps, ldp, 1, nP, HF + k * r, 1, Mr, r, nF, stg);
-#pragma unroll
-      for (int p = 0; p < RR; ++p)
-#pragma unroll
-        for (int q = 0; q < RC; ++q) {
-          int row = acc.row(p), col = acc.col(q);
-          if (row < nP && col < r) U[(long)row * Mr + k * r + col] -= acc.v[p][q];
-        }
+      mma_rows<TILE>(Ps, ldp, 1, nP, HF + k * r, 1, Mr, r, nF, stg,
+                     [&](int row, int col, double v) { U[(long)row * Mr + k * r + col] -= v; });
     }
   }
   // ---- posterior basis recursion, l = M-1..0 -----------------------------------
   for (int l = M - 1; l >= 0; --l) {
     const long a = anc[l];
     __syncthreads();
-    acc.zero();
-    tile_mma_r<TP, TILE>(acc, U + l * r, Mr, 1, nP, st.Lt[l] + a * (long)r * r, r, 1, r, r, stg);
-#pragma unroll
-    for (int p = 0; p < RR; ++p)
-#pragma unroll
-      for (int q = 0; q < RC; ++q) {
-        int row = acc.row(p), col = acc.col(q);
-        if (row < nP && col < r) Ys[row * ldy + col] = acc.v[p][q];
-      }
+    mma_lower_t(U + l * r, Mr, 1, nP, st.Lt[l] + a * (long)r * r, r, 1, r, stg,
+                [&](int row, int col, double v) { Ys[row * ldy + col] = v; });
     __syncthreads();
     const double* g = st.gv[l] + a * r;
     for (int t = threadIdx.x; t < nP; t += NT) {
@@ -232,15 +199,8 @@ __global__ void __launch_bounds__(NT) predict_kernel(const Desc* __restrict__ D,
       }
     const double* Gl = st.G[l] + a * (long)r * (l * r);
     for (int k = 0; k < l; ++k) {
-      acc.zero();
-      tile_mma_r<TP, TILE>(acc, Ys, ldy, 1, nP, Gl + k * r, 1, l * r, r, r, stg);
-#pragma unroll
-      for (int p = 0; p < RR; ++p)
-#pragma unroll
-        for (int q = 0; q < RC; ++q) {
-          int row = acc.row(p), col = acc.col(q);
-          if (row < nP && col < r) U[(long)row * Mr + k * r + col] -= acc.v[p][q];
-        }
+      mma_rows<TILE>(Ys, ldy, 1, nP, Gl + k * r, 1, l * r, r, r, stg,
+                     [&](int row, int col, double v) { U[(long)row * Mr + k * r + col] -= v; });
     }
   }
   __syncthreads();
