@@ -639,6 +639,41 @@ __device__ inline bool em_mma(EmCtx& cx, EmAcc& acc, const double* A, long sai, 
   return ok;
 }
 
+// A thread's N consecutive doubles at p, n of them kept (all: four at a time where
+// p allows).  The 32 lanes of a warp hold 32 rows, so every access touches 32
+// lines: 128 bytes of a row in 4 instructions instead of 16.
+__device__ __forceinline__ bool em_wide(const double* p) {
+  return (reinterpret_cast<uintptr_t>(p) & 31) == 0 && __isGlobal(p);
+}
+template <int N>
+__device__ __forceinline__ void em_get(const double* p, int n, double* v) {
+  if (n >= N && em_wide(p)) {
+#pragma unroll
+    for (int c = 0; c < N; c += 4)
+      asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+                   : "=d"(v[c]), "=d"(v[c + 1]), "=d"(v[c + 2]), "=d"(v[c + 3])
+                   : "l"(p + c)
+                   : "memory");
+  } else {
+#pragma unroll
+    for (int c = 0; c < N; ++c) v[c] = c < n ? p[c] : 0.0;
+  }
+}
+template <int N>
+__device__ __forceinline__ void em_put(double* p, int n, const double* v) {
+  if (n >= N && em_wide(p)) {
+#pragma unroll
+    for (int c = 0; c < N; c += 4)
+      asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p + c), "d"(v[c]), "d"(v[c + 1]), "d"(v[c + 2]),
+                   "d"(v[c + 3])
+                   : "memory");
+  } else {
+#pragma unroll
+    for (int c = 0; c < N; ++c)
+      if (c < n) p[c] = v[c];
+  }
+}
+
 // A product and what becomes of it, for kernels with many products: one call,
 // since inlined at every product the engine's state and the kernel's own crowd
 // each other out of the 128 registers a thread has.
@@ -676,16 +711,17 @@ static __device__ __noinline__ bool em_rows(EmCtx* pcx, const EmRows* pq) {
   if (ok && row < pq->na && c0 < nb) {
     double* const o = pq->out + (long)row * pq->ldo + c0;
     if (pq->sub) {
+      double v[EmAcc::NC];
+      em_get<EmAcc::NC>(o, nb - c0, v);
 #pragma unroll
-      for (int c = 0; c < EmAcc::NC; ++c)
-        if (c0 + c < nb) acc.v[c] = o[c] - acc.v[c];
+      for (int c = 0; c < EmAcc::NC; ++c) acc.v[c] = v[c] - acc.v[c];
     }
+    em_put<EmAcc::NC>(o, nb - c0, acc.v);
     int e0 = -2000, e1 = -2000, ex = -2000;      // a thread's columns touch at most two groups
     const int x0 = pq->xe0 - c0, g0 = EM_KG - ((pq->gcol + c0) & (EM_KG - 1));
 #pragma unroll
     for (int c = 0; c < EmAcc::NC; ++c)
       if (c0 + c < nb) {
-        o[c] = acc.v[c];
         const int e = xexp_of(acc.v[c]);
         if (c < g0) e0 = max(e0, e);
         else e1 = max(e1, e);

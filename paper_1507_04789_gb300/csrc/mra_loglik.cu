@@ -298,9 +298,7 @@ __global__ void __launch_bounds__(EMU ? EM_NT : NT) post_level_kernel(int m, con
       const double* Aml = A + (long)tri_index(m, l) * r * r;
       ok = em_mma(cx, ea, W, ldw, 1, r, Aml, 1, r, r, r);
       if (ok && row < r) {
-#pragma unroll
-        for (int c = 0; c < EmAcc::NC; ++c)
-          if (c0 + c < r) Gr[(long)row * mr + l * r + c0 + c] = ea.v[c];
+        em_put<EmAcc::NC>(Gr + (long)row * mr + l * r + c0, r - c0, ea.v);
       }
     }
   } else {

@@ -194,15 +194,15 @@ __global__ void __launch_bounds__(Engine<EMU>::NTH) prior_level_kernel_tc(int m,
       if (!ok) break;
       if (row < R) {
         int e = -2000;
-        #pragma unroll
+        double* const x = Vrow + (long)row * mr + l * r + c0;
+        double v[NC];
+        em_get<NC>(x, r - c0, v);
+#pragma unroll
         for (int c = 0; c < NC; ++c) {
-          const int col = c0 + c;
-          if (col < r) {
-            const double v = Vrow[(long)row * mr + l * r + col] - acc.v[c];
-            Vrow[(long)row * mr + l * r + col] = v;
-            e = max(e, xexp_of(v));
-          }
+          v[c] -= acc.v[c];
+          if (c0 + c < r) e = max(e, xexp_of(v[c]));
         }
+        em_put<NC>(x, r - c0, v);
         if (EMU) atomicMax(xsc + row, e);
       }
     }
@@ -212,13 +212,13 @@ __global__ void __launch_bounds__(Engine<EMU>::NTH) prior_level_kernel_tc(int m,
                  EMU ? st.liexp[l] + a * r : nullptr, 0);
     if (!ok) break;
     if (row < R) {
+      em_put<NC>(Vrow + (long)row * mr + l * r + c0, r - c0, acc.v);
       int e0 = -2000, e1 = -2000;       // a thread's columns touch at most two groups
       const int gbase = (l * r + c0) / 128;
       #pragma unroll
       for (int c = 0; c < NC; ++c) {
         const int col = c0 + c;
         if (col < r) {
-          Vrow[(long)row * mr + l * r + col] = acc.v[c];
           const int e = xexp_of(acc.v[c]);
           if ((l * r + col) / 128 == gbase) e0 = max(e0, e);
           else e1 = max(e1, e);
@@ -419,15 +419,15 @@ __global__ void __launch_bounds__(EM_NT) chain_forward_kernel_em(const Desc* __r
         if (!ok) break;
         if (row < nr) {
           int e = -2000;
+          double* const x = Hseg + (long)row * Mr + l * r + c0;
+          double v[NC];
+          em_get<NC>(x, r - c0, v);
 #pragma unroll
           for (int c = 0; c < NC; ++c) {
-            const int col = c0 + c;
-            if (col < r) {
-              const double v = Hseg[(long)row * Mr + l * r + col] - acc.v[c];
-              Hseg[(long)row * Mr + l * r + col] = v;
-              e = max(e, xexp_of(v));
-            }
+            v[c] -= acc.v[c];
+            if (c0 + c < r) e = max(e, xexp_of(v[c]));
           }
+          em_put<NC>(x, r - c0, v);
           atomicMax(xsc + ra + row, e);
         }
       }
@@ -437,13 +437,13 @@ __global__ void __launch_bounds__(EM_NT) chain_forward_kernel_em(const Desc* __r
                    st.liexp[l] + a * r, 0);
       if (!ok) break;
       if (row < nr) {
+        em_put<NC>(Hseg + (long)row * Mr + l * r + c0, r - c0, acc.v);
         int e0 = -2000, e1 = -2000;       // a thread's columns touch at most two groups
         const int gbase = (l * r + c0) / 128;
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
           const int col = c0 + c;
           if (col < r) {
-            Hseg[(long)row * Mr + l * r + col] = acc.v[c];
             const int e = xexp_of(acc.v[c]);
             if ((l * r + col) / 128 == gbase) e0 = max(e0, e);
             else e1 = max(e1, e);
@@ -583,15 +583,15 @@ __global__ void __launch_bounds__(Engine<EMU>::NTH) leaf_kernel_tc(const Desc* _
       if (!ok) break;
       if (row < nF) {
         int e = -2000;
-        #pragma unroll
+        double* const x = Hrow + (long)row * Mr + l * r + c0;
+        double v[NC];
+        em_get<NC>(x, r - c0, v);
+#pragma unroll
         for (int c = 0; c < NC; ++c) {
-          const int col = c0 + c;
-          if (col < r) {
-            const double v = Hrow[(long)row * Mr + l * r + col] - acc.v[c];
-            Hrow[(long)row * Mr + l * r + col] = v;
-            e = max(e, xexp_of(v));
-          }
+          v[c] -= acc.v[c];
+          if (c0 + c < r) e = max(e, xexp_of(v[c]));
         }
+        em_put<NC>(x, r - c0, v);
         if (EMU) atomicMax(xsc + row, e);
       }
     }
@@ -601,13 +601,13 @@ __global__ void __launch_bounds__(Engine<EMU>::NTH) leaf_kernel_tc(const Desc* _
                  EMU ? st.liexp[l] + a * r : nullptr, 0);
     if (!ok) break;
     if (row < nF) {
+      em_put<NC>(Hrow + (long)row * Mr + l * r + c0, r - c0, acc.v);
       int e0 = -2000, e1 = -2000;       // a thread's columns touch at most two groups
       const int gbase = (l * r + c0) / 128;
       #pragma unroll
       for (int c = 0; c < NC; ++c) {
         const int col = c0 + c;
         if (col < r) {
-          Hrow[(long)row * Mr + l * r + col] = acc.v[c];
           const int e = xexp_of(acc.v[c]);
           if ((l * r + col) / 128 == gbase) e0 = max(e0, e);
           else e1 = max(e1, e);
@@ -751,13 +751,13 @@ __global__ void __launch_bounds__(Engine<EMU>::NTH) leaf_kernel_tc(const Desc* _
       ok = eng.mma(acc, S, lds, 1, nF, Hrow + cb, 1, Mr, nbc, nF, EMU ? ssc : nullptr, 0);
       if (!ok) break;
       if (row < nF) {
+        em_put<NC>(Hrow + (long)row * Mr + cb + c0, nbc - c0, acc.v);
         int e0 = -2000, e1 = -2000;       // a thread's columns touch at most two groups
         const int gbase = (cb + c0) / 128;
         #pragma unroll
         for (int c = 0; c < NC; ++c) {
           const int col = c0 + c;
           if (col < nbc) {
-            Hrow[(long)row * Mr + cb + col] = acc.v[c];
             const int e = xexp_of(acc.v[c]);
             if ((cb + col) / 128 == gbase) e0 = max(e0, e);
             else e1 = max(e1, e);
@@ -849,6 +849,30 @@ __device__ inline bool em_tile(int t, int nblk, int S, int CB, int& l, int& k0) 
 // at r = 64, two at r = 32, four at r = 16).
 __host__ __device__ inline int em_cblocks(int r) { return r <= 16 ? 4 : (r <= 32 ? 2 : 1); }
 
+// out[a] = sum_{k < K} f(a, k).x f(a, k).y for a < r <= 64, the terms shared out over
+// every thread (a DFMA takes 64 cycles: one thread a column spent 8 us on 256
+// rows, on two of the four FP64 units) and summed in a fixed order; red: NTH
+// doubles of shared memory.  All threads call it; thread a < r writes out[a].
+template <int NTH, typename F>
+__device__ __forceinline__ void em_column_sums(double* red, int r, int K, double* out, F&& f) {
+  const int parts = NTH / r, a = threadIdx.x % r, q = threadIdx.x / r;
+  double s = 0.0;
+  if (q < parts)
+    for (int k = q; k < K; k += parts) {
+      const double2 t = f(a, k);
+      s = fma(t.x, t.y, s);
+    }
+  __syncthreads();
+  red[threadIdx.x] = s;
+  __syncthreads();
+  if (threadIdx.x < r) {
+    double t = 0.0;
+    for (int p = 0; p < parts; ++p) t += red[p * r + threadIdx.x];
+    out[threadIdx.x] = t;
+  }
+  __syncthreads();
+}
+
 // One column block per tile (r > 32).  (A separate kernel: the same body
 // compiled as a branch of the several-block kernel below ran 10 % slower.)
 __global__ void __launch_bounds__(EM_NT) leaf_syrk_kernel_em1(const Desc* __restrict__ D, const int2* __restrict__ work,
@@ -905,18 +929,12 @@ __global__ void __launch_bounds__(EM_NT) leaf_syrk_kernel_em1(const Desc* __rest
   if (ok && row < nk * r) {
     const int k = k0 + row / r, ri = row % r;
     double* out = st.Acc[m] + (p * T + tri_index(k, l)) * (long)r * r + (long)ri * r;
-#pragma unroll
-    for (int c = 0; c < NC; ++c)
-      if (c0 + c < r) out[c0 + c] = acc.v[c];
+    em_put<NC>(out + c0, r - c0, acc.v);
   }
   eng.release();
   if (k0 == l) {
     double* om = st.Om[m] + (p * (m + 1) + l) * (long)r;
-    for (int a = threadIdx.x; a < r; a += NTH) {
-      double s = 0.0;
-      for (long o = 0; o < K; ++o) s = fma(Hb[o * Mr + l * r + a], lf.z[row0 + o], s);
-      om[a] = s;
-    }
+    em_column_sums<NTH>(reinterpret_cast<double*>(dsm), r, K, om, [&](int a, int o) { return make_double2(Hb[(long)o * Mr + l * r + a], lf.z[row0 + o]); });
   }
   if (!ok && threadIdx.x == 0) flag_error(status, ST_TIMEOUT, M - 1, p);
 }
@@ -979,9 +997,7 @@ __global__ void __launch_bounds__(EM_NT) leaf_syrk_kernel_em(const Desc* __restr
     const int k = k0 + row / r, ri = row % r;
     if (!MULTI) {                                     // (r > 32: one column block)
       double* out = st.Acc[m] + (p * T + tri_index(k, l)) * (long)r * r + (long)ri * r;
-#pragma unroll
-      for (int c = 0; c < NC; ++c)
-        if (c0 + c < r) out[c0 + c] = acc.v[c];
+      em_put<NC>(out + c0, r - c0, acc.v);
     } else {
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
@@ -995,11 +1011,7 @@ __global__ void __launch_bounds__(EM_NT) leaf_syrk_kernel_em(const Desc* __restr
   if (k0 == l)
     for (int lb = l; lb < l + nl; ++lb) {
       double* om = st.Om[m] + (p * (m + 1) + lb) * (long)r;
-      for (int a = threadIdx.x; a < r; a += NTH) {
-        double s = 0.0;
-        for (long o = 0; o < K; ++o) s = fma(Hb[o * Mr + lb * r + a], lf.z[row0 + o], s);
-        om[a] = s;
-      }
+      em_column_sums<NTH>(reinterpret_cast<double*>(dsm), r, K, om, [&](int a, int o) { return make_double2(Hb[(long)o * Mr + lb * r + a], lf.z[row0 + o]); });
     }
   if (!ok && threadIdx.x == 0) flag_error(status, ST_TIMEOUT, M - 1, p);
 }
@@ -1058,15 +1070,16 @@ __global__ void __launch_bounds__(EM_NT) aggregate_kernel_em(int m, const Desc* 
     if (!MULTI) {                                     // (r > 32: one column block)
       const int t = tri_index(k, l);
       double* out = st.Acc[m - 1] + (p * Tp + t) * (long)r * r + (long)ri * r;
+      double s[NC];
 #pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        const int col = c0 + c;
-        if (col < r) {
-          double s = -acc.v[c];
-          for (long ch = cf; ch < cf + cc; ++ch) s += st.Acc[m][(ch * Tc + t) * (long)r * r + (long)ri * r + col];
-          out[col] = s;
-        }
+      for (int c = 0; c < NC; ++c) s[c] = -acc.v[c];
+      for (long ch = cf; ch < cf + cc; ++ch) {
+        double a[NC];
+        em_get<NC>(st.Acc[m] + (ch * Tc + t) * (long)r * r + (long)ri * r + c0, r - c0, a);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) s[c] += a[c];
       }
+      em_put<NC>(out + c0, r - c0, s);
     } else {
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
@@ -1084,14 +1097,13 @@ __global__ void __launch_bounds__(EM_NT) aggregate_kernel_em(int m, const Desc* 
   if (k0 == l)
     for (int lb = l; lb < l + nl; ++lb) {
       double* om = st.Om[m - 1] + (p * m + lb) * (long)r;
+      // (the children's rows of G and entries of g are contiguous)
+      em_column_sums<NTH>(reinterpret_cast<double*>(dsm), r, K, om, [&](int a, int q) {
+        return make_double2(-Gb[(long)q * mr + lb * r + a], st.gv[m][cf * r + q]);
+      });
       for (int a = threadIdx.x; a < r; a += NTH) {
-        double s = 0.0;
-        for (long ci = cf; ci < cf + cc; ++ci) {
-          s += st.Om[m][(ci * (m + 1) + lb) * (long)r + a];
-          const double* Gc = st.G[m] + ci * (long)r * mr;
-          const double* gc = st.gv[m] + ci * r;
-          for (int q = 0; q < r; ++q) s = fma(-Gc[(long)q * mr + lb * r + a], gc[q], s);
-        }
+        double s = om[a];
+        for (long ci = cf; ci < cf + cc; ++ci) s += st.Om[m][(ci * (m + 1) + lb) * (long)r + a];
         om[a] = s;
       }
     }
@@ -1291,7 +1303,8 @@ __global__ void __launch_bounds__(EM_NT) hbar_kernel_em(const Desc* __restrict__
       double* out = gs.HB + (t0 + row) * Mr + l * r;
 #pragma unroll
       for (int c = 0; c < NC; ++c)
-        if (c0 + c < r) out[c0 + c] = 2.0 * acc.v[c] + zr * wb[c0 + c];
+        if (c0 + c < r) acc.v[c] = 2.0 * acc.v[c] + zr * wb[c0 + c];
+      em_put<NC>(out + c0, r - c0, acc.v);
     }
   }
   eng.release();
@@ -1338,8 +1351,8 @@ __global__ void __launch_bounds__(EM_NT) leaf_partial_kernel_em(const Desc* __re
     const double sg = diag ? 1.0 : -1.0;
     double* out = gs.PartLeaf + (p * T + tri_index(l, k)) * (long)r * r + (long)i * r;
 #pragma unroll
-    for (int c = 0; c < NC; ++c)
-      if (c0 + c < r) out[c0 + c] = sg * acc.v[c];
+    for (int c = 0; c < NC; ++c) acc.v[c] *= sg;
+    em_put<NC>(out + c0, r - c0, acc.v);
   }
   eng.release();
   if (!ok && threadIdx.x == 0) flag_error(status, ST_TIMEOUT, M - 1, p);
@@ -1427,7 +1440,6 @@ __global__ void __launch_bounds__(EM_NT) chain_adjoint_kernel_em(const Desc* __r
           const int col = c0 + c;
           if (col < r) {
             const double xb = acc.v[c];
-            XB[(long)row * Mr + l * r + col] = xb;
             double d1, d2, d3 = 0.0;
             if (lf.dc) {   // stored by the forward chain kernel (families without d/dnu)
               const double2 dd = *reinterpret_cast<const double2*>(lf.dc + 2 * ((t0 + row) * Mr + l * r + col));
@@ -1441,7 +1453,8 @@ __global__ void __launch_bounds__(EM_NT) chain_adjoint_kernel_em(const Desc* __r
             g_nu = fma(xb, d3, g_nu);
           }
         }
-        int e = -2000;   // row scale of Xbar^l (two threads per row)
+        em_put<NC>(XB + (long)row * Mr + l * r + c0, r - c0, acc.v);
+        int e = -2000;   // row scale of Xbar^l (four threads per row)
 #pragma unroll
         for (int c = 0; c < NC; ++c)
           if (c0 + c < r) e = max(e, xexp_of(acc.v[c]));
@@ -1452,15 +1465,16 @@ __global__ void __launch_bounds__(EM_NT) chain_adjoint_kernel_em(const Desc* __r
         ok = eng.mma(acc, XB + l * r, Mr, 1, na, Va + k * r, 1, l * r, r, r, xbsc, 0,
                      tab ? st.vcol[l] + a * (long)(l * r) + k * r : nullptr, 0);
         if (ok && row < na) {
-          double* out = VB + (long)row * Mr + k * r;
+          double* out = VB + (long)row * Mr + k * r + c0;
           int e = -2000;
+          double v[NC];
+          em_get<NC>(out, r - c0, v);
 #pragma unroll
-          for (int c = 0; c < NC; ++c)
-            if (c0 + c < r) {
-              const double v = out[c0 + c] - acc.v[c];
-              out[c0 + c] = v;
-              e = max(e, xexp_of(v));
-            }
+          for (int c = 0; c < NC; ++c) {
+            v[c] -= acc.v[c];
+            if (c0 + c < r) e = max(e, xexp_of(v[c]));
+          }
+          em_put<NC>(out, r - c0, v);
           if (k == l - 1) atomicMax(vbsc + k * TC_M + row, e);   // the last update of block k
         }
       }
@@ -1574,7 +1588,8 @@ __global__ void __launch_bounds__(EM_NT) gbar_kernel_em(int m, const Desc* __res
       double* out = gs.GB[m] + (t0 + row) * mr + l * r;
 #pragma unroll
       for (int c = 0; c < NC; ++c)
-        if (c0 + c < r) out[c0 + c] = -2.0 * acc.v[c] - gr * wb[c0 + c];
+        if (c0 + c < r) acc.v[c] = -2.0 * acc.v[c] - gr * wb[c0 + c];
+      em_put<NC>(out + c0, r - c0, acc.v);
     }
   }
   eng.release();
