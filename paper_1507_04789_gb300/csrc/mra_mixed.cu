@@ -493,6 +493,7 @@ __global__ void __launch_bounds__(Engine<EMU>::NTH) leaf_kernel_tc(const Desc* _
   __shared__ __align__(16) int rexp[EMU ? EM_REXP : 1], cexp[EMU ? EM_CEXP : 1];
   // emulation: row scales of H rows per 128-column group, of the current X^l block, of L_Sigma^{-1}
   __shared__ int hsc[EMU ? EM_GMAX * TC_M : 1], xsc[EMU ? TC_M : 1], ssc[EMU ? TC_M : 1];
+  __shared__ int vcs[EMU ? EM_GMAX * EM_KG : 1];   // emulation: column scales of V_F over the tile's rows
   const Item it = work_item(work);
   const Desc& ds = D[it.d];
   const Shape sh = ds.sh;
@@ -651,19 +652,27 @@ __global__ void __launch_bounds__(Engine<EMU>::NTH) leaf_kernel_tc(const Desc* _
     }
     S[fi * lds + fj] = v + (fi == fj ? tau2 : 0.0);
   }
+  if (EMU)   // column scales for the products H = L^{-1} V_F below, in one pass instead of one a product
+    for (int c = threadIdx.x; c < Mr; c += NTH) {
+      int e = -2000;
+#pragma unroll 8
+      for (int i = 0; i < nF; ++i) e = max(e, xexp_of(Hrow[(long)i * Mr + c]));
+      vcs[c] = e;
+    }
   __syncthreads();
   const int nct = (nF + TC_N - 1) / TC_N;
-  for (int ct = 0; ct < nct && ok && M > 0; ++ct) {
-    const int ncol = min(TC_N, nF - ct * TC_N);
+  for (int ct = 0; ct < nct && ok && M > 0; ++ct) {   // (the lower triangle: rows from the tile's first column on)
+    const int r0 = ct * TC_N, ncol = min(TC_N, nF - r0);
     acc.zero();
-    ok = eng.mma(acc, Hrow, Mr, 1, nF, Hrow + (long)ct * TC_N * Mr, Mr, 1, ncol, Mr, hsc, TC_M,
-                 hsc + ct * TC_N, TC_M);
+    ok = eng.mma(acc, Hrow + (long)r0 * Mr, Mr, 1, nF - r0, Hrow + (long)r0 * Mr, Mr, 1, ncol, Mr, hsc + r0, TC_M,
+                 hsc + r0, TC_M);
     if (!ok) break;
-    if (row < nF)
+    const int oi = r0 + row;
+    if (oi < nF)
       #pragma unroll
       for (int c = 0; c < NC; ++c) {
-        const int oj = ct * TC_N + c0 + c;
-        if (c0 + c < ncol && oj <= row && (G == 1 || oj >= gseg[growb[row]])) S[row * lds + oj] -= acc.v[c];
+        const int oj = r0 + c0 + c;
+        if (c0 + c < ncol && oj <= oi && (G == 1 || oj >= gseg[growb[oi]])) S[oi * lds + oj] -= acc.v[c];
       }
   }
   double ld = 0.0, zz = 0.0;   // (a group: leaf k's in thread k)
@@ -748,7 +757,7 @@ __global__ void __launch_bounds__(Engine<EMU>::NTH) leaf_kernel_tc(const Desc* _
     for (int cb = 0; cb < Mr && ok; cb += TC_N) {   // 64 columns of H a product (two levels at r = 32)
       const int nbc = min(TC_N, Mr - cb);
       acc.zero();
-      ok = eng.mma(acc, S, lds, 1, nF, Hrow + cb, 1, Mr, nbc, nF, EMU ? ssc : nullptr, 0);
+      ok = eng.mma(acc, S, lds, 1, nF, Hrow + cb, 1, Mr, nbc, nF, EMU ? ssc : nullptr, 0, EMU ? vcs + cb : nullptr, 0);
       if (!ok) break;
       if (row < nF) {
         em_put<NC>(Hrow + (long)row * Mr + cb + c0, nbc - c0, acc.v);
@@ -1125,7 +1134,7 @@ static size_t leaf_tc_smem(int nlmax) {
 }
 // Dynamic plus (an upper bound of) static shared memory of the leaf kernel.
 size_t leaf_tc_smem_bytes(int nlmax, int emu) {
-  return emu ? 1024 + sizeof(int) * (EM_REXP + EM_CEXP + EM_GMAX * TC_M + 2 * TC_M) + leaf_tc_smem<true>(nlmax)
+  return emu ? 1024 + sizeof(int) * (EM_REXP + EM_CEXP + EM_GMAX * TC_M + 2 * TC_M + EM_GMAX * EM_KG) + leaf_tc_smem<true>(nlmax)
              : 1024 + leaf_tc_smem<false>(nlmax);
 }
 
