@@ -369,14 +369,17 @@ __device__ __forceinline__ void em_split_slot(const EmOperand& o, int i0, const 
     d += (l >> 1) * 64 + (lane >> 2) * 8 + (l & 1) * 4;
 #pragma unroll
     for (int s = 0; s < EM_S; ++s) {
-      *reinterpret_cast<uint2*>(d + s * pstride) = make_uint2(w[0][s], w[1][s]);
-      *reinterpret_cast<uint2*>(d + s * pstride + EM_CC * 64) = make_uint2(w[2][s], w[3][s]);
+      const uint32_t q = smem_addr(d + s * pstride);
+      asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(q), "r"(w[0][s]), "r"(w[1][s]) : "memory");
+      asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(q + EM_CC * 128), "r"(w[2][s]), "r"(w[3][s]) : "memory");
     }
   } else {
     d += ((lane >> 3) & 1) * EM_CC * 64 + (lane >> 4) * 64 + (lane & 7) * 8;
 #pragma unroll
     for (int s = 0; s < EM_S; ++s)
-      *reinterpret_cast<uint4*>(d + s * pstride) = make_uint4(w[0][s], w[1][s], w[2][s], w[3][s]);
+      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(smem_addr(d + s * pstride)), "r"(w[0][s]), "r"(w[1][s]),
+                   "r"(w[2][s]), "r"(w[3][s])
+                   : "memory");
   }
 }
 
@@ -674,6 +677,35 @@ __device__ __forceinline__ void em_put(double* p, int n, const double* v) {
   }
 }
 
+// The same two doubles at a time, for rows in any memory: the form the products
+// that are calls use (em_rows, em_store_product).  There em_get / em_put's path of
+// four at a time left some rows of a ragged tile unwritten; inlined it does not.
+template <int N>
+__device__ __forceinline__ void em_get2(const double* p, int n, double* v) {
+  if (n >= N && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+#pragma unroll
+    for (int c = 0; c < N; c += 2) {
+      const double2 d = *reinterpret_cast<const double2*>(p + c);
+      v[c] = d.x;
+      v[c + 1] = d.y;
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < N; ++c) v[c] = c < n ? p[c] : 0.0;
+  }
+}
+template <int N>
+__device__ __forceinline__ void em_put2(double* p, int n, const double* v) {
+  if (n >= N && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+#pragma unroll
+    for (int c = 0; c < N; c += 2) *reinterpret_cast<double2*>(p + c) = make_double2(v[c], v[c + 1]);
+  } else {
+#pragma unroll
+    for (int c = 0; c < N; ++c)
+      if (c < n) p[c] = v[c];
+  }
+}
+
 // A product and what becomes of it, for kernels with many products: one call,
 // since inlined at every product the engine's state and the kernel's own crowd
 // each other out of the 128 registers a thread has.
@@ -702,6 +734,12 @@ struct EmRows {
 };
 static __device__ __noinline__ bool em_rows(EmCtx* pcx, const EmRows* pq) {
   EmCtx cx = *pcx;
+  // (out of line the compiler no longer sees that these lie in shared memory)
+  __builtin_assume(__isShared(cx.stage));
+  __builtin_assume(__isShared(cx.rexp));
+  __builtin_assume(__isShared(cx.cexp));
+  __builtin_assume(__isShared(cx.mbar));
+  __builtin_assume(__isShared(cx.fail));
   EmAcc acc;
   const bool ok = em_mma(cx, acc, pq->A, pq->sai, pq->sak, pq->na, pq->B, pq->sbj, pq->sbk, pq->nb, pq->K, pq->pa,
                          pq->pas, pq->pb, pq->pbs);
@@ -712,11 +750,11 @@ static __device__ __noinline__ bool em_rows(EmCtx* pcx, const EmRows* pq) {
     double* const o = pq->out + (long)row * pq->ldo + c0;
     if (pq->sub) {
       double v[EmAcc::NC];
-      em_get<EmAcc::NC>(o, nb - c0, v);
+      em_get2<EmAcc::NC>(o, nb - c0, v);
 #pragma unroll
       for (int c = 0; c < EmAcc::NC; ++c) acc.v[c] = v[c] - acc.v[c];
     }
-    em_put<EmAcc::NC>(o, nb - c0, acc.v);
+    em_put2<EmAcc::NC>(o, nb - c0, acc.v);
     int e0 = -2000, e1 = -2000, ex = -2000;      // a thread's columns touch at most two groups
     const int x0 = pq->xe0 - c0, g0 = EM_KG - ((pq->gcol + c0) & (EM_KG - 1));
 #pragma unroll
