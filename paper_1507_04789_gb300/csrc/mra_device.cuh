@@ -980,6 +980,16 @@ __device__ __forceinline__ void dcov0(const Cov& c, double x1, double y1, double
   dnu *= gg;
 }
 
+// The same two derivatives for families 0 and 1 with c0_eval's few FP64
+// operations (10 instead of about 35): u the squared scaled distance
+// (c0_scale), sc the variance factor with sigma2, is2 = 1 / sigma2.
+__device__ __forceinline__ void dcov_fast(const Cov& c, double u, double sc, double is2, double& ds2, double& dk) {
+  const C0Val z = c0_eval(c.family, u, sc);
+  const double ea = z.e * z.a * c.ik;
+  ds2 = z.v * is2;
+  dk = c.family == 0 ? ea : ea * z.a;
+}
+
 // C0 at one pair of points (rounded exactly as cov0) and, from the same
 // exponential, dcov0's two derivatives (rounded exactly as dcov0).
 __device__ __forceinline__ double cov0_d(const Cov& c, double x1, double y1, double x2, double y2, double& ds2,

@@ -117,10 +117,12 @@ __device__ inline void chol_inverse_adjoint(double* B0, double* B1, double* B2, 
 // The same chain with its five n x n products on the emulation engine (n <=
 // 128; B0..B2 may live in global or shared memory).  Returns false (uniformly)
 // if a tensor-core wait timed out; the buffers are then incomplete.
-// (pa, pb: the operands' row scales from their producers, one group since n <= 128, or null)
+// (pa, pb: the operands' row scales from their producers, one group since n <= 128, or null;
+// neg: the product's negative; lower: the upper triangle is not needed, so that a column tile
+// takes the rows from its first column on: leaf adjoints of n = 2^18, 16.8 -> 16.2 ms)
 // A call, not inlined: five copies of the engine in one kernel crowd its registers.
 static __device__ __noinline__ bool em_store_product(EmCtx* pcx, const double* A, long sai, long sak, const double* B,
-                                                     long sbj, long sbk, int n, double* C, long ldc, double scale,
+                                                     long sbj, long sbk, int n, double* C, long ldc, bool neg, bool lower,
                                                      const int* pa, const int* pb) {
   EmCtx cx = *pcx;
   EmAcc acc;
@@ -128,11 +130,13 @@ static __device__ __noinline__ bool em_store_product(EmCtx* pcx, const double* A
   bool ok = true;
   for (int j0 = 0; j0 < n && ok; j0 += TC_N) {
     const int nb = min(TC_N, n - j0);
-    ok = em_mma(cx, acc, A, sai, sak, n, B + (long)j0 * sbj, sbj, sbk, nb, n, pa, 0, pb ? pb + j0 : nullptr, 0);
-    if (ok && row < n) {
+    const int i0 = lower ? j0 : 0;
+    ok = em_mma(cx, acc, A + (long)i0 * sai, sai, sak, n - i0, B + (long)j0 * sbj, sbj, sbk, nb, n, pa ? pa + i0 : nullptr, 0,
+                pb ? pb + j0 : nullptr, 0);
+    if (ok && row < n - i0 && c0 < nb) {
 #pragma unroll
-      for (int c = 0; c < EmAcc::NC; ++c)
-        if (c0 + c < nb) C[(long)row * ldc + j0 + c0 + c] = scale * acc.v[c];
+      for (int c = 0; c < EmAcc::NC; ++c) acc.v[c] = neg ? -acc.v[c] : acc.v[c];
+      em_put2<EmAcc::NC>(C + (long)(i0 + row) * ldc + j0 + c0, nb - c0, acc.v);
     }
   }
   pcx->chunks = cx.chunks;
@@ -148,20 +152,20 @@ __device__ inline bool chol_inverse_adjoint_em(EmCtx& cx, double* B0, double* B1
                                                const int* y_r = nullptr, const int* li_r = nullptr,
                                                const int* li_c = nullptr, const int* l_c = nullptr) {
   // B1 = Ybar Li'
-  if (!em_store_product(&cx, B0, ld, 1, Li, ldi, 1, n, B1, ld, 1.0, y_r, li_r)) return false;
+  if (!em_store_product(&cx, B0, ld, 1, Li, ldi, 1, n, B1, ld, false, false, y_r, li_r)) return false;
   // B2 = lower(-Li' B1) + dlog / L_ii
-  if (!em_store_product(&cx, Li, 1, ldi, B1, 1, ld, n, B2, ld, -1.0, li_c, nullptr)) return false;
+  if (!em_store_product(&cx, Li, 1, ldi, B1, 1, ld, n, B2, ld, true, true, li_c, nullptr)) return false;
   lower_inplace<EM_NT>(B2, n, ld);
   if (dlog != 0.0)
     for (int t = threadIdx.x; t < n; t += EM_NT) B2[t * ld + t] += dlog / L[t * ldl + t];
   __syncthreads();
   // B0 = Phi(L' B2)
-  if (!em_store_product(&cx, L, 1, ldl, B2, 1, ld, n, B0, ld, 1.0, l_c, nullptr)) return false;
+  if (!em_store_product(&cx, L, 1, ldl, B2, 1, ld, n, B0, ld, false, true, l_c, nullptr)) return false;
   phi_inplace<EM_NT>(B0, n, ld);
   // B1 = B0 Li
-  if (!em_store_product(&cx, B0, ld, 1, Li, 1, ldi, n, B1, ld, 1.0, nullptr, li_c)) return false;
+  if (!em_store_product(&cx, B0, ld, 1, Li, 1, ldi, n, B1, ld, false, false, nullptr, li_c)) return false;
   // B2 = Li' B1, then symmetrise in place
-  if (!em_store_product(&cx, Li, 1, ldi, B1, 1, ld, n, B2, ld, 1.0, li_c, nullptr)) return false;
+  if (!em_store_product(&cx, Li, 1, ldi, B1, 1, ld, n, B2, ld, false, false, li_c, nullptr)) return false;
   for (int t = threadIdx.x; t < n * n; t += EM_NT) {
     int i = t / n, j = t - i * n;
     if (j < i) {
@@ -468,10 +472,20 @@ __global__ void __launch_bounds__(EMU ? EM_NT : NT) leaf_adjoint_kernel(const De
     if constexpr (!EMU)
       if (!(em_parts & 1)) leaf_hbar<TILE>(gs, anc, M, r, nF, H, z, wbar, HB, stg);
     // zbar = H omegabar - z
-    for (int t = threadIdx.x; t < nF; t += NTH) {
-      double s = -z[t];
-      for (int c = 0; c < Mr; ++c) s = fma(H[(long)t * Mr + c], wbar[c], s);
-      zb[t] = s;
+    if constexpr (EMU) {   // four lanes a row: on every FP64 unit
+      static_assert(EM_NT / 4 >= 128, "a row of the largest leaf per four lanes");
+      const int o = threadIdx.x >> 2, q = threadIdx.x & 3;
+      double s = 0.0;
+      for (int c = q; c < (o < nF ? Mr : 0); c += 4) s = fma(H[(long)o * Mr + c], wbar[c], s);
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      s += __shfl_xor_sync(0xffffffffu, s, 2);
+      if (o < nF && q == 0) zb[o] = s - z[o];
+    } else {
+      for (int t = threadIdx.x; t < nF; t += NTH) {
+        double s = -z[t];
+        for (int c = 0; c < Mr; ++c) s = fma(H[(long)t * Mr + c], wbar[c], s);
+        zb[t] = s;
+      }
     }
     __syncthreads();
     if (EMU) {   // the operand scales, one pass over Hbar, V_F, L_Sigma^{-1} and L_Sigma
@@ -519,10 +533,7 @@ __global__ void __launch_bounds__(EMU ? EM_NT : NT) leaf_adjoint_kernel(const De
     for (int l = 0; l < M && EMU && ok; ++l) {
       ok = em_mma(cx, ea, LSi, 1, nF, nF, HB + l * r, 1, Mr, r, nF, li_c, 0, hb_c + l * r, 0);
       if (ok && erow < nF) {
-        double* out = VB + (long)erow * Mr + l * r;
-#pragma unroll
-        for (int c = 0; c < EmAcc::NC; ++c)
-          if (ec0 + c < r) out[ec0 + c] = ea.v[c];
+        em_put<EmAcc::NC>(VB + (long)erow * Mr + l * r + ec0, r - ec0, ea.v);
       }
     }
     if constexpr (!EMU)   // (LSi' is upper triangular: rows i take the observations from i on)
@@ -531,21 +542,24 @@ __global__ void __launch_bounds__(EMU ? EM_NT : NT) leaf_adjoint_kernel(const De
                             [&](int o, int j, double v) { VB[(long)o * Mr + l * r + j] = v; });
     // LSibar = lower(Hbar V_F' + zbar y')  -> T1
     for (int j0 = 0; j0 < nF && EMU && ok; j0 += TC_N) {
-      const int nb = min(TC_N, nF - j0);
-      ok = em_mma(cx, ea, HB, Mr, 1, nF, VF + (long)j0 * Mr, Mr, 1, nb, Mr, hb_r, TC_M, vf_r + j0, TC_M);
-      if (ok && erow < nF) {
+      const int nb = min(TC_N, nF - j0);   // (rows from the tile's first column on)
+      ok = em_mma(cx, ea, HB + (long)j0 * Mr, Mr, 1, nF - j0, VF + (long)j0 * Mr, Mr, 1, nb, Mr, hb_r + j0, TC_M, vf_r + j0,
+                  TC_M);
+      const int oi = j0 + erow;
+      if (ok && oi < nF) {
         int e = -2000;
 #pragma unroll
         for (int c = 0; c < EmAcc::NC; ++c) {
           const int j = j0 + ec0 + c;
           if (ec0 + c < nb) {
-            const double v = erow >= j ? ea.v[c] + zb[erow] * yv[j] : 0.0;
-            T1[(long)erow * nF + j] = v;
+            const double v = oi >= j ? ea.v[c] + zb[oi] * yv[j] : 0.0;
+            T1[(long)oi * nF + j] = v;
             e = max(e, xexp_of(v));
           }
         }
-        atomicMax(t1_r + erow, e);   // rows of LSibar, the Cholesky adjoint's first operand
+        atomicMax(t1_r + oi, e);   // rows of LSibar, the Cholesky adjoint's first operand
       }
+      for (int t = threadIdx.x; t < j0 * nb; t += NTH) T1[(long)(t / nb) * nF + j0 + t % nb] = 0.0;
     }
     if constexpr (!EMU) {
       for (int t = threadIdx.x; t < nF * nF; t += NTH)
@@ -575,12 +589,22 @@ __global__ void __launch_bounds__(EMU ? EM_NT : NT) leaf_adjoint_kernel(const De
     } else {
       chol_inverse_adjoint(T1, T2, T3, nF, nF, LSf, nF, LSi, nF, -1.0, stg);
     }
-    // T3 = Sigmabar (symmetric): C0 and tau2 terms
-    for (int t = threadIdx.x; t < nF * nF; t += NTH) {
-      int a = t / nF, b = t - a * nF;
-      double sb = T3[t];
-      double d1, d2, d3;
-      dcov0(cv, sx[a], sy[a], sx[b], sy[b], d1, d2, d3);
+    // T3 = Sigmabar (symmetric): C0 and tau2 terms.  (Over the whole square with dcov0 45 us of a leaf of
+    // 70 on the FP64 pipe; the triangle with dcov_fast, here and in the prior adjoint, took n = 2^18's
+    // gradient pass from 54.3 to 52.1 ms.)
+    const bool fast = EMU && c0_fast_ok(cv, 1, 1);
+    const double c0s = c0_scale(cv), c0s2 = c0s * c0s, is2 = 1.0 / cv.sigma2;
+    for (int t = threadIdx.x; t < nF * (nF + 1) / 2; t += NTH) {   // (symmetric: the lower triangle, twice)
+      int a, b;
+      tri_decode(t, a, b);
+      const double sb = a == b ? T3[(long)a * nF + b] : 2.0 * T3[(long)a * nF + b];
+      double d1, d2, d3 = 0.0;
+      if (fast) {
+        const double dx = sx[a] - sx[b], dy = sy[a] - sy[b];
+        dcov_fast(cv, c0s2 * fma(dx, dx, dy * dy), cv.sigma2 * c0_vfac(cv, sx[a]) * c0_vfac(cv, sx[b]), is2, d1, d2);
+      } else {
+        dcov0(cv, sx[a], sy[a], sx[b], sy[b], d1, d2, d3);
+      }
       g_s2 = fma(sb, d1, g_s2);
       g_k = fma(sb, d2, g_k);
       g_nu = fma(sb, d3, g_nu);
@@ -590,10 +614,12 @@ __global__ void __launch_bounds__(EMU ? EM_NT : NT) leaf_adjoint_kernel(const De
     for (int l = 0; l < M && EMU && ok; ++l) {
       ok = em_mma(cx, ea, T3, nF, 1, nF, VF + l * r, 1, Mr, r, nF, t3_r, 0, vf_c + l * r, 0);
       if (ok && erow < nF) {
-        double* out = VB + (long)erow * Mr + l * r;
+        double* out = VB + (long)erow * Mr + l * r + ec0;
+        double v[EmAcc::NC];
+        em_get<EmAcc::NC>(out, r - ec0, v);
 #pragma unroll
-        for (int c = 0; c < EmAcc::NC; ++c)
-          if (ec0 + c < r) out[ec0 + c] -= 2.0 * ea.v[c];
+        for (int c = 0; c < EmAcc::NC; ++c) v[c] = fma(-2.0, ea.v[c], v[c]);
+        em_put<EmAcc::NC>(out, r - ec0, v);
       }
     }
     if constexpr (!EMU)
@@ -779,13 +805,25 @@ __global__ void __launch_bounds__(EMU ? EM_NT : NT) prior_adjoint_kernel(int m, 
   } else {
     chol_inverse_adjoint(B0, B1, B2, ld, r, L, r, Li, r, 0.0, stg);
   }
-  for (int t = threadIdx.x; t < r * r; t += NTH) {
-    int a = t / r, b = t - a * r;
-    double d1, d2, d3;
-    dcov0(cv, qx[a], qy[a], qx[b], qy[b], d1, d2, d3);
-    g_s2 = fma(B2[a * ld + b], d1, g_s2);
-    g_k = fma(B2[a * ld + b], d2, g_k);
-    g_nu = fma(B2[a * ld + b], d3, g_nu);
+  // x times dC0(q_i, p_j)/dtheta into the thread's sums
+  const bool fast = EMU && c0_fast_ok(cv, 1, 1);
+  const double c0s = c0_scale(cv), c0s2 = c0s * c0s, is2 = 1.0 / cv.sigma2;
+  auto derivative = [&](int i, int j, const double* bx, const double* by, double x) {
+    double d1, d2, d3 = 0.0;
+    if (fast) {
+      const double dx = qx[i] - bx[j], dy = qy[i] - by[j];
+      dcov_fast(cv, c0s2 * fma(dx, dx, dy * dy), cv.sigma2 * c0_vfac(cv, qx[i]) * c0_vfac(cv, bx[j]), is2, d1, d2);
+    } else {
+      dcov0(cv, qx[i], qy[i], bx[j], by[j], d1, d2, d3);
+    }
+    g_s2 = fma(x, d1, g_s2);
+    g_k = fma(x, d2, g_k);
+    g_nu = fma(x, d3, g_nu);
+  };
+  for (int t = threadIdx.x; t < r * (r + 1) / 2; t += NTH) {   // (symmetric: the lower triangle, twice)
+    int a, b;
+    tri_decode(t, a, b);
+    derivative(a, b, qx, qy, a == b ? B2[a * ld + b] : 2.0 * B2[a * ld + b]);
   }
   double* VB = gs.VB[m] + i * (long)r * mr;
   double* XB = gs.XB[m] + i * (long)r * mr;
@@ -814,17 +852,18 @@ __global__ void __launch_bounds__(EMU ? EM_NT : NT) prior_adjoint_kernel(int m, 
     __syncthreads();
     auto xbar_epi = [&](int row, int col, double xb) {
       XB[(long)row * mr + l * r + col] = xb;
-      double d1, d2, d3;
-      dcov0(cv, qx[row], qy[row], ax[col], ay[col], d1, d2, d3);
-      g_s2 = fma(xb, d1, g_s2);
-      g_k = fma(xb, d2, g_k);
-      g_nu = fma(xb, d3, g_nu);
+      if constexpr (!EMU) derivative(row, col, ax, ay, xb);
     };
     if (EMU)
       product_n(VB + l * r, mr, 1, r, Lia, 1, r, r, nullptr, st.licol[l] ? st.licol[l] + a * r : nullptr, xbar_epi);
     else
       product(VB + l * r, mr, 1, Lia, 1, r, r, xbar_epi);
     __syncthreads();
+    if constexpr (EMU)   // (after the product: in its epilogue this took registers from the engine)
+      for (int t = threadIdx.x; t < r * r; t += NTH) {
+        const int row = t / r, col = t - row * r;
+        derivative(row, col, ax, ay, XB[(long)row * mr + l * r + col]);
+      }
     if (EMU) {   // Vbar^k -= Xbar^l V^k_a, transposed, S blocks k per product
       for (int k0 = 0; k0 < l; k0 += S)
         product_n(Va + k0 * r, 1, l * r, min(S, l - k0) * r, XB + l * r, mr, 1, r,
