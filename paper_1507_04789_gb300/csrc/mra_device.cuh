@@ -612,13 +612,15 @@ __device__ __forceinline__ void mma_rows_tile(const double* A, long sai, long sa
       if (row < na && col < nb) f(row, col, acc.v[p][q]);
     }
 }
-template <int TC, typename F>
+// (RMAX: the most rows the caller has; the wider tiles would only cost the kernel registers)
+template <int TC, int RMAX = 64, typename F>
 __device__ __forceinline__ void mma_rows(const double* A, long sai, long sak, int na, const double* B, long sbj,
                                          long sbk, int nb, int K, double* smem, F&& f) {
-  if (na <= 16) mma_rows_tile<16, TC>(A, sai, sak, na, B, sbj, sbk, nb, K, smem, f);
-  else if (na <= 32) mma_rows_tile<32, TC>(A, sai, sak, na, B, sbj, sbk, nb, K, smem, f);
-  else if (na <= 48) mma_rows_tile<48, TC>(A, sai, sak, na, B, sbj, sbk, nb, K, smem, f);
-  else mma_rows_tile<64, TC>(A, sai, sak, na, B, sbj, sbk, nb, K, smem, f);
+  static_assert(RMAX == 16 || RMAX == 32 || RMAX == 64, "rows of a tile");
+  if (RMAX == 16 || na <= 16) mma_rows_tile<16, TC>(A, sai, sak, na, B, sbj, sbk, nb, K, smem, f);
+  else if (RMAX == 32 || na <= 32) mma_rows_tile<RMAX == 16 ? 16 : 32, TC>(A, sai, sak, na, B, sbj, sbk, nb, K, smem, f);
+  else if (na <= 48) mma_rows_tile<RMAX == 64 ? 48 : 16, TC>(A, sai, sak, na, B, sbj, sbk, nb, K, smem, f);
+  else mma_rows_tile<RMAX == 64 ? 64 : 16, TC>(A, sai, sak, na, B, sbj, sbk, nb, K, smem, f);
 }
 constexpr int mma_rows_smem(int tc) { return KC * (64 + 2 + tc + 2); }
 
@@ -626,12 +628,12 @@ constexpr int mma_rows_smem(int tc) { return KC * (64 + 2 + tc + 2); }
 // triangular (L(j, k) = 0 for k > j): 16 columns at a time over the k they have,
 // 5/8 of the full product at n = 64.  The columns are taken from the last, so f
 // may overwrite X(i, j): the columns still to come read X(., k <= j) only.
-template <typename F>
+template <int RMAX = 64, typename F>
 __device__ __forceinline__ void mma_lower_t(const double* X, long sxi, long sxk, int na, const double* L, long slj,
                                             long slk, int n, double* smem, F&& f) {
   for (int c0 = ((n - 1) >> 4) << 4; c0 >= 0; c0 -= 16) {
     const int nb = min(16, n - c0);
-    mma_rows<16>(X, sxi, sxk, na, L + c0 * slj, slj, slk, nb, c0 + nb, smem,
+    mma_rows<16, RMAX>(X, sxi, sxk, na, L + c0 * slj, slj, slk, nb, c0 + nb, smem,
                  [&](int i, int j, double v) { f(i, c0 + j, v); });
   }
 }

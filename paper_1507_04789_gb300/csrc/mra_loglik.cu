@@ -505,7 +505,7 @@ cudaError_t launch_loglik(const Plan& pl, const Desc* d_desc, int* status, cudaS
     if (pl.n_lvl[m] > 0) {
       tm->start(3, s, 4, m);
       // (the emulated form's G = Lt^{-1} Ahat products have K = r: at r <= 32 the engine's fixed cost per
-      // product exceeds the FP64 tile product, measured 208 against 104 ms on the ragged batch)
+      // product exceeds the FP64 tile product: 21.5 against 12.5 ms on 16 datasets of 1.2M observations, r = 32)
       if ((e = launch_post_level(pl.mixed == 2 && pl.r > 32, tile, m, pl.n_lvl[m], s, d_desc, pl.w_lvl[m], status)))
         return e;
       tm->stop(s);

@@ -33,8 +33,9 @@ namespace mra {
 // one CTA holds all points of its leaf (at most TILE).  TP: the points of one
 // CTA (TILE, or 16 in mode 0 where leaves hold few points): the products are
 // TP x TILE tiles, the TILE columns covering the r knots of a block.
+// Three CTAs an SM for the small tiles: few points a leaf leave latency, not work.
 template <int TP, int TILE, int MODE>
-__global__ void __launch_bounds__(NT) predict_kernel(const Desc* __restrict__ D, PredState ps, int* status) {
+__global__ void __launch_bounds__(NT, TP <= 32 && TILE <= 32 ? 3 : 2) predict_kernel(const Desc* __restrict__ D, PredState ps, int* status) {
   static_assert(MODE == 0 || TP == TILE, "the joint modes take whole leaves in square tiles");
   extern __shared__ double smem[];
   const Desc& ds = D[ps.desc];
@@ -78,6 +79,14 @@ __global__ void __launch_bounds__(NT) predict_kernel(const Desc* __restrict__ D,
   }
   __syncthreads();
   double* U = ps.U + p0 * Mr;                   // nP x (M r), row-major
+  // Few points a leaf (16-row tiles of 64 columns) leave the latency of the staged steps, not FP64 work: full
+  // column tiles then, where a triangular operand otherwise takes 16 columns at a time over the k they have
+  // (1000 points at n = 100,000, r = 64: 5.7 ms full, 6.6 ms by 16).
+  constexpr bool FEW = TP == 16 && TILE == 64;
+  auto lower_t = [&](const double* X, long ldx, const double* L, auto&& f) {
+    if constexpr (FEW) mma_rows<TILE, TP>(X, ldx, 1, nP, L, r, 1, r, r, stg, f);
+    else mma_lower_t<TP>(X, ldx, 1, nP, L, r, 1, r, stg, f);
+  };
   TileAccR<TP, TILE> acc;
   constexpr int RR = TileAccR<TP, TILE>::RR, RC = TileAccR<TP, TILE>::RC;
   // ---- Uhat chain (same recursion as the leaf basis) --------------------------
@@ -86,12 +95,12 @@ __global__ void __launch_bounds__(NT) predict_kernel(const Desc* __restrict__ D,
     __syncthreads();
     load_knots(sh, l, st.mort[l][a], ax, ay);
     __syncthreads();
-    mma_rows<TILE>(U, Mr, 1, nP, st.V[l] + a * (long)r * (l * r), l * r, 1, r, l * r, stg, [&](int row, int col, double v) {
+    mma_rows<TILE, TP>(U, Mr, 1, nP, st.V[l] + a * (long)r * (l * r), l * r, 1, r, l * r, stg, [&](int row, int col, double v) {
       U[(long)row * Mr + l * r + col] = cov0(cv, px[row], py[row], ax[col], ay[col]) - v;
     });
     __syncthreads();
-    mma_lower_t(U + l * r, Mr, 1, nP, st.Li[l] + a * (long)r * r, r, 1, r, stg,
-                [&](int row, int col, double v) { U[(long)row * Mr + l * r + col] = v; });
+    lower_t(U + l * r, Mr, st.Li[l] + a * (long)r * r,
+            [&](int row, int col, double v) { U[(long)row * Mr + l * r + col] = v; });
   }
   __syncthreads();
   // ---- prior variance v^P = C0(s, s) - |Uhat row|^2 --------------------------
@@ -112,17 +121,20 @@ __global__ void __launch_bounds__(NT) predict_kernel(const Desc* __restrict__ D,
     __syncthreads();
     // (L_Sigma^{-1} is lower triangular: 16 columns at a time over the observations they have; then the
     // columns of Uhat H_F' in tiles as wide as are full, and 16)
-    for (int c0 = 0; c0 < nF; c0 += 16)
-      mma_rows<16>(Cs, ldc, 1, nP, LS + (long)c0 * nF, nF, 1, min(16, nF - c0), min(c0 + 16, nF), stg,
+    for (int c0 = 0; FEW && c0 < nF; c0 += TILE)
+      mma_rows<TILE, TP>(Cs, ldc, 1, nP, LS + (long)c0 * nF, nF, 1, min(TILE, nF - c0), min(c0 + TILE, nF), stg,
+                         [&](int row, int col, double v) { Ps[row * ldp + c0 + col] = v; });
+    for (int c0 = 0; !FEW && c0 < nF; c0 += 16)
+      mma_rows<16, TP>(Cs, ldc, 1, nP, LS + (long)c0 * nF, nF, 1, min(16, nF - c0), min(c0 + 16, nF), stg,
                    [&](int row, int col, double v) { Ps[row * ldp + c0 + col] = v; });
     auto sub = [&](int c0, int row, int col, double v) { Ps[row * ldp + c0 + col] -= v; };
     for (int c0 = 0; c0 < nF && M > 0;) {
       const double* Hc = HF + (long)c0 * Mr;
-      if (nF - c0 >= TILE) {
-        mma_rows<TILE>(U, Mr, 1, nP, Hc, Mr, 1, TILE, Mr, stg, [&](int i, int j, double v) { sub(c0, i, j, v); });
+      if (FEW || nF - c0 >= TILE) {
+        mma_rows<TILE, TP>(U, Mr, 1, nP, Hc, Mr, 1, min(TILE, nF - c0), Mr, stg, [&](int i, int j, double v) { sub(c0, i, j, v); });
         c0 += TILE;
       } else {
-        mma_rows<16>(U, Mr, 1, nP, Hc, Mr, 1, min(16, nF - c0), Mr, stg, [&](int i, int j, double v) { sub(c0, i, j, v); });
+        mma_rows<16, TP>(U, Mr, 1, nP, Hc, Mr, 1, min(16, nF - c0), Mr, stg, [&](int i, int j, double v) { sub(c0, i, j, v); });
         c0 += 16;
       }
     }
@@ -170,7 +182,7 @@ __global__ void __launch_bounds__(NT) predict_kernel(const Desc* __restrict__ D,
     __syncthreads();
     // Bhat^{M,k} = Uhat^k - P H^k_F  (in place in U)
     for (int k = 0; k < M; ++k) {
-      mma_rows<TILE>(Ps, ldp, 1, nP, HF + k * r, 1, Mr, r, nF, stg,
+      mma_rows<TILE, TP>(Ps, ldp, 1, nP, HF + k * r, 1, Mr, r, nF, stg,
                      [&](int row, int col, double v) { U[(long)row * Mr + k * r + col] -= v; });
     }
   }
@@ -178,8 +190,7 @@ __global__ void __launch_bounds__(NT) predict_kernel(const Desc* __restrict__ D,
   for (int l = M - 1; l >= 0; --l) {
     const long a = anc[l];
     __syncthreads();
-    mma_lower_t(U + l * r, Mr, 1, nP, st.Lt[l] + a * (long)r * r, r, 1, r, stg,
-                [&](int row, int col, double v) { Ys[row * ldy + col] = v; });
+    lower_t(U + l * r, Mr, st.Lt[l] + a * (long)r * r, [&](int row, int col, double v) { Ys[row * ldy + col] = v; });
     __syncthreads();
     const double* g = st.gv[l] + a * r;
     for (int t = threadIdx.x; t < nP; t += NT) {
@@ -199,7 +210,7 @@ __global__ void __launch_bounds__(NT) predict_kernel(const Desc* __restrict__ D,
       }
     const double* Gl = st.G[l] + a * (long)r * (l * r);
     for (int k = 0; k < l; ++k) {
-      mma_rows<TILE>(Ys, ldy, 1, nP, Gl + k * r, 1, l * r, r, r, stg,
+      mma_rows<TILE, TP>(Ys, ldy, 1, nP, Gl + k * r, 1, l * r, r, r, stg,
                      [&](int row, int col, double v) { U[(long)row * Mr + k * r + col] -= v; });
     }
   }
