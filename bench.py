@@ -11,7 +11,7 @@ observations per leaf).  Three forms are timed on the same steps:
   fp64   every product on the FP64 pipe
   mixed  prior and leaf contractions on the tensor cores as 3xTF32
   emu    every large contraction (prior, leaf and both Gram products) on the
-         tensor cores as a bf16-slice FP64 emulation (about 1e-14 per product)
+         tensor cores as a f16-digit FP64 emulation (below 1e-14 per product)
 
 The headline is the fastest form whose log-likelihoods stay within
 |d loglik| / n <= 1e-6 of the FP64 form; the others are reported beside it,
@@ -24,7 +24,7 @@ FP64 emulation, beside the FP64 form). `--grad-only` times only the emulated log
                copies locations and data from pinned host memory, re-partitions
                them on the device and reads the result back
   roofline     the dominant kernel of the headline form: for a tensor-core
-               kernel, the bf16 (emu) or TF32 (mixed) tensor FLOP/s its
+               kernel, the f16 (emu) or TF32 (mixed) tensor FLOP/s its
                contractions need (algorithmic FP64 MACs x slice products) over
                its CUDA-event time, against the measured bf16 peak (TF32 at the
                nominal TF32/bf16 ratio); for an FP64 kernel, algorithmic FP64
@@ -64,7 +64,7 @@ WORKLOAD = "n1M_matern15_M7_r64"
 FP64_PEAK_TFLOPS = 1.10     # GB300 FP64 pipe, measured: DMMA m8n8k4 1.103, DFMA 1.059 TFLOP/s (tests/peaks.cu)
 BF16_PEAK_FALLBACK = 1900.0  # TFLOP/s, used only without a measured peak file
 TF32_PER_BF16 = 1.1 / 2.25   # nominal dense TF32 / bf16 tensor rates
-EMU_PAIRS = 28               # bf16 slice products per emulated FP64 MAC (7 slices, weights t <= 8)
+EMU_PAIRS = 26               # f16 digit products per emulated FP64 MAC (6 digits, weights p + q <= 8)
 TF32_PAIRS = 3               # TF32 products per 3xTF32 MAC
 ORACLE_SAMPLE_LEVEL = 3     # cpu baseline: level-3 subtrees, 1/64 of the leaves each
 
@@ -435,13 +435,13 @@ def run_batch(args, world, rank, mra, np, torch):
 
 
 # Stages whose contractions run on the tensor cores in each form (the others on the FP64 pipe).
-TENSOR_STAGES = {"fp64": set(), "mixed": {"prior", "leaf"},
+TENSOR_STAGES = {"fp64": set(), "mixed": {"prior", "leaf", "leaf_syrk", "aggregate"},
                  "emu": {"prior", "chain", "leaf", "leaf_syrk", "post", "aggregate"}}
 STAGE_KERNEL = {
     "fp64": {"prior": "prior_level_kernel", "leaf": "leaf_kernel", "leaf_syrk": "leaf_syrk_kernel",
              "post": "post_level_kernel", "aggregate": "aggregate_kernel"},
-    "mixed": {"prior": "prior_level_kernel_tc<0>", "leaf": "leaf_kernel_tc<0>", "leaf_syrk": "leaf_syrk_kernel",
-              "post": "post_level_kernel", "aggregate": "aggregate_kernel"},
+    "mixed": {"prior": "prior_level_kernel_tc<0>", "leaf": "leaf_kernel_tc<0>",
+              "leaf_syrk": "leaf_syrk_kernel_em", "post": "post_level_kernel", "aggregate": "aggregate_kernel_em"},
     "emu": {"prior": "prior_level_kernel_tc<1>", "chain": "chain_forward_kernel_em", "leaf": "leaf_kernel_tc<1>",
             "leaf_syrk": "leaf_syrk_kernel_em", "post": "post_level_kernel<EMU>", "aggregate": "aggregate_kernel_em"},
 }
@@ -476,7 +476,6 @@ def level_table(st, prec, M, r, nF, bf16_peak, hbm_peak):
     """Per level and stage of one form: time per evaluation, algorithmic FLOPs and
     bytes (mra_stats), their rates and the fraction of the pipe's peak."""
     ev = max(1, st["evaluations"])
-    pairs = EMU_PAIRS if prec == "emu" else TF32_PAIRS
     rows = []
     for m, row in enumerate(st["levels"]):
         for stage, v in row.items():
@@ -484,7 +483,8 @@ def level_table(st, prec, M, r, nF, bf16_peak, hbm_peak):
                 continue
             sec = v["ms"] / ev * 1e-3
             tensor = stage in TENSOR_STAGES[prec] or (prec == "mixed" and stage == "chain")
-            peak = bf16_peak * (1.0 if prec == "emu" else TF32_PER_BF16) if tensor else FP64_PEAK_TFLOPS
+            engine = prec == "emu" or stage in ("leaf_syrk", "aggregate")   # (the mixed form's Gram products too)
+            peak = bf16_peak * (1.0 if engine else TF32_PER_BF16) if tensor else FP64_PEAK_TFLOPS
             alg = v["flops"] / sec / 1e12
             out = {"level": m, "stage": stage, "kernel": STAGE_KERNEL[prec].get(stage, stage),
                    "ms_per_step": v["ms"] / ev, "launches_per_step": v["launches"] / ev, "units": v["units"],
@@ -492,8 +492,9 @@ def level_table(st, prec, M, r, nF, bf16_peak, hbm_peak):
                    "pipe": "tensor" if tensor else "alu", "peak": peak, "frac": alg / peak,
                    "hbm_gbs": v["bytes"] / sec / 1e9, "hbm_frac": v["bytes"] / sec / 1e9 / hbm_peak,
                    "per_unit": ("algorithmic FP64 FLOPs (mra_stats) of the level's units"
-                                + (" against the bf16 tensor peak" if tensor and prec == "emu" else ""))}
+                                + (" against the bf16 tensor peak" if tensor and engine else ""))}
             if tensor:
+                pairs = EMU_PAIRS if engine else TF32_PAIRS
                 eng = pairs * contraction_share(stage, m, M, r, nF) / sec / 1e12
                 out["engine_tflops"] = eng
                 out["engine_frac"] = eng / peak
@@ -667,7 +668,7 @@ def run_sharded(args, rank, world, local, mra, np, torch):
         print(json.dumps({
             "metric": METRIC, "value": 1e3 / ms, "unit": "evals/s", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "strong",
-            "vs_baseline": None, "dtype": "f64+bf16x7 (emulated f64)", "data": "synthetic",
+            "vs_baseline": None, "dtype": "f64+f16x6 (emulated f64)", "data": "synthetic",
             "config": {"workload": w.name, "n": w.n, "M": w.M, "r": w.r, "family": w.family,
                        "parallelism": f"level-2 subtrees sharded over {world} ranks, one all-gather of "
                                       f"{nsub} x {length} doubles per evaluation",
@@ -754,7 +755,7 @@ def run_large(args, mra, np, torch):
     line = {
         "metric": f"M-RA loglik evals/s at n=2^24 swath field (M={w.M}, r={w.r}), streamed level-s subtrees",
         "value": 1e3 / ms, "unit": "evals/s", "ms_per_step": ms, "steps": args.steps, "warmup": args.warmup,
-        "higher_is_better": True, "dtype": "f64+bf16x7 (emulated f64)", "data": "synthetic",
+        "higher_is_better": True, "dtype": "f64+f16x6 (emulated f64)", "data": "synthetic",
         "config": {"workload": w.name, "n": w.n, "M": w.M, "r": w.r, "family": w.family, "nonstat": w.nonstat,
                    "sigma2": w.sigma2, "range": w.kappa, "tau2": w.tau2, "stream_level": args.stream_level,
                    "tree": "complete (every region, so that every grid point has its ancestors)",
@@ -1048,7 +1049,7 @@ def main():
     level_J = run_level_J(args, mra, np, torch, stream, locs, y, w, thetas)
 
     if rank == 0:
-        dtypes = {"fp64": "f64", "mixed": "f64+tf32x3", "emu": "f64+bf16x7 (emulated f64)"}
+        dtypes = {"fp64": "f64", "mixed": "f64+tf32x3", "emu": "f64+f16x6 (emulated f64)"}
 
         def form_line(p):
             out = {"value": forms[p]["value"], "ms_per_step": forms[p]["ms_per_step"], "kernels": kernel_table(p),

@@ -75,9 +75,9 @@ extern "C" {
 #define MRA_PREC_EMU      2 /* every large contraction (prior chain, leaf covariance and solve,
                                leaf and child-to-parent Gram products, posterior G, and in
                                mra_loglik_grad the adjoint's products) on the tensor cores as an
-                               FP64-grade emulation: operands cut into seven 7-bit bf16 slices
+                               FP64-grade emulation: operands cut into six 8-bit f16 digits
                                per 128-column group, exact FP32 accumulation, double-float sums
-                               (about 1e-14 relative error per product); factorisations and
+                               (below 1e-14 relative error per product); factorisations and
                                the rest in binary64 */
 
 #define MRA_HOST          0 /* pointer argument is host memory */

@@ -92,7 +92,7 @@ cudaError_t launch_gather_roots(const Desc* d_desc, int nd, double* out, cudaStr
 size_t leaf_smem_bytes(int r, int nlmax);
 
 // Mixed-precision prior level and leaf pass (tensor cores, mra_mixed.cu).
-// emu = 1: FP64-grade bf16-slice emulation engine; 0: 3xTF32.
+// emu = 1: FP64-grade f16-digit emulation engine; 0: 3xTF32.
 cudaError_t launch_prior_tc(int m, const Desc* d_desc, const int2* work, int nblocks, int emu, int* status,
                             cudaStream_t s, const int* gcnt = nullptr, int rcap = 0);
 cudaError_t launch_leaf_tc(const Desc* d_desc, const int2* work, int nblocks, int nlmax, int emu, int* status,

@@ -2,7 +2,8 @@
 // with the products on the emulation engine, for handles of MRA_PREC_EMU.
 //
 // The same quantities as predict_kernel (mra_predict.cu), whose 2^18 points at
-// n = 2^18, r = 64 take 121 ms of the FP64 pipe (0.86 of its 1.06 TFLOP/s).  One
+// n = 2^18, r = 64 take 121 ms of the FP64 pipe (0.86 of its 1.06 TFLOP/s) and
+// 29 ms here, where the digit splitting (integer pipe) bounds the products.  One
 // CTA takes up to 128 points of one level-(M-1) region: the chain and the
 // posterior recursion read the region's ancestors, which its leaves share, as
 // one 128-row product per block; only the leaf term goes leaf by leaf.
@@ -252,7 +253,7 @@ static size_t predict_em_smem(int nlmax) {
 
 // Whether the marginal prediction of an emulated handle runs on the engine: a
 // 16-row FP64 tile of r <= 16 knots costs less than the engine's fixed time a
-// product (about 7 us; measured, see the launcher), and the flat grid is 31 bits.
+// product (about 7 us), and the flat grid is 31 bits.
 bool predict_on_engine(int M, int r, int lb, int max_per_leaf, long nleaf) {
   if (M < 1 || r <= 16 || max_per_leaf <= 0) return false;
   const long tiles = (((long)max_per_leaf << lb) + TC_M - 1) / TC_M;
