@@ -1805,8 +1805,11 @@ int mra_predict(mra_handle* h, const mra_params* theta, const double* plocs, int
   ps.mean = where == MRA_DEVICE ? mean_out : h->p_mean;
   ps.var = where == MRA_DEVICE ? var_out : h->p_var;
   const int lb = M > 0 ? mra::leaf_bits(h->hd.sh) : 0;
+  // (decided for the whole tree, so that a streamed handle's chunks take its kernel)
+  const bool engine = h->cfg.precision == MRA_PREC_EMU &&
+                      mra::predict_on_engine(M, r, lb, maxp, ps.nleaves, (double)np / (double)ps.nleaves);
   auto launch = [&](long nleaf) {                // the points of nleaf leaves from ps.leaf0
-    if (h->cfg.precision == MRA_PREC_EMU && mra::predict_on_engine(M, r, lb, maxp, nleaf))
+    if (engine)
       return mra::launch_predict_em(h->d_desc, lb, h->nlmax, ps, maxp, nleaf, h->status, h->stream, &g_launches, &h->timer);
     return mra::launch_predict(h->d_desc, M, r, h->nlmax, ps, maxp, h->status, h->stream, &g_launches, &h->timer, nleaf);
   };

@@ -251,13 +251,21 @@ static size_t predict_em_smem(int nlmax) {
   return EM_STAGE_BYTES + sizeof(double) * std::max((size_t)TC_M * (nlmax + 1), (size_t)2 * TC_M * C0_GMAX);
 }
 
-// Whether the marginal prediction of an emulated handle runs on the engine: a
-// 16-row FP64 tile of r <= 16 knots costs less than the engine's fixed time a
-// product (about 7 us), and the flat grid is 31 bits.
-bool predict_on_engine(int M, int r, int lb, int max_per_leaf, long nleaf) {
+// Whether the marginal prediction of an emulated handle runs on the engine (per_leaf: points a leaf on
+// average over the tree).  A product costs the engine about the same for one row as for 128, the FP64
+// kernel pays by 16-row tiles (of 32 columns for r <= 32, else 64), and a region is one CTA where its
+// leaves are four: few points a leaf, small blocks and trees with fewer regions than SMs stay on the FP64 kernel.
+// Kernel times at n = 100,000, M = 6 (engine / FP64, ms): r = 64: 0.15 points a leaf 4.2 / 3.8, 0.5 7.6 / 10.1,
+// 64 30 / 105; r = 36: 0.15 3.3 / 2.3, 0.5 5.8 / 6.1, 64 21 / 57; r = 32: 4 7.2 / 6.4, 16 8.1 / 9.9; r = 18: 4
+// 5.9 / 4.4, 16 6.6 / 6.8, 64 14.5 / 20.8.  64 regions (M = 4), r = 36: 8 0.80 / 0.67, 16 0.85 / 0.97; 16 regions,
+// r = 64: 32 1.24 / 1.11, 64 1.12 / 1.54; r = 32: 64 0.83 / 0.46, 256 0.72 / 1.16.  The flat grid is 31 bits.
+bool predict_on_engine(int M, int r, int lb, int max_per_leaf, long nleaf, double per_leaf) {
   if (M < 1 || r <= 16 || max_per_leaf <= 0) return false;
+  const long regions = nleaf >> lb;
+  const double few = regions >= 256 ? (r > 32 ? 0.5 : 16.0) : regions >= 64 ? (r > 32 ? 16.0 : 64.0) : (r > 32 ? 64.0 : 256.0);
+  if (per_leaf < few) return false;
   const long tiles = (((long)max_per_leaf << lb) + TC_M - 1) / TC_M;
-  return (nleaf >> lb) * tiles < (1L << 31);
+  return regions * tiles < (1L << 31);
 }
 
 cudaError_t launch_predict_em(const Desc* d_desc, int lb, int nlmax, const PredState& ps, int max_per_leaf, long nleaf,
