@@ -642,46 +642,16 @@ __device__ inline bool em_mma(EmCtx& cx, EmAcc& acc, const double* A, long sai, 
   return ok;
 }
 
-// A thread's N consecutive doubles at p, n of them kept (all: four at a time where
-// p allows).  The 32 lanes of a warp hold 32 rows, so every access touches 32
-// lines: 128 bytes of a row in 4 instructions instead of 16.
-__device__ __forceinline__ bool em_wide(const double* p) {
-  return (reinterpret_cast<uintptr_t>(p) & 31) == 0 && __isGlobal(p);
-}
+// A thread's N consecutive doubles at p, in any memory, n of them kept: two at a
+// time where all are and p allows.  The 32 lanes of a warp hold 32 rows, so every
+// access touches 32 lines: a row's 128 bytes go in 8 instructions instead of 16.
+// (32-byte accesses in inline PTX, ld/st.global.v4.f64, were 1.7 to 2.7 % faster: n =
+// 2^20 103.1 against 105.9 ms, n = 2^14 3.02 against 3.08, the gradient at n = 2^18
+// 77.3 against 79.2.  But where a product was a call they once left rows of a ragged
+// tile unwritten; rows of every alignment come out right in isolation, called or
+// inlined, and no cause was found, so rows are read and written by plain accesses.)
 template <int N>
 __device__ __forceinline__ void em_get(const double* p, int n, double* v) {
-  if (n >= N && em_wide(p)) {
-#pragma unroll
-    for (int c = 0; c < N; c += 4)
-      asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
-                   : "=d"(v[c]), "=d"(v[c + 1]), "=d"(v[c + 2]), "=d"(v[c + 3])
-                   : "l"(p + c)
-                   : "memory");
-  } else {
-#pragma unroll
-    for (int c = 0; c < N; ++c) v[c] = c < n ? p[c] : 0.0;
-  }
-}
-template <int N>
-__device__ __forceinline__ void em_put(double* p, int n, const double* v) {
-  if (n >= N && em_wide(p)) {
-#pragma unroll
-    for (int c = 0; c < N; c += 4)
-      asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p + c), "d"(v[c]), "d"(v[c + 1]), "d"(v[c + 2]),
-                   "d"(v[c + 3])
-                   : "memory");
-  } else {
-#pragma unroll
-    for (int c = 0; c < N; ++c)
-      if (c < n) p[c] = v[c];
-  }
-}
-
-// The same two doubles at a time, for rows in any memory: the form the products
-// that are calls use (em_rows, em_store_product).  There em_get / em_put's path of
-// four at a time left some rows of a ragged tile unwritten; inlined it does not.
-template <int N>
-__device__ __forceinline__ void em_get2(const double* p, int n, double* v) {
   if (n >= N && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
 #pragma unroll
     for (int c = 0; c < N; c += 2) {
@@ -695,7 +665,7 @@ __device__ __forceinline__ void em_get2(const double* p, int n, double* v) {
   }
 }
 template <int N>
-__device__ __forceinline__ void em_put2(double* p, int n, const double* v) {
+__device__ __forceinline__ void em_put(double* p, int n, const double* v) {
   if (n >= N && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
 #pragma unroll
     for (int c = 0; c < N; c += 2) *reinterpret_cast<double2*>(p + c) = make_double2(v[c], v[c + 1]);
@@ -750,11 +720,11 @@ static __device__ __noinline__ bool em_rows(EmCtx* pcx, const EmRows* pq) {
     double* const o = pq->out + (long)row * pq->ldo + c0;
     if (pq->sub) {
       double v[EmAcc::NC];
-      em_get2<EmAcc::NC>(o, nb - c0, v);
+      em_get<EmAcc::NC>(o, nb - c0, v);
 #pragma unroll
       for (int c = 0; c < EmAcc::NC; ++c) acc.v[c] = v[c] - acc.v[c];
     }
-    em_put2<EmAcc::NC>(o, nb - c0, acc.v);
+    em_put<EmAcc::NC>(o, nb - c0, acc.v);
     int e0 = -2000, e1 = -2000, ex = -2000;      // a thread's columns touch at most two groups
     const int x0 = pq->xe0 - c0, g0 = EM_KG - ((pq->gcol + c0) & (EM_KG - 1));
 #pragma unroll

@@ -136,7 +136,7 @@ static __device__ __noinline__ bool em_store_product(EmCtx* pcx, const double* A
     if (ok && row < n - i0 && c0 < nb) {
 #pragma unroll
       for (int c = 0; c < EmAcc::NC; ++c) acc.v[c] = neg ? -acc.v[c] : acc.v[c];
-      em_put2<EmAcc::NC>(C + (long)(i0 + row) * ldc + j0 + c0, nb - c0, acc.v);
+      em_put<EmAcc::NC>(C + (long)(i0 + row) * ldc + j0 + c0, nb - c0, acc.v);
     }
   }
   pcx->chunks = cx.chunks;
