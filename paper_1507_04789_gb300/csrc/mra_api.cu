@@ -1807,7 +1807,7 @@ int mra_predict(mra_handle* h, const mra_params* theta, const double* plocs, int
   const int lb = M > 0 ? mra::leaf_bits(h->hd.sh) : 0;
   // (decided for the whole tree, so that a streamed handle's chunks take its kernel)
   const bool engine = h->cfg.precision == MRA_PREC_EMU &&
-                      mra::predict_on_engine(M, r, lb, maxp, ps.nleaves, (double)np / (double)ps.nleaves);
+                      mra::predict_on_engine(M, r, lb, maxp, ps.nleaves, (long)np, (long)h->n);
   auto launch = [&](long nleaf) {                // the points of nleaf leaves from ps.leaf0
     if (engine)
       return mra::launch_predict_em(h->d_desc, lb, h->nlmax, ps, maxp, nleaf, h->status, h->stream, &g_launches, &h->timer);

@@ -113,7 +113,7 @@ size_t predict_smem_bytes(int r, int nlmax);
 // The same for an emulated handle, on the emulation engine (lb = leaf_bits, the
 // leaves [ps.leaf0, ps.leaf0 + nleaf) whole regions of level M - 1), and whether
 // a prediction takes it.
-bool predict_on_engine(int M, int r, int lb, int max_per_leaf, long nleaf, double per_leaf);
+bool predict_on_engine(int M, int r, int lb, int max_per_leaf, long nleaf, long np, long n);
 cudaError_t launch_predict_em(const Desc* d_desc, int lb, int nlmax, const PredState& ps, int max_per_leaf, long nleaf,
                               int* status, cudaStream_t s, int64_t* launches, Timer* tm);
 // Joint posterior predictive (Prop. 2): mode 1 keeps D and the Y_l for the

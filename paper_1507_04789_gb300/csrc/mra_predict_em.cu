@@ -251,21 +251,44 @@ static size_t predict_em_smem(int nlmax) {
   return EM_STAGE_BYTES + sizeof(double) * std::max((size_t)TC_M * (nlmax + 1), (size_t)2 * TC_M * C0_GMAX);
 }
 
-// Whether the marginal prediction of an emulated handle runs on the engine (per_leaf: points a leaf on
-// average over the tree).  A product costs the engine about the same for one row as for 128, the FP64
-// kernel pays by 16-row tiles (of 32 columns for r <= 32, else 64), and a region is one CTA where its
-// leaves are four: few points a leaf, small blocks and trees with fewer regions than SMs stay on the FP64 kernel.
-// Kernel times at n = 100,000, M = 6 (engine / FP64, ms): r = 64: 0.15 points a leaf 4.2 / 3.8, 0.5 7.6 / 10.1,
-// 64 30 / 105; r = 36: 0.15 3.3 / 2.3, 0.5 5.8 / 6.1, 64 21 / 57; r = 32: 4 7.2 / 6.4, 16 8.1 / 9.9; r = 18: 4
-// 5.9 / 4.4, 16 6.6 / 6.8, 64 14.5 / 20.8.  64 regions (M = 4), r = 36: 8 0.80 / 0.67, 16 0.85 / 0.97; 16 regions,
-// r = 64: 32 1.24 / 1.11, 64 1.12 / 1.54; r = 32: 64 0.83 / 0.46, 256 0.72 / 1.16.  The flat grid is 31 bits.
-bool predict_on_engine(int M, int r, int lb, int max_per_leaf, long nleaf, double per_leaf) {
+// Whether the marginal prediction of np points on an emulated handle (n observations) runs on the engine.
+// A product costs the engine about the same for one row as for 128, the FP64 kernel pays by 16-row tiles (of
+// 32 columns for r <= 32, else 64) and by the observations a leaf, and a region is one CTA where its leaves
+// are four: few points a leaf, small blocks on sparse leaves and trees with fewer regions than SMs stay on the
+// FP64 kernel.  The line is where the engine is first faster for points over the whole domain and (to a tenth
+// of a millisecond) over a sixteenth of it.  FP64 / engine, kernel times at so many points a leaf (domain,
+// sixteenth):
+//   1024 regions: r = 17: 24 1.20, 1.39, 16 0.97, 1.41;  25: 16 1.14, 1.70, 4 0.82, 1.21;  33: 1 1.27, 1.48, 0.5
+//     1.02, 0.91;  49: 0.5 1.19, 1.00;  64: 0.5 1.28, 1.44.
+//   256 regions: 25: 16 1.13, 1.86, 4 0.75, 1.21;  33: 4 1.41, 1.86, 2 1.17, 0.96, 1 1.09, 0.80;
+//     49: 1 1.25, 0.88;  64: 2 1.54, 1.22, 1 1.42, 0.98.
+//   64 regions: 17: 96 1.10, 1.21, 64 0.96, 1.58;  25: 64 0.96 to 1.08, 1.64;  33: 16 1.20, 2.76, 8 0.73, 1.38;
+//     64: 16 1.63, 1.78, 8 0.94, 1.79.
+//   16 regions: 32: 256 1.62, 1.75, 128 1.01, 1.38;  33: 64 1.17, 1.42, 32 0.74, 1.45.
+//   4 regions: 33: 1024 2.18, 2.86, 512 (6 observations a leaf) 0.94;  49: 256 1.33, 1.66.
+//   1 region: 33: 4096 1.67, 2.53 (6 observations a leaf 1.17), 1024 0.92, 1.32;  48: 1024 (6) 0.73.
+// r <= 32 stays on the FP64 kernel below M r = 96 columns (r = 17, M = 4 or 5, 24 to 30 observations a leaf: 0.90
+// to 0.95 at the line and above), with fewer than 16 regions (0.77 to 1.5 whatever the points) and on leaves of
+// few observations (6: 64 regions, r = 17 0.81, 512 regions 0.78; but 1024 regions, r = 25 1.27).  Regions of two
+// leaves (J_M = 2) hold half the points: r = 33, 256 regions 16 1.55, 8 0.92, 1024 regions 4 1.10, 2 0.98; r = 17,
+// 256 regions 64 1.22, 16 0.85: eight times the line.
+//   The grid holds the tiles of the fullest leaf for every region, and an empty CTA costs about 25 ns (one
+// of the FP64 kernel's 1 ns): points crowded into so few regions that more than 64 times the tiles needed
+// would be launched stay on the FP64 kernel (r = 17, 16 a leaf of 4096, all in one: engine 13.0 ms, FP64 8.9).
+// The flat grid is 31 bits.
+bool predict_on_engine(int M, int r, int lb, int max_per_leaf, long nleaf, long np, long n) {
+  constexpr long NEVER = 1L << 40;
+  // half points a leaf; rows: regions from 1024, 256, 64, 16, 4, 1 on; columns: r <= 24, <= 32, < 48, up to 64
+  constexpr long LINE[6][4] = {{48, 32, 2, 1},       {48, 32, 5, 3},            {192, 192, 32, 32},
+                               {512, 512, 128, 128}, {NEVER, NEVER, 2048, 512}, {NEVER, NEVER, 8192, 8192}};
   if (M < 1 || r <= 16 || max_per_leaf <= 0) return false;
   const long regions = nleaf >> lb;
-  const double few = regions >= 256 ? (r > 32 ? 0.5 : 16.0) : regions >= 64 ? (r > 32 ? 16.0 : 64.0) : (r > 32 ? 64.0 : 256.0);
-  if (per_leaf < few) return false;
+  if (r <= 32 && (M * r < 96 || (n < 24 * nleaf && (r <= 24 || regions < 1024)))) return false;
+  const int row = regions >= 1024 ? 0 : regions >= 256 ? 1 : regions >= 64 ? 2 : regions >= 16 ? 3 : regions >= 4 ? 4 : 5;
+  const long line = LINE[row][r <= 24 ? 0 : r <= 32 ? 1 : r < 48 ? 2 : 3];
+  if (2 * np < (lb < 2 ? 8 * line : line) * nleaf) return false;
   const long tiles = (((long)max_per_leaf << lb) + TC_M - 1) / TC_M;
-  return regions * tiles < (1L << 31);
+  return regions * tiles <= 64 * (np / TC_M + regions) && regions * tiles < (1L << 31);
 }
 
 cudaError_t launch_predict_em(const Desc* d_desc, int lb, int nlmax, const PredState& ps, int max_per_leaf, long nleaf,
