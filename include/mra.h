@@ -73,11 +73,14 @@ extern "C" {
                                in binary64; the Gram products of the posterior pass in the
                                FP64-grade emulation below (r > 16 and J_M <= 4, else binary64) */
 #define MRA_PREC_EMU      2 /* every large contraction (prior chain, leaf covariance and solve,
-                               leaf and child-to-parent Gram products, posterior G, and in
-                               mra_loglik_grad the adjoint's products) on the tensor cores as an
+                               leaf and child-to-parent Gram products, posterior G, in
+                               mra_loglik_grad the adjoint's products and in mra_predict, for
+                               many points, the prediction's) on the tensor cores as an
                                FP64-grade emulation: operands cut into six 8-bit f16 digits
                                per 128-column group, exact FP32 accumulation, double-float sums
-                               (below 1e-14 relative error per product); factorisations and
+                               (within 1e-14 of sum |a b| per product; operands are rounded to
+                               2^-49 of a power of two above their row's largest element in
+                               the group, or in a range holding it); factorisations and
                                the rest in binary64 */
 
 #define MRA_HOST          0 /* pointer argument is host memory */
@@ -212,6 +215,12 @@ int mra_loglik_grad(mra_handle* h, const mra_params* theta, double* loglik_out, 
  *   mean_out, var_out : np doubles each, same memory space as plocs, caller-owned.
  * The handle keeps a prediction buffer (about np (M r + 8) doubles) that is
  * allocated on the first call and grown when np exceeds every earlier call's.
+ * A point's result does not depend on the other points of the call, bit for bit,
+ * except on a MRA_PREC_EMU handle with r > 16: there a call with enough points for
+ * the tree and r runs in the FP64-grade emulation and a smaller one in binary64,
+ * so that the last digits of a point (1e-9 of the largest mean or variance at
+ * most) can differ between calls with few and with many points, and between
+ * this call and mra_predict_joint, which is always in binary64.
  * Errors: MRA_ERR_ARG (theta out of range, a location outside bbox),
  * MRA_ERR_STATE (a batch handle), MRA_ERR_NOT_PD, MRA_ERR_OOM, MRA_ERR_CUDA.
  */

@@ -298,7 +298,10 @@ class Handle:
         return out.value, (g if four else g[:3].copy())
 
     def predict(self, theta, plocs):
-        """Posterior predictive mean and variance of y at plocs (Sec. 3.4, Prop. 2)."""
+        """Posterior predictive mean and variance of y at plocs (Sec. 3.4, Prop. 2).
+
+        On an emulated handle (r > 16) many points run in the FP64-grade emulation and few
+        in binary64, so a point's last digits can depend on how many are passed."""
         p = MraParams(*[float(v) for v in theta])
         if _is_torch_cuda(plocs):
             import torch
