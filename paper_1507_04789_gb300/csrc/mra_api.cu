@@ -23,6 +23,7 @@
 
 #include "../../include/mra.h"
 #include "mra_launch.h"
+#include "mra_sizes.h"
 
 static_assert(mra::JOINT_TILE == MRA_MAX_JOINT_LEAF, "one CTA holds a leaf's prediction points");
 
@@ -765,17 +766,6 @@ int mra_build(const mra_config* cfg, const double* locs, const double* y, int64_
       lmax = std::max(lmax, c.ls1 - c.ls0);
     }
   };
-  // bytes of the factors with rc[m] regions' storage at every level and the leaf stores sized (obs, ls, leaves)
-  auto factor_bytes = [&](const std::vector<int64_t>& rc, int64_t obs, int64_t ls, int64_t leaves) {
-    double b = 0;
-    for (int m = 0; m < M; ++m) {
-      const double R = (double)rc[m], T = (m + 1) * (m + 2) / 2.0;
-      b += 8.0 * R * ((double)r * m * r * 2 + r * r * 2 + T * r * r + (m + 1) * r + r);
-      if (emu) b += 4.0 * R * (((m * r + 127) / 128) * r + m * r + r);
-    }
-    b += 8.0 * ((double)obs * M * r + obs + ls) + (emu ? 4.0 * ((double)leaves * M * r + obs * ((M * r + 127) / 128)) : 0);
-    return b;
-  };
   std::vector<int64_t> full(M + 1);
   for (int m = 0; m <= M; ++m) full[m] = nreg[m];
   if (cfg->stream_level == 0 && M >= 2) {   // automatic: stream only when the factors of every level do not fit
@@ -784,7 +774,7 @@ int mra_build(const mra_config* cfg, const double* locs, const double* y, int64_
       fr = SIZE_MAX;
       cudaGetLastError();
     }
-    if (factor_bytes(full, n, tail, nreg[M]) > 0.8 * (double)fr) {
+    if (mra::factor_bytes(M, r, emu, gram, full.data(), n, tail, nreg[M]) > 0.8 * (double)fr) {
       for (int sl = 1; sl < M && !s_lvl; ++sl) {
         std::vector<Chunk> ch;
         std::vector<int64_t> cm;
@@ -792,7 +782,7 @@ int mra_build(const mra_config* cfg, const double* locs, const double* y, int64_
         make_chunks(sl, ch, cm, om, lm);
         std::vector<int64_t> rc(M + 1);
         for (int m = 0; m <= M; ++m) rc[m] = m <= sl ? nreg[m] : cm[m];
-        if (factor_bytes(rc, om, lm, cm[M]) <= 0.5 * (double)fr) s_lvl = sl;
+        if (mra::factor_bytes(M, r, emu, gram, rc.data(), om, lm, cm[M]) <= 0.5 * (double)fr) s_lvl = sl;
       }
       if (!s_lvl) { mra_free(h); return fail(MRA_ERR_OOM, "the factors do not fit in device memory even streamed"); }
     }
