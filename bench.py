@@ -1,5 +1,6 @@
 #!/usr/bin/env python
-"""Benchmark of the M-RA log-likelihood on GB300 (prints one JSON line).
+"""Benchmark of the M-RA log-likelihood on GB300 (prints one JSON line, after lines "# table <name>: ..."
+with the per-level and per-kernel tables).
 
 One step = one log-likelihood evaluation of the whole hot path at a new
 parameter value: the prior pass over every level, the leaf factorisation, the
@@ -348,6 +349,41 @@ def oracle_sample(workload: str, level: int, seed: int):
 
 # ---------------------------------------------------------------------------
 
+# Parts of the result that are tables: printed on lines of their own before the result line, which a
+# reader of a log's last few kilobytes then sees whole.
+RESULT_TABLES = ("roofline.per_level", "roofline.kernels", "emu.kernels", "emu.per_level", "emu.clocks",
+                 "mixed.kernels", "mixed.per_level", "mixed.clocks", "fp64.kernels", "fp64.per_level", "fp64.clocks",
+                 "cpu_baseline.oracle_check", "oracle_check", "gradient.fp64", "gradient.mle", "batch", "prediction",
+                 "level_J")
+
+
+def split_result(line: dict):
+    """(tables, the rest of the line with the tables' headline numbers)."""
+    short = {k: dict(v) if isinstance(v, dict) else v for k, v in line.items()}
+    tables = {}
+    for path in RESULT_TABLES:
+        *outer, key = path.split(".")
+        at = short if not outer else short.get(outer[0])
+        if at and at.get(key) is not None:
+            tables[path] = at.pop(key)
+    if "batch" in tables:
+        short["batch_ms"] = {p: v["ms_per_batch"] for p, v in tables["batch"].items()
+                             if isinstance(v, dict) and "ms_per_batch" in v}
+    if "prediction" in tables:
+        short["prediction_points_per_s"] = {p: v["points_per_s"] for p, v in tables["prediction"].items()
+                                            if isinstance(v, dict) and "points_per_s" in v}
+    if "level_J" in tables:
+        short["level_J_ms"] = tables["level_J"]["ms_per_step"]
+    return tables, short
+
+
+def print_result(line: dict) -> None:
+    tables, short = split_result(line)
+    for name, value in tables.items():
+        print(f"# table {name}: {json.dumps(value)}")
+    print(json.dumps(short), flush=True)
+
+
 def dist_env():
     rank = int(os.environ.get("RANK", "0"))
     world = int(os.environ.get("WORLD_SIZE", "1"))
@@ -511,6 +547,15 @@ def predict_flops_per_point(M: int, r: int, c: float) -> float:
     return chain + rec + 2.0 * M * r + c * (c + 1) + 2.0 * M * r * c + 4.0 * c + 2.0 * c * M * r
 
 
+def prediction_kernel(prec: str, r: int, alg_tflops: float, bf16_peak: float) -> dict:
+    """The kernel that predicts many points in a form, its pipe and the fraction of that pipe's peak."""
+    tensor = prec == "emu" and r > 16
+    peak = bf16_peak if tensor else FP64_PEAK_TFLOPS
+    return {"kernel": "predict_kernel_em" if tensor else "predict_kernel", "pipe": "tensor" if tensor else "alu",
+            "kernel_fp64_alg_tflops": alg_tflops, "peak": peak, "kernel_frac": alg_tflops / peak,
+            "per_unit": "algorithmic FP64 FLOPs" + (" against the bf16 tensor peak" if tensor else "")}
+
+
 def run_prediction(args, world, rank, mra, np, torch, stream, handles, w, theta0, off):
     """Kriging throughput (points/s) and errors: 2^20 cell-centred grid points on
     the n = 2^20 problem (emulated-form factors against the FP64 form's), and the
@@ -525,6 +570,8 @@ def run_prediction(args, world, rank, mra, np, torch, stream, handles, w, theta0
     dgrid = torch.tensor(grid, device="cuda")
     res = {}
     nF = np.diff(off)
+    peaks = measured_peaks()
+    bf16_peak = peaks["bf16_tflops_sustained"] if peaks else BF16_PEAK_FALLBACK
     pts_per_leaf = grid.shape[0] / 4 ** w.M
     flops_pt = predict_flops_per_point(w.M, w.r, float(nF.mean()))
     for p in ("emu", "fp64"):
@@ -551,15 +598,13 @@ def run_prediction(args, world, rank, mra, np, torch, stream, handles, w, theta0
         res[p] = (mean.cpu().numpy(), var.cpu().numpy())
         alg = flops_pt * grid.shape[0] / (kms * 1e-3) / 1e12
         out[p] = {"points_per_s": world * grid.shape[0] / (ms * 1e-3), "ms_per_call": ms,
-                  "kernel_ms": kms, "kernel_fp64_alg_tflops": alg,
-                  "kernel_frac": alg / FP64_PEAK_TFLOPS,
+                  "kernel_ms": kms, **prediction_kernel(p, w.r, alg, bf16_peak),
                   "e2e": {"points_per_s": world * grid.shape[0] / e2e_s, "h2d_bytes_per_call": int(grid.nbytes),
                           "d2h_bytes_per_call": int(2 * 8 * grid.shape[0])}}
     m64, v64 = res["fp64"]
     me, ve = res["emu"]
     out["grid"] = {"points": int(grid.shape[0]), "layout": f"{g} x {g} cell-centred grid on [0,1]^2",
-                   "points_per_leaf": pts_per_leaf, "kernel": "predict_kernel (FP64 pipe)",
-                   "fp64_flops_per_point": flops_pt, "peak": FP64_PEAK_TFLOPS,
+                   "points_per_leaf": pts_per_leaf, "fp64_flops_per_point": flops_pt,
                    "emu_vs_fp64": {"mean_max_abs": float(np.max(np.abs(me - m64))),
                                    "mean_max_rel": float(np.max(np.abs(me - m64)) / np.max(np.abs(m64))),
                                    "var_max_rel": float(np.max(np.abs(ve - v64) / np.abs(v64)))}}
@@ -1077,7 +1122,7 @@ def main():
             line[p]["per_level"] = [{k: r_[k] for k in ("level", "stage", "ms_per_step", "alg_tflops", "frac",
                                                         "hbm_gbs") + (("engine_frac",) if "engine_frac" in r_ else ())}
                                     for r_ in lvl_tabs[p]]
-        print(json.dumps(line), flush=True)
+        print_result(line)
     if world > 1:
         dist.destroy_process_group()
     return 0
