@@ -796,6 +796,8 @@ __device__ inline void chol_panels(const Blocks<STK, ONE> M, int* bad) {
     __syncthreads();
     // the trailing lower triangles; their first rows (the next diagonal blocks) by warp b, and while the
     // rest is less than that chain takes, the other warps of its sub-partition leave it the FP64 unit
+    // (log-likelihood at n = 2^14, emulated: 3.023 ms; 3.027 never leaving it, 3.038 always; n = 4096, FP64:
+    // 0.648, 0.648, 0.650)
     auto rest = [&](int b) {
       const int m = below(b);
       return m < FB ? 0 : m * (m + 1) / 2 - FB * (FB + 1) / 2;

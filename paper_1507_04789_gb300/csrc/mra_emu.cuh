@@ -21,12 +21,15 @@
 //
 // Signed digits carry 8 bits a slice where sign-and-magnitude slices of the
 // same magnitude (|a| < 128) carry 7: 6 slices and 26 products against 7 and 28,
-// with the operand error (at most 2^-49 of the group's largest element) rounded
-// instead of truncated.  The pairs of weight 8 matter: without them (21 products,
+// with the operand error (at most 2^(e - 49)) rounded instead of truncated.  The pairs of weight 8 matter: without them (21 products,
 // 2 % of an evaluation) the squares d_4^2 a Gram product drops are all positive,
 // and the gradient at n = 2^16 is off by 2e-11 to 3e-10 instead of 6e-13 to 3e-12.
-// So a product matches FP64 to about 1e-15 relative to sum |a b| while running on
-// the tensor cores; only rare sums touch the FP64 pipe.
+// So a term a b is off by at most 2^-46.5 2^(e + f) and a product by about 1e-15 of
+// sum |a b| where 2^e and 2^f are within a few times the elements, while running on
+// the tensor cores; only rare sums touch the FP64 pipe.  (2^e is at most twice the
+// group's largest element when it comes from the scale pass; a producer's scale may
+// cover more than the group, as H's column scales a whole leaf, and rows of wide
+// dynamic range keep fewer bits of their small elements.)
 // Range: the running sums are FP32 pairs, so |results| < 2^127, and a group
 // whose scale product 2^(e_i + f_j) is below 2^-110 is dropped.
 //

@@ -10,7 +10,7 @@
 //    the Gram products of the posterior pass (leaf_syrk, aggregate) need more
 //    than FP32 accuracy: they run on the emulation engine below (r > 16), else
 //    in the FP64 kernels;
-//  * MRA_PREC_EMU: em_mma (f16-digit FP64 emulation, about 1e-14 relative),
+//  * MRA_PREC_EMU: em_mma (f16-digit FP64 emulation, error bound in mra_emu.cuh),
 //    which also runs the two Gram products (leaf_syrk_kernel_em,
 //    aggregate_kernel_em below).
 // The Cholesky factorisations, triangular inverses, log-determinants and the
