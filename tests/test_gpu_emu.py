@@ -1,12 +1,14 @@
-"""FP64-emulation form (every large contraction on the bf16 tensor cores as
-seven 7-bit slices per operand) against the FP64 oracle.
+"""FP64-emulation form (every large contraction on the f16 tensor cores as six
+signed 8-bit digits per operand) against the FP64 oracle.
 
-Each emulated product carries about 1e-14 relative error (operands truncated to
-49 bits below their 64-column group's largest element, double-float sums).  The
-prior chain cancels by up to 1e5 at the finest levels, which the FP64 form
-shares; measured, the emulated form stays within the FP64 form's own bars: a
-relative 1e-10 on the log-likelihood and 1e-9 on predictions, on uniform data
-and on the dense swath data where the 3xTF32 form loses most.
+Each emulated product is within about 1e-14 of sum |a b| (operands rounded to 49
+bits below a power of two above their 128-column group's largest element,
+double-float sums).  The prior chain cancels by up to 1e5 at the finest levels,
+which the FP64 form shares; measured, the emulated form stays within the FP64
+form's own bars: a relative 1e-10 on the log-likelihood and 1e-9 on predictions,
+on uniform data and on the dense swath data where the 3xTF32 form loses most.
+Few-point predictions run on the FP64 kernel (test_gpu_predict_emu.py has the
+engine's).
 """
 import numpy as np
 import pytest
