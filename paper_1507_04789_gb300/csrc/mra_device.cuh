@@ -227,6 +227,24 @@ __device__ __forceinline__ double cov0(const Cov& c, double x1, double y1, doubl
   return v;
 }
 
+// The same with the free-smoothness family's quadrature as a call, for the kernels
+// of the emulation engine: inlined its loop shared their 128 registers a thread with
+// the engine's state (n = 60,000, r = 36: prior 13.9 -> 12.1 ms, chain 29.5 -> 24.9 ms;
+// the kernels of 256 threads and 255 registers took 12.4 and 24.9).
+static __device__ __noinline__ double matern_rho(double nu, double snu, double lcnu, double h) {
+  Cov c{};
+  c.nu = nu;
+  c.snu = snu;
+  c.lcnu = lcnu;
+  return matern_nu(c, h).rho;
+}
+__device__ __forceinline__ double cov0_em(const Cov& c, double x1, double y1, double x2, double y2) {
+  if (c.family != 2) return cov0(c, x1, y1, x2, y2);
+  double v = c.sigma2 * matern_rho(c.nu, c.snu, c.lcnu, dist_scaled(x1 - x2, y1 - y2, c.ik));
+  if (c.nonstat) v *= sqrt(gvar(x1) * gvar(x2));
+  return v;
+}
+
 // ---- C0 with few FP64 operations (families 0 and 1) -------------------------
 // GB300 retires about 2 FP64 FMA per clock per SM against 128 FP32 operations,
 // and the emulated form's kernels evaluate n M r covariances per evaluation,

@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(Engine<EMU>::NTH) prior_level_kernel_tc(int m,
     return fast ? c0_fast(cv.family, pdx[g * C0_GMAX * C0_GMAX + ci * gx + cj] +
                                          pdy[g * C0_GMAX * C0_GMAX + qrow[ql] * gy + qrow[qj]],
                           cv.nonstat ? pgp[g * gx + ci] * pgq[g * gx + cj] : cv.sigma2)
-                : cov0(cv, qx[qi], qy[qi], bx[qj], by[qj]);
+                : (EMU ? cov0_em : cov0)(cv, qx[qi], qy[qi], bx[qj], by[qj]);
   };
   if (threadIdx.x == 0) bad = 0;
   Engine<EMU> eng;
@@ -406,7 +406,7 @@ __global__ void __launch_bounds__(EM_NT) chain_forward_kernel_em(const Desc* __r
           v = cov0_d(cv, sx[fi], sy[fi], ax[qj], ay[qj], d1, d2);
           *reinterpret_cast<double2*>(lf.dc + 2 * ((t0 + fi) * Mr + l * r + qj)) = make_double2(d1, d2);
         } else {
-          v = cov0(cv, sx[fi], sy[fi], ax[qj], ay[qj]);
+          v = cov0_em(cv, sx[fi], sy[fi], ax[qj], ay[qj]);
         }
         Hrow[(long)fi * Mr + l * r + qj] = v;
         if (l == 0) atomicMax(xsc + fi, xexp_of(v));
@@ -648,7 +648,7 @@ __global__ void __launch_bounds__(Engine<EMU>::NTH) leaf_kernel_tc(const Desc* _
       const double dx = sx[fi] - sx[fj], dy = sy[fi] - sy[fj];
       v = c0_fast(cv.family, c0s2 * fma(dx, dx, dy * dy), cv.nonstat ? cv.sigma2 * lgq[fi] * lgq[fj] : cv.sigma2);
     } else {
-      v = cov0(cv, sx[fi], sy[fi], sx[fj], sy[fj]);
+      v = (EMU ? cov0_em : cov0)(cv, sx[fi], sy[fi], sx[fj], sy[fj]);
     }
     S[fi * lds + fj] = v + (fi == fj ? tau2 : 0.0);
   }
