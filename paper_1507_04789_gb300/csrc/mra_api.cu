@@ -1794,6 +1794,8 @@ int mra_predict(mra_handle* h, const mra_params* theta, const double* plocs, int
   mra::PredState ps = pred_state(h);
   ps.mean = where == MRA_DEVICE ? mean_out : h->p_mean;
   ps.var = where == MRA_DEVICE ? var_out : h->p_var;
+  ps.point_leaf = h->p_leaf;
+  ps.np = (long)np;
   const int lb = M > 0 ? mra::leaf_bits(h->hd.sh) : 0;
   // (decided for the whole tree, so that a streamed handle's chunks take its kernel)
   const bool engine = h->cfg.precision == MRA_PREC_EMU &&

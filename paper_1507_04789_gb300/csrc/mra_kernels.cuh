@@ -167,6 +167,11 @@ struct PredState {
   long leaf0;
   int desc;
   long nleaves;           // leaves of the complete tree (the launch's grid where it covers them all)
+  // marginal predictions: the number of points and the leaf of each in caller's order (null: the grid goes
+  // by leaves), and the end of the leaves a grid of points covers
+  long np;
+  const int32_t* point_leaf;
+  long leaf1;
 };
 
 struct Shape {
