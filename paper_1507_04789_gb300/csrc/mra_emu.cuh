@@ -293,8 +293,8 @@ __device__ __forceinline__ void em_split_pair(double x0, double x1, int E, uint3
 // One operand of a product as its slots see it.
 //
 // A slot is 16 rows x 16 columns, a warp's 8 elements per lane.  Rows that are
-// contiguous along K and aligned are read four elements at a time, four lanes
-// to a row's 128 bytes (lane: row l / 4 and row l / 4 + 8, columns 4 (l % 4) ..):
+// contiguous along K and aligned are read four elements a lane in two loads, four
+// lanes to a row's 128 bytes (lane: row l / 4 and row l / 4 + 8, columns 4 (l % 4) ..):
 // 8 cache lines a load, where a lane to a row took 16 and kept the L1's tag
 // stage busier than anything else in the engine.  Other operands give every
 // lane 8 columns of one row (row l % 16, columns 8 (l / 16) ..), so that loads
@@ -303,13 +303,11 @@ struct EmOperand {
   const double* p;
   long si, sk;      // element (i, k) at p[i * si + k * sk]
   int n;            // rows kept
-  int vec;          // elements a load (4: 32-byte aligned global rows, 2: 16-byte aligned rows, 1: any layout)
+  bool vec;         // rows contiguous and 16-byte aligned (else: any layout)
 };
 
 __device__ __forceinline__ EmOperand em_operand(const double* p, long si, long sk, int n) {
-  const uintptr_t a = reinterpret_cast<uintptr_t>(p);
-  const int vec = sk != 1 ? 1 : ((a & 31) == 0 && (si & 3) == 0 && __isGlobal(p) ? 4 : ((a & 15) == 0 && (si & 1) == 0 ? 2 : 1));
-  return EmOperand{p, si, sk, n, vec};
+  return EmOperand{p, si, sk, n, sk == 1 && (reinterpret_cast<uintptr_t>(p) & 15) == 0 && (si & 1) == 0};
 }
 
 // This lane's 8 elements of the slot with first row i0 and first column k0 (zero
@@ -317,7 +315,7 @@ __device__ __forceinline__ EmOperand em_operand(const double* p, long si, long s
 // from tab (0 beyond).
 __device__ __forceinline__ void em_load(const EmOperand& o, const int* tab, int i0, int k0, int k1, double* x, int* e) {
   const int lane = threadIdx.x & 31;
-  if (o.vec > 1) {
+  if (o.vec) {
     const int k = k0 + 4 * (lane & 3), kn = k1 - k;
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
@@ -327,15 +325,11 @@ __device__ __forceinline__ void em_load(const EmOperand& o, const int* tab, int 
       const bool in = i < o.n;
       e[j] = in ? tab[i] : 0;
       if (in && kn >= 4) {
-        if (o.vec == 4) {
-          asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(y[0]), "=d"(y[1]), "=d"(y[2]), "=d"(y[3]) : "l"(p) : "memory");
-        } else {
-          const double2 u = *reinterpret_cast<const double2*>(p), v = *reinterpret_cast<const double2*>(p + 2);
-          y[0] = u.x;
-          y[1] = u.y;
-          y[2] = v.x;
-          y[3] = v.y;
-        }
+        const double2 u = *reinterpret_cast<const double2*>(p), v = *reinterpret_cast<const double2*>(p + 2);
+        y[0] = u.x;
+        y[1] = u.y;
+        y[2] = v.x;
+        y[3] = v.y;
       } else {
 #pragma unroll
         for (int c = 0; c < 4; ++c) y[c] = in && c < kn ? p[c] : 0.0;
@@ -367,7 +361,7 @@ __device__ __forceinline__ void em_split_slot(const EmOperand& o, int i0, const 
   em_split_pair(x[4], x[5], E1, w[2]);
   em_split_pair(x[6], x[7], E1, w[3]);
   uint16_t* d = planes + (i0 >> 3) * EM_CC * 64;   // (i0 is a multiple of 16)
-  if (o.vec > 1) {
+  if (o.vec) {
     const int l = lane & 3;
     d += (l >> 1) * 64 + (lane >> 2) * 8 + (l & 1) * 4;
 #pragma unroll
@@ -648,11 +642,12 @@ __device__ inline bool em_mma(EmCtx& cx, EmAcc& acc, const double* A, long sai, 
 // A thread's N consecutive doubles at p, in any memory, n of them kept: two at a
 // time where all are and p allows.  The 32 lanes of a warp hold 32 rows, so every
 // access touches 32 lines: a row's 128 bytes go in 8 instructions instead of 16.
-// (32-byte accesses in inline PTX, ld/st.global.v4.f64, were 1.7 to 2.7 % faster: n =
-// 2^20 103.1 against 105.9 ms, n = 2^14 3.02 against 3.08, the gradient at n = 2^18
-// 77.3 against 79.2.  But where a product was a call they once left rows of a ragged
-// tile unwritten; rows of every alignment come out right in isolation, called or
-// inlined, and no cause was found, so rows are read and written by plain accesses.)
+// (32-byte accesses in inline PTX, ld/st.global.v4.f64, here and in em_load were up to
+// 3 % faster: n = 2^20 103.0 against 105.2 ms, n = 2^14 3.04 against 3.06, the gradient
+// at n = 2^18 77.1 against 78.9, predictions there 29.2 against 29.4.  But where a
+// product was a call they once left rows of a ragged tile unwritten; rows of every
+// alignment come out right in isolation, called or inlined, and no cause was found, so
+// the engine reads and writes by plain accesses only.)
 template <int N>
 __device__ __forceinline__ void em_get(const double* p, int n, double* v) {
   if (n >= N && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
