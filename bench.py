@@ -136,22 +136,22 @@ def contraction_flops(M: int, r: int, nF, precision: str):
 SOURCES_EMU = ["mra_mixed.cu", "mra_emu.cuh", "mra_tc.cuh", "mra_device.cuh", "mra_kernels.cuh"]
 TRAFFIC = {
     ("emu", "chain_forward_kernel_em", "n1M_matern15_M7_r64"): {
-        "bytes": 7.5511e+09,
-        "how": "dram__bytes_read.sum + dram__bytes_write.sum of chain_forward_kernel_em (655.9 + 962.1 MB) "
+        "bytes": 7.7472e+09,
+        "how": "dram__bytes_read.sum + dram__bytes_write.sum of chain_forward_kernel_em (649.9 + 1010.1 MB) "
                "at n = 2^18, M = 6 (profiles/leaf_stage_emu_n256k_matern15_M6_r64.md), scaled by n M r "
                "(x 4.667) to n = 2^20, M = 7; the kernel writes V_F (8 B x n x M r) and reads the points "
                "and the ancestors' factors, both in proportion to n M r",
         "sources": SOURCES_EMU,
-        "sha1": "552fa40b6e72462cf0581de30c3e2a7df4a05009",
+        "sha1": "3d56ab77486d035e7369a77e716d1dbd2cbbdffe",
     },
     ("emu", "leaf_kernel_tc<1>", "n1M_matern15_M7_r64"): {
-        "bytes": 8.4688e+09,
-        "how": "dram__bytes_read.sum + dram__bytes_write.sum of leaf_kernel_tc<1> (844.2 + 970.4 MB) at "
+        "bytes": 8.4445e+09,
+        "how": "dram__bytes_read.sum + dram__bytes_write.sum of leaf_kernel_tc<1> (841.1 + 968.3 MB) at "
                "n = 2^18, M = 6 (profiles/leaf_stage_emu_n256k_matern15_M6_r64.md), scaled by n M r (x 4.667) "
                "to n = 2^20, M = 7; the kernel reads V_F and writes H (8 B x n x M r each) and the "
                "L_Sigma^{-1} blocks (8 B x sum n_F^2, about 1/7 of it)",
         "sources": SOURCES_EMU,
-        "sha1": "552fa40b6e72462cf0581de30c3e2a7df4a05009",
+        "sha1": "3d56ab77486d035e7369a77e716d1dbd2cbbdffe",
     },
 }
 
